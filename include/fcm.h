@@ -113,8 +113,8 @@ typedef struct {
     int schwarz_concurrent;   /* 1: shared-factor products run on a second stream beside the
                                  streamed factors; 0: after them                          */
     double tune_seconds[8];   /* S-apply time of each tried launch shape (0: not tried)  */
-    int device_error;         /* 1 if a Schwarz kernel gave up waiting for its factor copy
-                                 since the last fcm_precond_build or solve (its output is then wrong) */
+    int device_error;         /* 1 if a kernel of an S or K apply gave up waiting for its factor (or element matrix)
+                                 copy since the last fcm_precond_build or solve (its output is then wrong) */
     int64_t n_factors_ff;     /* factors stored as double-float pairs (FCM_PREC_MIXED, cond > cond_fp64) */
     int64_t n_gemm_blocks;    /* blocks applied by the shared-factor dense product        */
     int k_double_float;       /* 1: K applied in double-float arithmetic (fcm_set_k_precision) */
@@ -247,7 +247,8 @@ enum { FCM_K_FP64 = 0, FCM_K_DOUBLE_FLOAT = 1 };
  * sums on the FP32 pipe, about 2^-46 relative per contraction (K x within
  * ~1e-13 of the FP64 result); GB300's FP32 pipe is 64 times wider than its
  * FP64 pipe.  The first switch to double-float stores a float-pair copy of
- * the element matrices (fcm_info.element_bytes more device memory).  Captured
+ * the element matrices (as much device memory as fcm_info.element_bytes; half of
+ * it at p <= 2, where symmetric pairs of entries are stored once).  Captured
  * solver graphs are dropped.  FCM_EINVAL for another mode. */
 fcm_status fcm_set_k_precision(fcm_ctx *ctx, int mode);
 
@@ -256,9 +257,10 @@ fcm_status fcm_set_k_precision(fcm_ctx *ctx, int mode);
  * fcm_apply_S of column k.  FCM_EINVAL for nrhs outside 1..8. */
 fcm_status fcm_apply_S_many(fcm_ctx *ctx, const double *r_dev, int nrhs, double *z_dev);
 
-/* Failure detection: polls of the bounded mbarrier wait with which a Schwarz
- * kernel waits for a bulk copy of a shared factor into shared memory (default
- * 2^21).  A wait that runs out lets the copies in flight land, marks the apply
+/* Failure detection: polls of the bounded mbarrier wait with which a kernel of
+ * the S apply (factors) or of the double-float K apply (element matrices, p <= 2)
+ * waits for a bulk copy into shared memory (default 2^21).  A wait that runs
+ * out lets the copies in flight land, marks the apply
  * as failed and returns; the solves then stop with FCM_ETIMEOUT (and
  * fcm_info.device_error reports it after fcm_apply_S).  tries = 0 gives up at
  * the first poll (for tests); tries < 0 restores the default.  Captured solver

@@ -68,7 +68,6 @@ struct StreamScope {
 
 void apply_K_dev(fcm_ctx *C, const double *x, double *y, const int *done)
 {
-    fcm::launch_zero(y, C->nlat, done, C->stream);
     if (C->k_ff)
         fcm::launch_k_apply_ff(C->p, C->g, x, y, C->d_mask, C->d_elem_ff, C->kc, done, C->stream, C->ks);
     else
@@ -176,7 +175,8 @@ void free_ctx(fcm_ctx *C)
 {
     if (!C) return;
     destroy_graph(C);
-    void *ptrs[] = {C->d_elem, C->d_elem_ff, C->d_cell_elem, C->d_mask, C->d_rhs, C->d_cells, C->d_uncut, C->d_f64, C->d_f32,
+    void *ptrs[] = {C->d_elem, C->d_elem_ff, C->d_cell_elem, C->d_mask, C->d_rhs, C->d_cells, C->d_uncut, C->d_modal,
+                    C->d_zk, C->d_f64, C->d_f32,
                     C->d_slots, C->d_slot_of, C->d_items, C->d_zb, C->d_mzb, C->d_tc_tiles, C->d_tc_ft,
                     C->d_eta, C->d_jac, C->d_err,
                     C->d_x, C->d_r, C->d_z, C->d_p, C->d_q, C->d_b, C->d_t, C->d_partial, C->d_counter, C->d_s,
@@ -295,30 +295,49 @@ fcm_status fcm_setup(const fcm_grid *grid, const fcm_geometry *geom, int p, doub
         SETUP_CUDA(cudaStreamSynchronize(st));
     }
     C->element_bytes = (int64_t)(sizeof(double) * ne2 * nelem);
-    // active cells grouped by parity colour: uncut (matrix-free) and cut (own element matrix)
-    std::vector<int2> cells;
+    // active cells: uncut (matrix-free) and cut (own element matrix)
+    std::vector<fcm::CutCell> cells;
     std::vector<int> uncut;
+    auto cut_cell = [&](int64_t ci, int elem) {
+        const int64_t cx = ci % hp.n[0], cy = (ci / hp.n[0]) % hp.n[1], cz = ci / ((int64_t)hp.n[0] * hp.n[1]);
+        return fcm::CutCell{3 * (p * cx + hp.M[0] * (p * cy + hp.M[1] * (p * cz))), (int)ci, elem};
+    };
     cells.reserve(hp.ncut);
     uncut.reserve(hp.nactive);
-    C->kc.cut_off[0] = 0;
-    C->kc.uncut_off[0] = 0;
-    for (int col = 0; col < 8; ++col) {
-        for (int64_t ci = 0; ci < hp.ncells; ++ci) {
-            if (hp.cell_elem[ci] < 0) continue;
-            const int cx = (int)(ci % hp.n[0]), cy = (int)((ci / hp.n[0]) % hp.n[1]), cz = (int)(ci / ((int64_t)hp.n[0] * hp.n[1]));
-            if ((cx & 1) + 2 * (cy & 1) + 4 * (cz & 1) != col) continue;
-            if (hp.cell_elem[ci] == 0) uncut.push_back((int)ci);
-            else cells.push_back(make_int2((int)ci, hp.cell_elem[ci]));
-        }
-        C->kc.cut_off[col + 1] = (int)cells.size();
-        C->kc.uncut_off[col + 1] = (int)uncut.size();
+    for (int64_t ci = 0; ci < hp.ncells; ++ci) {
+        if (hp.cell_elem[ci] == 0) uncut.push_back((int)ci);
+        else if (hp.cell_elem[ci] > 0) cells.push_back(cut_cell(ci, hp.cell_elem[ci]));
+    }
+    if (fcm::k_dense_uncut(p, (int64_t)uncut.size())) {
+        for (int ci : uncut) cells.push_back(cut_cell(ci, 0));
+        uncut.clear();
     }
     SETUP_CUDA(dalloc(&C->d_cells, cells.size()));
-    SETUP_CUDA(cudaMemcpyAsync(C->d_cells, cells.data(), sizeof(int2) * cells.size(), cudaMemcpyHostToDevice, st));
+    SETUP_CUDA(cudaMemcpyAsync(C->d_cells, cells.data(), sizeof(fcm::CutCell) * cells.size(), cudaMemcpyHostToDevice, st));
     SETUP_CUDA(dalloc(&C->d_uncut, uncut.size()));
     SETUP_CUDA(cudaMemcpyAsync(C->d_uncut, uncut.data(), sizeof(int) * uncut.size(), cudaMemcpyHostToDevice, st));
+    std::vector<double> modal;
+    fcm::make_modal_tables(hp.h, hp.E, hp.nu, p, modal);
+    SETUP_CUDA(dalloc(&C->d_modal, 2 * modal.size()));
+    SETUP_CUDA(cudaMemcpyAsync(C->d_modal, modal.data(), sizeof(double) * modal.size(), cudaMemcpyHostToDevice, st));
+    float2 *modal_ff = reinterpret_cast<float2 *>(C->d_modal + modal.size());
+    fcm::launch_to_ff_pairs(C->d_modal, modal_ff, (int64_t)modal.size(), st);
+    SETUP_CUDA(cudaGetLastError());
+    SETUP_CUDA(dalloc(&C->d_zk, (size_t)hp.ne * hp.ncells));
     C->kc.cut = C->d_cells;
     C->kc.uncut = C->d_uncut;
+    C->kc.n_cut = (int)cells.size();
+    C->kc.n_uncut = (int)uncut.size();
+    C->kc.cell_elem = C->d_cell_elem;
+    C->kc.modal = C->d_modal;
+    C->kc.modal_ff = modal_ff;
+    C->kc.zk = C->d_zk;
+    SETUP_CUDA(dalloc(&C->d_err, 1));
+    SETUP_CUDA(cudaMemsetAsync(C->d_err, 0, sizeof(int), st));
+    C->kc.err = C->d_err;
+    C->kc.wait_tries = C->wait_tries;
+    SETUP_CUDA(fcm::k_prepare(p));
+    SETUP_CUDA(fcm::k_prepare_ff(p));
     fcm::make_sf_tables(hp, C->kc.sf);
     fcm::make_sf_tables_ff(C->kc.sf, C->kc.sff);
     // solver workspace
@@ -404,9 +423,7 @@ fcm_status fcm_info(const fcm_ctx *C, fcm_info_t *out)
         out->s_apply_launches = C->have_precond ? (tc ? 1 : 0) + ((tc ? pl.n_tiles32_plain : pl.n_tiles32) > 0) +
                                                       (pl.n_tiles64 > 0) + own + 1
                                                 : 0;
-        int k = 1;  // zero y
-        for (int c = 0; c < 8; ++c)
-            k += (C->kc.uncut_off[c + 1] > C->kc.uncut_off[c]) + (C->kc.cut_off[c + 1] > C->kc.cut_off[c]);
+        const int k = (C->kc.n_uncut > 0) + (C->kc.n_cut > 0) + 1;  // uncut cells, cut cells, sum
         out->k_apply_launches = k;
     }
     out->n_gemm_blocks = C->n_gemm_blocks;
@@ -735,9 +752,9 @@ fcm_status fcm_set_k_precision(fcm_ctx *C, int mode)
     }
     StreamScope sc(C);
     if (mode == FCM_K_DOUBLE_FLOAT && !C->d_elem_ff) {
-        const int64_t n = C->element_bytes / (int64_t)sizeof(double);
-        API_CUDA(C, cudaMalloc(&C->d_elem_ff, sizeof(float2) * (size_t)std::max<int64_t>(n, 1)));
-        fcm::launch_to_ff_pairs(C->d_elem, C->d_elem_ff, n, C->stream);
+        const int64_t nelem = 1 + C->hp.ncut;
+        API_CUDA(C, cudaMalloc(&C->d_elem_ff, sizeof(float2) * (size_t)fcm::element_ff_entries(C->p, nelem)));
+        fcm::launch_element_ff(C->p, C->d_elem, C->d_elem_ff, nelem, C->stream);
         API_CUDA(C, cudaGetLastError());
         API_CUDA(C, cudaStreamSynchronize(C->stream));
     }
@@ -755,6 +772,7 @@ fcm_status fcm_set_wait_limit(fcm_ctx *C, int tries)
     if (!C) return FCM_EINVAL;
     C->wait_tries = tries < 0 ? fcm::kWaitTries : tries;
     C->plan.wait_tries = C->wait_tries;
+    C->kc.wait_tries = C->wait_tries;
     // the captured graphs hold the plan's launch parameters
     destroy_graph(C);
     fcm::fcg_forget_graph(C->fcg);

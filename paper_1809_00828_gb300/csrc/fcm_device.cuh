@@ -48,16 +48,34 @@ struct SfTablesFF {
 };
 void make_sf_tables_ff(const SfTables &T, SfTablesFF &F);
 
-// Active cells of the K apply, grouped by parity colour: uncut cells (matrix-free,
-// sum-factorised) and cut cells (their own dense element matrix).
+// A cell of the dense product: its lattice DOF at the low corner, cell id and element matrix.
+struct CutCell {
+    int64_t base;
+    int cell, elem;
+};
+
+// Active cells of the K apply, in cell order: uncut cells (matrix-free) and cut cells (their own dense
+// element matrix).
 struct KCells {
-    const int *uncut;     // cell ids
-    const int2 *cut;      // (cell id, element id)
-    int uncut_off[9];
-    int cut_off[9];
-    SfTables sf;
+    const int *uncut;           // cell ids
+    const CutCell *cut;         // element 0 (the reference matrix) for uncut cells taken along (k_dense_uncut)
+    int n_uncut, n_cut;
+    int *err;                   // device flag, set to 1 by a bulk-copy wait that ran out
+    int wait_tries;             // polls of a bulk-copy wait before it gives up
+    const int32_t *cell_elem;   // per cell, negative where inactive
+    const double *modal;        // weight tables of the modal form (make_modal_tables; p <= 3)
+    const float2 *modal_ff;     // the same as float pairs
+    void *zk;                   // slots: 3 (p+1)^3 x ncells entries of 8 bytes (FP64 or float pairs)
+    SfTables sf;                // dense tables (p = 4)
     SfTablesFF sff;
 };
+// Whether n uncut cells go with the cut cells' dense product (a CTA per cell) instead of the modal form (32
+// cells per CTA): a grid of few cells leaves most SMs idle in the modal form, whose 32 cells take one SM's
+// FP64 pipe as long as about 5 (p = 2: 19 us, against 4.7 us for a cell's 81^2 dense product) or 2.5 (p = 3)
+// dense cells, so it pays from that many cells per SM on.  p = 1: 4.7 KB of K_ref against 250 operations.
+inline bool k_dense_uncut(int p, int64_t n) { return n <= 152 * (p == 1 ? 8 : p == 2 ? 4 : p == 3 ? 2 : 0); }
+// weight tables of fcm_modal.cuh: 3 components x kModalTabs x (p+1)^3
+void make_modal_tables(const double *h, double E, double nu, int p, std::vector<double> &tab);
 
 // Launch plan of the Schwarz apply (fcm_schwarz.cu).  Every block has a slot: its record
 // (factor offset, vertex or cell id, storage: 0 FP64, 1 FP32, 2 double-float) and nslots * zs
@@ -101,8 +119,8 @@ struct SchwarzPlan {
     cudaEvent_t ev_fork, ev_join;
 };
 
-// Second stream of the K apply: per colour, the cut cells run on `side` beside the uncut cells on the
-// main stream (the two sets are DOF-disjoint within a colour); null side: one stream.
+// Second stream of the K apply: the cut cells run on `side` beside the uncut cells on the main stream (every
+// cell has a slot of its own); null side: one stream.
 struct KStreams {
     cudaStream_t side;
     cudaEvent_t fork, join;
@@ -116,7 +134,14 @@ void launch_k_apply(int p, const Grid3 &g, const double *x, double *y, const uin
 // float pairs
 void launch_k_apply_ff(int p, const Grid3 &g, const double *x, double *y, const uint8_t *mask, const float2 *elem,
                        const KCells &kc, const int *done, cudaStream_t s, const KStreams &ks);
+// kernel attributes (dynamic shared memory); host calls, outside stream capture
+cudaError_t k_prepare(int p);
+cudaError_t k_prepare_ff(int p);
 void launch_to_ff_pairs(const double *in, float2 *out, int64_t n, cudaStream_t s);
+// float-pair copy of nelem element matrices in the layout of the double-float K apply (folded at p <= 2),
+// and its entries
+int64_t element_ff_entries(int p, int64_t nelem);
+void launch_element_ff(int p, const double *in, float2 *out, int64_t nelem, cudaStream_t s);
 void launch_schwarz_apply(int p, const Grid3 &g, const double *r, double *z, const double *fpool64,
                           const float *fpool32, const SchwarzPlan &plan, const int *done, cudaStream_t s);
 void launch_schwarz_apply_multi(int p, const double *r, double *z, int64_t nlat, int nr, const double *f64,
@@ -140,7 +165,6 @@ constexpr int kWaitTries = 1 << 21;
 void launch_mask_copy(const double *in, double *out, const uint8_t *mask, int64_t n, cudaStream_t s);
 // fcm_noalloc.cu: device address of the static scratch of fcm_apply_S_noalloc on the current device
 cudaError_t noalloc_scratch_address(double **out);
-void launch_zero(double *v, int64_t n, const int *done, cudaStream_t s);
 
 // CG building blocks (fcm_solver.cu)
 struct CgWork {
@@ -212,8 +236,10 @@ struct fcm_ctx {
     uint8_t *d_mask = nullptr;       // per lattice DOF
     double *d_rhs = nullptr;         // load case 0
     float *d_eta = nullptr;          // volume fraction per cell
-    int2 *d_cells = nullptr;         // cut cells by colour: (cell, element id)
-    int *d_uncut = nullptr;          // uncut cells by colour
+    fcm::CutCell *d_cells = nullptr; // cells of the dense product
+    int *d_uncut = nullptr;          // uncut cells
+    double *d_modal = nullptr;       // weight tables of the modal form, FP64 then float pairs
+    double *d_zk = nullptr;          // slots of the K apply
     fcm::KCells kc = {};
     int64_t element_bytes = 0;
     double setup_seconds = 0.0;
@@ -233,7 +259,7 @@ struct fcm_ctx {
     int64_t n_ff_factors = 0;        // factors stored as double-float pairs
     int64_t n_gemm_blocks = 0;       // blocks applied by the shared-factor GEMM
     double *d_jac = nullptr;         // diagonal part of S (element blocks), lattice; null if none
-    int *d_err = nullptr;            // set by a Schwarz CTA whose bulk-copy wait ran out
+    int *d_err = nullptr;            // set by a CTA (Schwarz or K apply) whose bulk-copy wait ran out
     double *noalloc_scratch = nullptr;  // device address of fcm_apply_S_noalloc's static scratch
     std::string noalloc_err;            // why it is null (problem too large, or the lookup failed)
     int device = 0;                     // CUDA device current at fcm_setup

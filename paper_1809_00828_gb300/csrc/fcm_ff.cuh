@@ -55,9 +55,17 @@ __device__ __forceinline__ void split_bits(double x, float &hi, float &lo)
     if (e > 0) lo = __uint_as_float(sign | ((unsigned)e << 23) | ((q & ((1u << MB) - 1)) << (23 - MB)));
 }
 
-// x as a float pair, x = hi + lo to 2^-48 relative
+// x as a float pair, x = hi + lo to 2^-48 relative.  2^-74 <= |x| < 2^128 (lo then is a normal number): hi
+// takes the top 23 fraction bits, the other 29 become lo by an integer-to-float conversion (round to nearest
+// even) and an exact scaling, 12 instructions where split_bits needs about 30; other values go there.
 __device__ __forceinline__ float2 split_ff(double x)
 {
+    const unsigned uh = (unsigned)__double2hiint(x), ul = (unsigned)__double2loint(x);
+    if ((uh & 0x7FF00000u) - (949u << 20) < (202u << 20)) {  // exponent field 949 .. 1150
+        const unsigned h = (__funnelshift_l(ul, uh, 3) - (896u << 23)) | (uh & 0x80000000u);
+        const float scale = __uint_as_float((h & 0xFF800000u) - (52u << 23));
+        return make_float2(__uint_as_float(h), __fmul_rn(__uint2float_rn(ul & 0x1FFFFFFFu), scale));
+    }
     float h, l;
     split_bits<23>(x, h, l);
     return make_float2(h, l);

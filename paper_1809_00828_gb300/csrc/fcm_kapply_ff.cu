@@ -1,17 +1,18 @@
-// Stiffness apply y += K x (Sec. 2.1 Eq. (1)) in double-float arithmetic on the FP32 pipe.
+// Stiffness apply y = K x (Sec. 2.1 Eq. (1)) in double-float arithmetic on the FP32 pipe.
 //
-// The same two kernels as fcm_kernels.cu -- matrix-free sum factorisation for uncut cells, the
-// cell's own dense element matrix for cut cells, 8 parity colours without atomics -- with every
-// FP64 multiply-add replaced by a compensated double-float one (fcm_ff.cuh): values and tables are
-// float pairs (hi, lo), a product is Dekker's exact product by FMA plus the cross terms, sums run by
-// TwoSum.  Each contraction of Q terms is accurate to about 2^-46 relative, so K x agrees with the
-// FP64 kernels to ~1e-13, while GB300's FP32 pipe (128 lanes per SM) replaces its FP64 pipe (2
-// multiply-adds per clock per SM).  x is read and split by integer operations; the result is added
-// into the FP64 vector y, the only FP64 arithmetic left (two adds per DOF and cell).
+// The same steps as fcm_kernels.cu -- uncut cells in Legendre modal form, cut cells with their own dense
+// element matrix, each into its slot of Zk, then one sum per lattice node -- with every FP64 multiply-add
+// replaced by a compensated double-float one (fcm_ff.cuh): values and tables are float pairs (hi, lo), a
+// product is Dekker's exact product by FMA plus the cross terms, sums run by TwoSum.  Each contraction is
+// accurate to about 2^-46 relative, so K x agrees with the FP64 kernels to ~1e-13, while GB300's FP32 pipe
+// (128 lanes per SM) replaces its FP64 pipe (2 multiply-adds per clock per SM).  x is read and split by
+// integer operations; the slots hold float pairs, and one FP64 add per DOF is left.
 #include <cuda_runtime.h>
 
 #include "fcm_device.cuh"
 #include "fcm_ff.cuh"
+#include "fcm_modal.cuh"
+#include "fcm_sym.cuh"
 
 namespace fcm {
 
@@ -38,44 +39,69 @@ struct FFAcc {
     __device__ __forceinline__ float2 get() const { return ff_norm(S, C); }
 };
 
-// y += K_e x_e over the cut cells of one colour, K_e stored as double-float pairs (symmetric; column t
-// read as row t); rows that are not free stay untouched.
+// Zk slots of the cut cells: K_e x_e, K_e stored as double-float pairs (symmetric; column t read as row t).
 template <int P>
 __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
-    ebe_apply_ff_kernel(const double *__restrict__ x, double *__restrict__ y, const uint8_t *__restrict__ mask,
-                        const float2 *__restrict__ elem, const int2 *__restrict__ cells, Grid3 g,
-                        const int *__restrict__ done)
+    ebe_apply_ff_kernel(const double *__restrict__ x, float2 *__restrict__ zk, const float2 *__restrict__ elem,
+                        const CutCell *__restrict__ cells, Grid3 g, int64_t nc, const int *__restrict__ done)
 {
-    constexpr int Q = P + 1, NL = Q * Q * Q, NE = 3 * NL;
+    constexpr int Q = P + 1, NE = 3 * Q * Q * Q;
     if (done && *done) return;
     __shared__ float2 xe[NE];
-    __shared__ int64_t node[NL];
-    const int2 ce = cells[blockIdx.x];
-    const int cx = ce.x % g.n[0], cy = (ce.x / g.n[0]) % g.n[1], cz = ce.x / (g.n[0] * g.n[1]);
-    for (int t = threadIdx.x; t < NL; t += blockDim.x) {
-        const int ix = t % Q, iy = (t / Q) % Q, iz = t / (Q * Q);
-        node[t] = (P * cx + ix) + (int64_t)g.M[0] * ((P * cy + iy) + (int64_t)g.M[1] * (P * cz + iz));
+    const CutCell ce = cells[blockIdx.x];
+    for (int t = threadIdx.x; t < NE; t += blockDim.x) {
+        const int l = t / 3, ix = l % Q, iy = (l / Q) % Q, iz = l / (Q * Q);
+        xe[t] = split_ff(x[ce.base + 3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3]);
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < NE; t += blockDim.x) xe[t] = split_ff(x[3 * node[t / 3] + t % 3]);
-    __syncthreads();
-    const float2 *__restrict__ K = elem + (size_t)ce.y * NE * NE;
+    const float2 *__restrict__ K = elem + (size_t)ce.elem * NE * NE;
     for (int t = threadIdx.x; t < NE; t += blockDim.x) {
         FFAcc s;
 #pragma unroll 8
         for (int j = 0; j < NE; ++j) s.add(__ldcs(K + (size_t)j * NE + t), xe[j]);
-        const int64_t gi = 3 * node[t / 3] + t % 3;
-        if (mask[gi]) y[gi] += ff_to_double(s.get());
+        zk[t * nc + ce.cell] = s.get();
     }
 }
 
-// y += K_ref x_e for the uncut cells of one colour, matrix-free: the steps of sf_apply_kernel
+// The same for p <= 2, K_e folded (fcm_sym.cuh): half of the matrix's bytes.  The FP32 pipe and the issue slots
+// bound it now (12 operations per entry and 8 around them): 370 us for 72,180 cells (1.92 GB, 285 us at the
+// copy rate) where streaming the full matrices took 697 us (3.8 GB).
+template <int P>
+__global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
+    ebe_fold_ff_kernel(const double *__restrict__ x, float2 *__restrict__ zk, const float2 *__restrict__ elem,
+                       const CutCell *__restrict__ cells, Grid3 g, int64_t nc, int *err, int wait_tries,
+                       const int *__restrict__ done)
+{
+    constexpr int Q = P + 1, NE = 3 * Q * Q * Q;
+    if (done && *done) return;
+    __shared__ __align__(16) float2 xe[(NE + 3) / 4 * 4], m[fold_entries(NE)];
+    __shared__ uint64_t bar;
+    const CutCell ce = cells[blockIdx.x];
+    const int t = threadIdx.x, l = t / 3, ix = l % Q, iy = (l / Q) % Q, iz = l / (Q * Q);
+    if (t == 0) {
+        mbar_init(&bar);
+        mbar_expect(&bar, fold_entries(NE) * 8);
+        bulk_g2s(m, elem + (size_t)ce.elem * fold_entries(NE), fold_entries(NE) * 8, &bar);
+    }
+    if (t < NE) xe[t] = split_ff(__ldg(x + ce.base + 3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3));
+    __syncthreads();
+    if (!mbar_wait(&bar, 0, wait_tries)) {
+        atomicExch(err, 1);
+        mbar_wait(&bar, 0, kDrainTries);
+        return;
+    }
+    float S[1] = {0.f}, C[1] = {0.f};
+    fold_dot<NE, 1>(m, NE, t & ~31, min(t, NE - 1), xe, 1, S, C);
+    if (t < NE) zk[t * nc + ce.cell] = ff_norm(S[0], C[0]);
+}
+
+// Zk slots K_ref x_e of the uncut cells (p = 4), matrix-free: the steps of sf_apply_kernel
 // (interpolation to the Gauss points by 1D contractions, collocation derivative, weighted stress,
 // transposed steps) in double-float arithmetic.  One thread per point (and node) of a cell.
 template <int P>
 __global__ void __launch_bounds__(256)
-    sf_apply_ff_kernel(const double *__restrict__ x, double *__restrict__ y, const uint8_t *__restrict__ mask,
-                       const int *__restrict__ cells, int ncells, Grid3 g, SfTablesFF T, const int *__restrict__ done)
+    sf_apply_ff_kernel(const double *__restrict__ x, float2 *__restrict__ zk, const int *__restrict__ cells, int ncells,
+                       Grid3 g, int64_t nc, SfTablesFF T, const int *__restrict__ done)
 {
     constexpr int Q = P + 1, Q3 = Q * Q * Q, TPC = rnd32k(Q3), CPC = 256 / TPC;
     if (done && *done) return;
@@ -93,8 +119,9 @@ __global__ void __launch_bounds__(256)
     const bool on = cidx < ncells && t < Q3;
     const int tx = t % Q, ty = (t / Q) % Q, tz = t / (Q * Q);
     int64_t node = 0;
+    int cell = 0;
     if (on) {
-        const int cell = cells[cidx];
+        cell = cells[cidx];
         const int cx = cell % g.n[0], cy = (cell / g.n[0]) % g.n[1], cz = cell / (g.n[0] * g.n[1]);
         node = (P * cx + tx) + (int64_t)g.M[0] * ((P * cy + ty) + (int64_t)g.M[1] * (P * cz + tz));
         for (int c = 0; c < 3; ++c) U[lc][c][t] = split_ff(x[3 * node + c]);
@@ -195,8 +222,21 @@ __global__ void __launch_bounds__(256)
         }
     }
     if (on)
-        for (int c = 0; c < 3; ++c)
-            if (mask[3 * node + c]) y[3 * node + c] += ff_to_double(out[c]);
+        for (int c = 0; c < 3; ++c) zk[(3 * t + c) * nc + cell] = out[c];
+}
+
+template <int P>
+void uncut_launch_ff(const Grid3 &g, const double *x, float2 *zk, const KCells &kc, const int *done, cudaStream_t s)
+{
+    const int64_t nc = (int64_t)g.n[0] * g.n[1] * g.n[2];
+    if constexpr (P <= 3) {
+        modal_apply_kernel<P, ModalFF><<<(kc.n_uncut + 31) / 32, kModalThreads, modal_smem_bytes(P), s>>>(
+            x, zk, kc.uncut, kc.n_uncut, g, nc, kc.modal_ff, done);
+    } else {
+        constexpr int CPC = 256 / rnd32k((P + 1) * (P + 1) * (P + 1));
+        sf_apply_ff_kernel<P><<<(kc.n_uncut + CPC - 1) / CPC, 256, 0, s>>>(x, zk, kc.uncut, kc.n_uncut, g, nc, kc.sff,
+                                                                          done);
+    }
 }
 
 template <int P>
@@ -204,35 +244,60 @@ void k_launch_ff(const Grid3 &g, const double *x, double *y, const uint8_t *mask
                  const KCells &kc, const int *done, cudaStream_t s, const KStreams &ks)
 {
     constexpr int NE = 3 * (P + 1) * (P + 1) * (P + 1);
-    constexpr int CPC = 256 / rnd32k((P + 1) * (P + 1) * (P + 1));
-    for (int c = 0; c < 8; ++c) {
-        const int nu = kc.uncut_off[c + 1] - kc.uncut_off[c];
-        const int nc = kc.cut_off[c + 1] - kc.cut_off[c];
-        // cut and uncut cells of one colour share no DOF: the cut cells (HBM-bound) run beside the uncut
-        // ones (FP32-pipe and latency bound)
-        const bool fork = ks.side && nu > 0 && nc > 0;
-        if (fork) {
-            cudaEventRecord(ks.fork, s);
-            cudaStreamWaitEvent(ks.side, ks.fork, 0);
-        }
-        if (nc > 0)
-            ebe_apply_ff_kernel<P><<<nc, ebe_threads(NE), 0, fork ? ks.side : s>>>(x, y, mask, elem,
-                                                                                  kc.cut + kc.cut_off[c], g, done);
-        if (nu > 0)
-            sf_apply_ff_kernel<P><<<(nu + CPC - 1) / CPC, 256, 0, s>>>(x, y, mask, kc.uncut + kc.uncut_off[c], nu, g,
-                                                                      kc.sff, done);
-        if (fork) {
-            cudaEventRecord(ks.join, ks.side);
-            cudaStreamWaitEvent(s, ks.join, 0);
-        }
+    const int64_t nc = (int64_t)g.n[0] * g.n[1] * g.n[2];
+    float2 *zk = reinterpret_cast<float2 *>(kc.zk);
+    // the cut cells (HBM-bound) run beside the uncut ones (FP32-pipe bound)
+    const bool fork = ks.side && kc.n_uncut > 0 && kc.n_cut > 0;
+    if (fork) {
+        cudaEventRecord(ks.fork, s);
+        cudaStreamWaitEvent(ks.side, ks.fork, 0);
     }
+    if (kc.n_cut > 0) {
+        if constexpr (P <= 2)
+            ebe_fold_ff_kernel<P><<<kc.n_cut, ebe_threads(NE), 0, fork ? ks.side : s>>>(x, zk, elem, kc.cut, g, nc, kc.err,
+                                                                                     kc.wait_tries, done);
+        else
+            ebe_apply_ff_kernel<P><<<kc.n_cut, ebe_threads(NE), 0, fork ? ks.side : s>>>(x, zk, elem, kc.cut, g, nc, done);
+    }
+    if (kc.n_uncut > 0) uncut_launch_ff<P>(g, x, zk, kc, done, s);
+    if (fork) {
+        cudaEventRecord(ks.join, ks.side);
+        cudaStreamWaitEvent(s, ks.join, 0);
+    }
+    k_sum_kernel<P, ModalFF><<<k_sum_blocks(g), dim3(32, kSumWarps), 0, s>>>(zk, kc.cell_elem, mask, y, g, nc, done);
 }
 
-// FP64 element matrices -> double-float pairs
+template <int P>
+cudaError_t k_prepare_ff_p()
+{
+    if constexpr (P <= 3)
+        return cudaFuncSetAttribute(modal_apply_kernel<P, ModalFF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    modal_smem_bytes(P));
+    return cudaSuccess;
+}
+
+int grid_of(int64_t n)
+{
+    const int64_t b = (n + 255) / 256;
+    return (int)(b < 1 ? 1 : b < 152 * 16 ? b : 152 * 16);
+}
+
+// FP64 values -> double-float pairs
 __global__ void to_ff_pairs_kernel(const double *__restrict__ in, float2 *__restrict__ out, int64_t n)
 {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
         out[e] = split_ff(in[e]);
+}
+
+// the same with every ne x ne matrix folded (padding entries 0)
+__global__ void fold_ff_pairs_kernel(const double *__restrict__ in, float2 *__restrict__ out, int ne, int64_t n)
+{
+    const int fe = fold_entries(ne), hw = fold_h(ne) * fold_w(ne);
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * fe; e += (int64_t)gridDim.x * blockDim.x) {
+        int i, j;
+        const bool on = fold_entry(ne, (int)(e % fe), i, j) && (int)(e % fe) < hw;
+        out[e] = on ? split_ff(in[e / fe * ne * ne + (int64_t)i * ne + j]) : make_float2(0.f, 0.f);
+    }
 }
 
 }  // namespace
@@ -249,10 +314,34 @@ void launch_k_apply_ff(int p, const Grid3 &g, const double *x, double *y, const 
     }
 }
 
+cudaError_t k_prepare_ff(int p)
+{
+    switch (p) {
+    case 1: return k_prepare_ff_p<1>();
+    case 2: return k_prepare_ff_p<2>();
+    case 3: return k_prepare_ff_p<3>();
+    default: return k_prepare_ff_p<4>();
+    }
+}
+
 void launch_to_ff_pairs(const double *in, float2 *out, int64_t n, cudaStream_t s)
 {
-    const int64_t b = (n + 255) / 256;
-    to_ff_pairs_kernel<<<(int)(b < 152 * 16 ? (b < 1 ? 1 : b) : 152 * 16), 256, 0, s>>>(in, out, n);
+    to_ff_pairs_kernel<<<grid_of(n), 256, 0, s>>>(in, out, n);
+}
+
+int64_t element_ff_entries(int p, int64_t nelem)
+{
+    const int ne = 3 * (p + 1) * (p + 1) * (p + 1);
+    return nelem * (p <= 2 ? fold_entries(ne) : ne * ne);
+}
+
+void launch_element_ff(int p, const double *in, float2 *out, int64_t nelem, cudaStream_t s)
+{
+    const int ne = 3 * (p + 1) * (p + 1) * (p + 1);
+    if (p <= 2)
+        fold_ff_pairs_kernel<<<grid_of(element_ff_entries(p, nelem)), 256, 0, s>>>(in, out, ne, nelem);
+    else
+        launch_to_ff_pairs(in, out, nelem * ne * ne, s);
 }
 
 void make_sf_tables_ff(const SfTables &T, SfTablesFF &F)

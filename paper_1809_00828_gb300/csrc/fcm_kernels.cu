@@ -1,49 +1,62 @@
-// Stiffness apply y = K x of the finite cell Schwarz-PCG on sm_103a (Sec. 2.1 Eq. (1)): cells
-// processed in 8 parity colours so that cells of one launch share no lattice DOF and the scatter
-// needs no atomics; uncut cells matrix-free by sum factorisation, cut cells with their own dense
-// element matrix.  (The Schwarz apply is in fcm_schwarz.cu.)
+// Stiffness apply y = K x of the finite cell Schwarz-PCG on sm_103a (Sec. 2.1 Eq. (1)).
+//
+// Every active cell's product K_e x_e goes to a slot of its own (uncut cells matrix-free in Legendre modal
+// form, cut cells with their dense element matrix on a second stream beside them), then one kernel adds the
+// slots node by node (fcm_modal.cuh): three launches, no atomics, one fixed order of additions.  Eight
+// parity colours that added into y in place took 16 dependent launches, which a small grid pays in latency
+// (4^3 cells: K 8.5 us per launch) and a large one in tails.  (The Schwarz apply is in fcm_schwarz.cu.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
 #include "fcm_device.cuh"
+#include "fcm_modal.cuh"
 
 namespace fcm {
 
 namespace {
 
+// Threads of the cut-cell product: PARTS column ranges of a row on different warps, so that a row's chain of
+// FP64 multiply-adds is short (the FP64 pipe does 2 per clock per SM; one chain per row left a 4^3 grid's
+// 34 cells waiting on latency).
 __host__ __device__ constexpr int round32(int v) { return (v + 31) / 32 * 32; }
-// One thread per row up to 512 rows; larger blocks loop over rows.
-__host__ __device__ constexpr int threads_for(int rows) { return round32(rows) < 512 ? round32(rows) : 512; }
+__host__ __device__ constexpr int ebe_parts(int P) { return P <= 2 ? 4 : P == 3 ? 2 : 1; }
+__host__ __device__ constexpr int ebe_rows(int P) { return 3 * (P + 1) * (P + 1) * (P + 1); }
+__host__ __device__ constexpr int ebe_threads(int P) { return round32(ebe_rows(P)) * ebe_parts(P); }
 
-// y += K_e x_e over the active cells of one colour; rows that are not free stay untouched.
+// Zk slots of the cut cells: K_e x_e with the cell's own dense matrix (symmetric: column t read as row t, so
+// consecutive threads read consecutive entries).
 template <int P>
-__global__ void __launch_bounds__(threads_for(3 * (P + 1) * (P + 1) * (P + 1)))
-    ebe_apply_kernel(const double *__restrict__ x, double *__restrict__ y, const uint8_t *__restrict__ mask,
-                     const double *__restrict__ elem, const int2 *__restrict__ cells, Grid3 g,
-                     const int *__restrict__ done)
+__global__ void __launch_bounds__(ebe_threads(P))
+    ebe_apply_kernel(const double *__restrict__ x, double *__restrict__ zk, const double *__restrict__ elem,
+                     const CutCell *__restrict__ cells, Grid3 g, int64_t nc, const int *__restrict__ done)
 {
-    constexpr int Q = P + 1, NL = Q * Q * Q, NE = 3 * NL;
+    constexpr int Q = P + 1, NE = 3 * Q * Q * Q, R32 = round32(NE), PARTS = ebe_parts(P), JP = (NE + PARTS - 1) / PARTS;
     if (done && *done) return;
-    __shared__ double xe[NE];
-    __shared__ int64_t node[NL];
-    const int2 ce = cells[blockIdx.x];
-    const int cx = ce.x % g.n[0], cy = (ce.x / g.n[0]) % g.n[1], cz = ce.x / (g.n[0] * g.n[1]);
-    for (int t = threadIdx.x; t < NL; t += blockDim.x) {
-        const int ix = t % Q, iy = (t / Q) % Q, iz = t / (Q * Q);
-        node[t] = (P * cx + ix) + (int64_t)g.M[0] * ((P * cy + iy) + (int64_t)g.M[1] * (P * cz + iz));
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < NE; t += blockDim.x) xe[t] = x[3 * node[t / 3] + t % 3];
-    __syncthreads();
-    const double *__restrict__ K = elem + (size_t)ce.y * NE * NE;
+    __shared__ double xe[NE], part[PARTS > 1 ? (PARTS - 1) * NE : 1];
+    const CutCell ce = cells[blockIdx.x];
+    const double *xc = x + ce.base;
     for (int t = threadIdx.x; t < NE; t += blockDim.x) {
-        double s = 0.0;
-#pragma unroll 8
-        for (int j = 0; j < NE; ++j) s = fma(__ldg(K + (size_t)j * NE + t), xe[j], s);
-        const int64_t gi = 3 * node[t / 3] + t % 3;
-        if (mask[gi]) y[gi] += s;
+        const int l = t / 3, ix = l % Q, iy = (l / Q) % Q, iz = l / (Q * Q);
+        xe[t] = xc[3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3];
     }
+    __syncthreads();
+    const int t = threadIdx.x % R32, pt = threadIdx.x / R32;
+    double s = 0.0;
+    if (t < NE) {
+        const double *__restrict__ K = elem + (size_t)ce.elem * NE * NE + t;
+        const int j1 = min(NE, (pt + 1) * JP);
+#pragma unroll 8
+        for (int j = pt * JP; j < j1; ++j) s = fma(__ldg(K + (size_t)j * NE), xe[j], s);
+        if (pt > 0) part[(pt - 1) * NE + t] = s;
+    }
+    if constexpr (PARTS > 1) {
+        __syncthreads();
+        if (pt > 0 || t >= NE) return;
+#pragma unroll
+        for (int k = 0; k < PARTS - 1; ++k) s += part[k * NE + t];
+    }
+    if (t < NE) zk[t * nc + ce.cell] = s;
 }
 
 // Barrier among the threads of one cell: a warp when the cell's points fit one warp (p <= 2), else
@@ -57,7 +70,7 @@ __device__ __forceinline__ void cell_sync()
         __syncthreads();
 }
 
-// y += K_ref x_e for uncut cells of one colour, without the matrix.  Each displacement
+// Zk slots K_ref x_e of uncut cells, without the matrix, by sum factorisation (p = 4).  Each displacement
 // component is interpolated to the (p+1)^3 Gauss points by one-dimensional contractions along
 // x, y, z (sum factorisation); its gradient there follows from the collocation derivative on
 // the Gauss points (exact: the field has degree <= p per axis).  The weighted stress
@@ -67,8 +80,8 @@ __device__ __forceinline__ void cell_sync()
 // takes 9 (p+1)^6) and no matrix traffic.  Threads of a cell: one per point.
 template <int P>
 __global__ void __launch_bounds__(256)
-    sf_apply_kernel(const double *__restrict__ x, double *__restrict__ y, const uint8_t *__restrict__ mask,
-                    const int *__restrict__ cells, int ncells, Grid3 g, SfTables T, const int *__restrict__ done)
+    sf_apply_kernel(const double *__restrict__ x, double *__restrict__ zk, const int *__restrict__ cells, int ncells,
+                    Grid3 g, int64_t nc, SfTables T, const int *__restrict__ done)
 {
     constexpr int Q = P + 1, Q3 = Q * Q * Q, TPC = round32(Q3), CPC = 256 / TPC;
     if (done && *done) return;
@@ -86,8 +99,9 @@ __global__ void __launch_bounds__(256)
     const bool on = cidx < ncells && t < Q3;
     const int tx = t % Q, ty = (t / Q) % Q, tz = t / (Q * Q);
     int64_t node = 0;
+    int cell = 0;
     if (on) {
-        const int cell = cells[cidx];
+        cell = cells[cidx];
         const int cx = cell % g.n[0], cy = (cell / g.n[0]) % g.n[1], cz = cell / (g.n[0] * g.n[1]);
         node = (P * cx + tx) + (int64_t)g.M[0] * ((P * cy + ty) + (int64_t)g.M[1] * (P * cz + tz));
         for (int c = 0; c < 3; ++c) U[lc][c][t] = x[3 * node + c];
@@ -184,8 +198,7 @@ __global__ void __launch_bounds__(256)
         }
     }
     if (on)
-        for (int c = 0; c < 3; ++c)
-            if (mask[3 * node + c]) y[3 * node + c] += out[c];
+        for (int c = 0; c < 3; ++c) zk[(3 * t + c) * nc + cell] = out[c];
 }
 
 __global__ void mask_copy_kernel(const double *__restrict__ in, double *__restrict__ out,
@@ -195,39 +208,48 @@ __global__ void mask_copy_kernel(const double *__restrict__ in, double *__restri
         out[i] = mask[i] ? in[i] : 0.0;
 }
 
-__global__ void zero_kernel(double *__restrict__ v, int64_t n, const int *__restrict__ done)
+// p = 4: modal arrays of 125 modes do not fit a thread's registers; the dense-table form stays there.
+template <int P>
+void uncut_launch(const Grid3 &g, const double *x, double *zk, const KCells &kc, const int *done, cudaStream_t s)
 {
-    if (done && *done) return;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        v[i] = 0.0;
+    const int64_t nc = (int64_t)g.n[0] * g.n[1] * g.n[2];
+    if constexpr (P <= 3) {
+        modal_apply_kernel<P, ModalF64><<<(kc.n_uncut + 31) / 32, kModalThreads, modal_smem_bytes(P), s>>>(
+            x, zk, kc.uncut, kc.n_uncut, g, nc, kc.modal, done);
+    } else {
+        constexpr int CPC = 256 / round32((P + 1) * (P + 1) * (P + 1));
+        sf_apply_kernel<P><<<(kc.n_uncut + CPC - 1) / CPC, 256, 0, s>>>(x, zk, kc.uncut, kc.n_uncut, g, nc, kc.sf, done);
+    }
 }
 
 template <int P>
 void k_launch(const Grid3 &g, const double *x, double *y, const uint8_t *mask, const double *elem, const KCells &kc,
               const int *done, cudaStream_t s, const KStreams &ks)
 {
-    constexpr int NE = 3 * (P + 1) * (P + 1) * (P + 1);
-    constexpr int CPC = 256 / round32((P + 1) * (P + 1) * (P + 1));
-    for (int c = 0; c < 8; ++c) {
-        const int nu = kc.uncut_off[c + 1] - kc.uncut_off[c];
-        const int nc = kc.cut_off[c + 1] - kc.cut_off[c];
-        // cut and uncut cells of one colour share no DOF: the cut cells may run beside the uncut ones
-        const bool fork = ks.side && nu > 0 && nc > 0;
-        if (fork) {
-            cudaEventRecord(ks.fork, s);
-            cudaStreamWaitEvent(ks.side, ks.fork, 0);
-        }
-        if (nc > 0)
-            ebe_apply_kernel<P><<<nc, threads_for(NE), 0, fork ? ks.side : s>>>(x, y, mask, elem, kc.cut + kc.cut_off[c],
-                                                                               g, done);
-        if (nu > 0)
-            sf_apply_kernel<P><<<(nu + CPC - 1) / CPC, 256, 0, s>>>(x, y, mask, kc.uncut + kc.uncut_off[c], nu, g, kc.sf,
-                                                                   done);
-        if (fork) {
-            cudaEventRecord(ks.join, ks.side);
-            cudaStreamWaitEvent(s, ks.join, 0);
-        }
+    const int64_t nc = (int64_t)g.n[0] * g.n[1] * g.n[2];
+    double *zk = reinterpret_cast<double *>(kc.zk);
+    const bool fork = ks.side && kc.n_uncut > 0 && kc.n_cut > 0;
+    if (fork) {
+        cudaEventRecord(ks.fork, s);
+        cudaStreamWaitEvent(ks.side, ks.fork, 0);
     }
+    if (kc.n_cut > 0)
+        ebe_apply_kernel<P><<<kc.n_cut, ebe_threads(P), 0, fork ? ks.side : s>>>(x, zk, elem, kc.cut, g, nc, done);
+    if (kc.n_uncut > 0) uncut_launch<P>(g, x, zk, kc, done, s);
+    if (fork) {
+        cudaEventRecord(ks.join, ks.side);
+        cudaStreamWaitEvent(s, ks.join, 0);
+    }
+    k_sum_kernel<P, ModalF64><<<k_sum_blocks(g), dim3(32, kSumWarps), 0, s>>>(zk, kc.cell_elem, mask, y, g, nc, done);
+}
+
+template <int P>
+cudaError_t k_prepare_p()
+{
+    if constexpr (P <= 3)
+        return cudaFuncSetAttribute(modal_apply_kernel<P, ModalF64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    modal_smem_bytes(P));
+    return cudaSuccess;
 }
 
 int grid_for(int64_t n, int threads)
@@ -256,9 +278,48 @@ void launch_mask_copy(const double *in, double *out, const uint8_t *mask, int64_
     mask_copy_kernel<<<grid_for(n, 256), 256, 0, s>>>(in, out, mask, n);
 }
 
-void launch_zero(double *v, int64_t n, const int *done, cudaStream_t s)
+cudaError_t k_prepare(int p)
 {
-    zero_kernel<<<grid_for(n, 256), 256, 0, s>>>(v, n, done);
+    switch (p) {
+    case 1: return k_prepare_p<1>();
+    case 2: return k_prepare_p<2>();
+    case 3: return k_prepare_p<3>();
+    default: return k_prepare_p<4>();
+    }
+}
+
+void make_modal_tables(const double *h, double E, double nu, int p, std::vector<double> &tab)
+{
+    const int q = p + 1, q3 = q * q * q;
+    const double lam = E * nu / ((1.0 + nu) * (1.0 - 2.0 * nu)), mu = E / (2.0 * (1.0 + nu));
+    const double detJ = h[0] * h[1] * h[2] / 8.0;
+    const double k4 = kModalK42 * kModalK2;
+    const double kap[5] = {1.0, 1.0, kModalK2, kModalK3, k4}, rho[5] = {1.0, kModalK2, kModalK3, k4, 0.0};
+    tab.assign((size_t)3 * kModalTabs * q3, 0.0);
+    for (int c = 0; c < 3; ++c) {
+        const double H[3] = {2.0 / h[c], 2.0 / h[(c + 1) % 3], 2.0 / h[(c + 2) % 3]};
+        double *T = tab.data() + (size_t)c * kModalTabs * q3;
+        for (int i = 0; i < q3; ++i) {
+            const int a[3] = {i % q, (i / q) % q, i / (q * q)};
+            double own[3], mass[3], mix[3];  // per axis: both sides derived, neither, one
+            for (int d = 0; d < 3; ++d) {
+                own[d] = 2.0 * (2 * a[d] + 1) * rho[a[d]] * rho[a[d]];
+                mass[d] = kap[a[d]] * kap[a[d]] * 2.0 / (2 * a[d] + 1);
+                mix[d] = 2.0 * rho[a[d]] * kap[a[d]];
+            }
+            const double w = detJ / 64.0;
+            const double A0 = w * H[0] * H[0] * own[0] * mass[1] * mass[2], A1 = w * H[1] * H[1] * own[1] * mass[0] * mass[2],
+                         A2 = w * H[2] * H[2] * own[2] * mass[0] * mass[1];
+            const double B1 = w * H[0] * H[1] * mix[0] * mix[1] * mass[2], B2 = w * H[0] * H[2] * mix[0] * mix[2] * mass[1];
+            T[i] = (lam + 2.0 * mu) * A0;
+            T[q3 + i] = lam * B1;
+            T[2 * q3 + i] = lam * B2;
+            T[3 * q3 + i] = mu * A1;
+            T[4 * q3 + i] = mu * B1;
+            T[5 * q3 + i] = mu * A2;
+            T[6 * q3 + i] = mu * B2;
+        }
+    }
 }
 
 }  // namespace fcm

@@ -715,7 +715,6 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
     std::vector<int2> tiles(tiles32);
     tiles.insert(tiles.end(), tiles64.begin(), tiles64.end());
     PC_CUDA(cudaMemcpyAsync(d_tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, st));
-    if (!C->d_err) PC_CUDA(cudaMalloc(&C->d_err, sizeof(int)));
     PC_CUDA(cudaMemsetAsync(C->d_err, 0, sizeof(int), st));
     if (!C->side) {
         PC_CUDA(cudaStreamCreateWithFlags(&C->side, cudaStreamNonBlocking));

@@ -28,6 +28,8 @@
 
 #include "fcm_device.cuh"
 #include "fcm_ff.cuh"
+#include "fcm_sym.cuh"
+#include "fcm_tma.cuh"
 
 namespace fcm {
 
@@ -356,50 +358,6 @@ __global__ void __launch_bounds__(cols_threads(P))
 // accumulates rows 8 rg .. 8 rg + 7 for 8 columns (NC/8): two 16-byte reads of the stage and two of
 // the panel feed 64 multiply-adds.  Blocks with more rows than 8 x (threads / 8) take several passes
 // over the factor.
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_expect(uint64_t *bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-
-// dst, src and bytes multiples of 16
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Waits for phase `parity` of the barrier, giving up (false) after `tries` polls.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int tries)
-{
-    for (int i = 0; i < tries; ++i)
-        if (mbar_test(bar, parity)) return true;
-    return false;
-}
-
-// Polls of the wait that lets copies still in flight land before a CTA that gave up leaves.
-constexpr int kDrainTries = 1 << 22;
 
 // m consecutive values from shared memory at a pointer aligned to min(16, m sizeof(T)) bytes, in
 // 16-byte (or 8-byte) vector reads
