@@ -177,7 +177,7 @@ void free_ctx(fcm_ctx *C)
     destroy_graph(C);
     void *ptrs[] = {C->d_elem, C->d_elem_ff, C->d_cell_elem, C->d_mask, C->d_rhs, C->d_cells, C->d_uncut, C->d_modal,
                     C->d_zk, C->d_f64, C->d_f32,
-                    C->d_slots, C->d_slot_of, C->d_items, C->d_zb, C->d_mzb, C->d_tc_tiles, C->d_tc_ft,
+                    C->d_slots, C->d_slot_of, C->d_items, C->d_fold, C->d_zb, C->d_mzb, C->d_tc_tiles, C->d_tc_ft,
                     C->d_eta, C->d_jac, C->d_err,
                     C->d_x, C->d_r, C->d_z, C->d_p, C->d_q, C->d_b, C->d_t, C->d_partial, C->d_counter, C->d_s,
                     C->d_out2};
@@ -421,7 +421,7 @@ fcm_status fcm_info(const fcm_ctx *C, fcm_info_t *out)
         const bool tc = pl.n_tc_tiles > 0;
         const int own = (fcm::schwarz_uses_rows_kernel(C->p) ? pl.n_row_items : pl.n_col_items) > 0;
         out->s_apply_launches = C->have_precond ? (tc ? 1 : 0) + ((tc ? pl.n_tiles32_plain : pl.n_tiles32) > 0) +
-                                                      (pl.n_tiles64 > 0) + own + 1
+                                                      (pl.n_tiles64 > 0) + (pl.n_fold32 > 0) + (pl.n_fold_ff > 0) + own + 1
                                                 : 0;
         const int k = (C->kc.n_uncut > 0) + (C->kc.n_cut > 0) + 1;  // uncut cells, cut cells, sum
         out->k_apply_launches = k;

@@ -92,6 +92,13 @@ struct TcTile {
     int nch, pad;
 };
 
+// A block with a folded factor of its own: factor offset (floats), lattice DOF at the low corner of its box,
+// slot, nodes of the box per axis.
+struct FoldItem {
+    int64_t off, base;
+    int slot, d[3];
+};
+
 struct SchwarzPlan {
     Grid3 g;
     int rule;                 // 0 vertex patches, 3 element blocks (FCM_BLOCKS_*)
@@ -103,6 +110,8 @@ struct SchwarzPlan {
     int n_row_items, rows;
     const int2 *col_items;
     int n_col_items;
+    const FoldItem *fold_items;  // n_fold32 blocks with FP32 factors, then n_fold_ff with double-float ones
+    int n_fold32, n_fold_ff;
     const int2 *tiles;        // n_tiles32 FP32 tiles, then n_tiles64 FP64 tiles
     int n_tiles32, n_tiles64;
     int n_tiles32_plain;      // FP32 tiles of the factors without tensor-core tiles (listed first)
@@ -158,6 +167,11 @@ bool schwarz_tc_supported(int p);
 int64_t schwarz_tc_factor_floats(int p, int n);
 cudaError_t schwarz_tc_factor(int p, const double *F, int n, float *ft, cudaStream_t s);
 int schwarz_rows_threads();
+// whether own FP32 and double-float factors are stored folded; floats of one (prec 1 or 2), and the kernel
+// that folds an FP64 factor (rows padded to factor_ld<double>(n))
+bool schwarz_folds(int p);
+int64_t schwarz_fold_floats(int n, int prec);
+cudaError_t schwarz_fold_factor(const double *F, int n, int prec, float *out, cudaStream_t s);
 // kernel attributes (dynamic shared memory); host call, outside stream capture
 cudaError_t schwarz_prepare(int p);
 // polls of a bulk-copy wait before it gives up (default)
@@ -250,6 +264,7 @@ struct fcm_ctx {
     fcm::PatchRec *d_slots = nullptr;
     int *d_slot_of = nullptr;
     int2 *d_items = nullptr;         // row items, column items, GEMM tiles
+    fcm::FoldItem *d_fold = nullptr; // blocks with folded factors
     fcm::TcTile *d_tc_tiles = nullptr;
     float *d_tc_ft = nullptr;        // tensor-core factor tiles
     double *d_zb = nullptr;          // block products of one S apply

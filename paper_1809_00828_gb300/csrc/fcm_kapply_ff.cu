@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
         return;
     }
     float S[1] = {0.f}, C[1] = {0.f};
-    fold_dot<NE, 1>(m, NE, t & ~31, min(t, NE - 1), xe, 1, S, C);
+    fold_dot<NE, 1>(m, NE, t & ~31, min(t, NE - 1), xe, S, C);
     if (t < NE) zk[t * nc + ce.cell] = ff_norm(S[0], C[0]);
 }
 

@@ -530,10 +530,18 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
     std::vector<int> prec(fac.size(), 0);
     std::vector<int64_t> off(fac.size(), 0);
     int64_t n64 = 0, n32 = 0, alg_bytes = 0;
+    // own FP32 and double-float factors of small blocks keep each symmetric pair of entries once
+    std::vector<char> folded(fac.size(), 0);
     for (size_t f = 0; f < fac.size(); ++f) {
         const int n = fac[f].n;
         if (mixed) prec[f] = fac[f].cond <= o.cond_fp64 ? 1 : (o.precision == FCM_PREC_MIXED && !shared[f] ? 2 : 0);
-        if (prec[f] == 1) {
+        folded[f] = schwarz_folds(p) && !shared[f] && prec[f] != 0;
+        if (folded[f]) {
+            n32 = (n32 + 3) / 4 * 4;
+            off[f] = n32;
+            n32 += schwarz_fold_floats(n, prec[f]);
+            alg_bytes += (int64_t)n * (n + 1) / 2 * (prec[f] == 2 ? 8 : 4);
+        } else if (prec[f] == 1) {
             n32 = (n32 + 3) / 4 * 4;
             off[f] = n32;
             n32 += (int64_t)n * factor_ld<float>(n);
@@ -564,7 +572,9 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
         for (size_t f = 0; f < fac.size(); ++f) {
             const int64_t sz = (int64_t)fac[f].n * factor_ld<double>(fac[f].n);
             const int grid = (int)std::min<int64_t>((sz + 255) / 256, 1024);
-            if (prec[f] == 1)
+            if (folded[f])
+                PC_CUDA(schwarz_fold_factor(stage + fac[f].off, fac[f].n, prec[f], C->d_f32 + off[f], st));
+            else if (prec[f] == 1)
                 to_f32_kernel<<<grid, 256, 0, st>>>(stage + fac[f].off, C->d_f32 + off[f], fac[f].n);
             else if (prec[f] == 2)
                 to_ff_kernel<<<grid, 256, 0, st>>>(stage + fac[f].off, C->d_f32 + off[f], fac[f].n);
@@ -626,14 +636,31 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
             if (ft_off[f] >= 0) PC_CUDA(schwarz_tc_factor(p, stage + fac[f].off, fac[f].n, C->d_tc_ft + ft_off[f], st));
         PC_CUDA(cudaStreamSynchronize(st));
     }
-    std::vector<int> own_slots[3];  // by storage
+    std::vector<int> own_slots[3];  // by storage, without the folded factors
+    std::vector<FoldItem> fold_items[3];
     for (size_t f = 0; f < fac.size(); ++f) {
         if (shared[f]) continue;
         for (int v : blocks_of[f]) {
             slot_of[v] = (int)slots.size();
-            own_slots[prec[f]].push_back((int)slots.size());
+            if (folded[f]) {
+                const BoxInfo bx = block_box_of(rule, p, g, v);
+                fold_items[prec[f]].push_back({off[f], 3 * (bx.lo[0] + (int64_t)g.M[0] * (bx.lo[1] + (int64_t)g.M[1] * bx.lo[2])),
+                                               (int)slots.size(), {bx.d[0], bx.d[1], bx.d[2]}});
+            } else {
+                own_slots[prec[f]].push_back((int)slots.size());
+            }
             slots.push_back({off[f], v, prec[f]});
         }
+    }
+    const int n_fold32 = (int)fold_items[1].size(), n_fold_ff = (int)fold_items[2].size();
+    if (C->d_fold) cudaFree(C->d_fold);
+    C->d_fold = nullptr;
+    if (n_fold32 + n_fold_ff > 0) {
+        fold_items[1].insert(fold_items[1].end(), fold_items[2].begin(), fold_items[2].end());
+        PC_CUDA(cudaMalloc(&C->d_fold, sizeof(FoldItem) * fold_items[1].size()));
+        PC_CUDA(cudaMemcpyAsync(C->d_fold, fold_items[1].data(), sizeof(FoldItem) * fold_items[1].size(),
+                                cudaMemcpyHostToDevice, st));
+        PC_CUDA(cudaStreamSynchronize(st));
     }
     C->n_blocks = 0;
     C->sapply_fmas = 0;
@@ -736,6 +763,9 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
     plan.row_items = C->d_items;
     plan.col_items = d_col;
     plan.n_col_items = (int)col_items.size();
+    plan.fold_items = C->d_fold;
+    plan.n_fold32 = n_fold32;
+    plan.n_fold_ff = n_fold_ff;
     plan.tiles = d_tiles;
     plan.n_tiles32 = (int)tiles32.size();
     plan.n_tiles64 = (int)tiles64.size();
@@ -832,7 +862,7 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
     for (size_t f = 0; f < fac.size(); ++f) C->n_ff_factors += prec[f] == 2;
     C->n_gemm_blocks = gemm_blocks;
     C->n_factors = (int64_t)fac.size();
-    C->factor_bytes = alg_bytes;  // n^2 entries per factor (the stored rows carry < 16 bytes of padding)
+    C->factor_bytes = alg_bytes;  // n^2 entries per factor, n (n + 1) / 2 where folded (padding not counted)
     C->max_block = maxn;
     C->n_fp32_factors = 0;
     C->max_cond = 0.0;

@@ -5,10 +5,10 @@
 // Two phases, so that no block waits for another:
 //   1. block products Zb[B] = F_B r_B for every block at once, each written to its own slot of a
 //      buffer (no scatter, no colours):
-//        - blocks with their own factor (cut blocks) stream the factor from HBM once; a work item is
-//          a tile of rows of one block (schwarz_rows_kernel: a warp per row, the lanes split the row
-//          into 16-byte vectors; schwarz_cols_kernel: a thread per row, for small blocks and for
-//          several right-hand sides);
+//        - blocks with their own factor (cut blocks) stream the factor from HBM once: FP32 and double-float
+//          factors of p <= 2 folded, the symmetric pairs of entries once (schwarz_fold_kernel); else a work
+//          item is a tile of rows of one block (schwarz_rows_kernel: a warp per row, the lanes split the
+//          row into 16-byte vectors; schwarz_cols_kernel: a thread per row);
 //        - blocks that share a factor (uncut patches with equal boundary patterns) form a dense
 //          product F [r_B1 ... r_Bm]: schwarz_gemm_kernel stages the factor through shared memory
 //          by bulk copies (cp.async.bulk, completed on mbarriers, double-buffered) and keeps an
@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "fcm_device.cuh"
 #include "fcm_ff.cuh"
@@ -323,8 +324,7 @@ __device__ __forceinline__ void cols_ff(const double *__restrict__ r, int64_t nl
     for (int j = 0; j < n; ++j) {
         const float2 f = __ldcs(col + (size_t)j * ld);
 #pragma unroll
-        for (int k = 0; k < NR; ++k)
-            if (k < nr) ff_fma(f.x, f.y, rbT[j][k].x, rbT[j][k].y, S[k], C[k]);
+        for (int k = 0; k < NR; ++k) ff_fma(f.x, f.y, rbT[j][k].x, rbT[j][k].y, S[k], C[k]);
     }
 #pragma unroll
     for (int k = 0; k < NR; ++k)
@@ -347,6 +347,101 @@ __global__ void __launch_bounds__(cols_threads(P))
     if (pr.prec == 1) cols_plain<P, NR, float>(r, nlat, nr, f32 + pr.off, b, g, it.y, zout, zsize, pairs, smem);
     else if (pr.prec == 2) cols_ff<P, NR>(r, nlat, nr, f32 + pr.off, b, g, it.y, zout, zsize, pairs, smem);
     else cols_plain<P, NR, double>(r, nlat, nr, f64 + pr.off, b, g, it.y, zout, zsize, pairs, smem);
+}
+
+// ---- phase 1b': own FP32 and double-float factors of small blocks (p <= 2), folded (fcm_sym.cuh)
+//
+// Half of a symmetric factor's bytes, which bound the apply: a CTA per block, a thread per row, the columns in
+// ascending order as in schwarz_cols_kernel (an FP32 row's additions are the same, bit for bit).  At 80^3
+// p = 2 (107,741 FP32 and 37,771 double-float blocks, 1.43 + 1.00 GB): 246 + 211 us, the full factors 752 us.
+
+__host__ __device__ constexpr int fold_threads(int P) { return rnd32(sbox_max(P)); }
+
+template <int P, int NR, class T>
+__global__ void __launch_bounds__(fold_threads(P))
+    schwarz_fold_kernel(const double *__restrict__ r, int64_t nlat, int nr, const float *__restrict__ f32,
+                        const FoldItem *__restrict__ items, Grid3 g, double *__restrict__ zb, int zs, int64_t zsize,
+                        int pairs, int *err, int wait_tries, const int *__restrict__ done)
+{
+    constexpr int NM = sbox_max(P);
+    if (done && *done) return;
+    __shared__ __align__(16) T m[fold_entries(NM)], xs[(NM + 3) / 4 * 4 * NR];
+    __shared__ uint64_t bar;
+    const FoldItem it = items[blockIdx.x];
+    const int n = 3 * it.d[0] * it.d[1] * it.d[2], bytes = fold_entries(n) * (int)sizeof(T);
+    if (threadIdx.x == 0) {
+        mbar_init(&bar);
+        mbar_expect(&bar, bytes);
+        bulk_g2s(m, f32 + it.off, bytes, &bar);
+    }
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+        const int l = t / 3;
+        int ix, iy, iz;
+        if (n == NM) {  // the box of an inner block: constant divisors
+            constexpr int W = sbox_width(P);
+            ix = l % W;
+            iy = (l / W) % W;
+            iz = l / (W * W);
+        } else {
+            ix = l % it.d[0];
+            iy = (l / it.d[0]) % it.d[1];
+            iz = l / (it.d[0] * it.d[1]);
+        }
+        const double *rt = r + it.base + 3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            const double v = k < nr ? __ldg(rt + k * nlat) : 0.0;
+            if constexpr (sizeof(T) == 4) xs[t * NR + k] = to_f32(v);
+            else xs[t * NR + k] = split_ff(v);
+        }
+    }
+    __syncthreads();
+    if (!mbar_wait(&bar, 0, wait_tries)) {
+        atomicExch(err, 1);
+        mbar_wait(&bar, 0, kDrainTries);
+        return;
+    }
+    const int t0 = threadIdx.x & ~31;
+    if (t0 >= n) return;
+    const int row = threadIdx.x, t = min(row, n - 1);
+    double *zout = zb + (size_t)it.slot * zs;
+    if constexpr (sizeof(T) == 4) {
+        float acc[NR];
+#pragma unroll
+        for (int k = 0; k < NR; ++k) acc[k] = 0.f;
+        if (n == NM) fold_dot<NM, NR>(m, NM, t0, t, xs, acc);
+        else fold_dot<0, NR>(m, n, t0, t, xs, acc);
+#pragma unroll
+        for (int k = 0; k < NR; ++k)
+            if (k < nr && row < n) put_f32(zout + k * zsize, row, acc[k], pairs);
+    } else {
+        float S[NR], C[NR];
+#pragma unroll
+        for (int k = 0; k < NR; ++k) S[k] = C[k] = 0.f;
+        if (n == NM) fold_dot<NM, NR>(m, NM, t0, t, xs, S, C);
+        else fold_dot<0, NR>(m, n, t0, t, xs, S, C);
+#pragma unroll
+        for (int k = 0; k < NR; ++k)
+            if (k < nr && row < n) put_ff(zout + k * zsize, row, S[k], C[k], pairs);
+    }
+}
+
+// folded copy of an FP64 factor (rows padded to factor_ld<double>): FP32, or float pairs
+template <class T>
+__global__ void fold_factor_kernel(const double *__restrict__ in, T *__restrict__ out, int n)
+{
+    const int ld = factor_ld<double>(n), hw = fold_h(n) * fold_w(n);
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < fold_entries(n); e += gridDim.x * blockDim.x) {
+        int i, j;
+        double v = 0.0;
+        if (e < hw && fold_entry(n, e, i, j)) v = in[(size_t)i * ld + j];
+        if constexpr (sizeof(T) == 4) {
+            out[e] = (float)v;
+        } else {
+            const float h = __double2float_rn(v);
+            out[e] = make_float2(h, __double2float_rn(v - (double)h));
+        }
+    }
 }
 
 // ---- phase 1c: blocks sharing a factor, Zb[B_1 .. B_m] = F [r_B1 .. r_Bm] (m = count of the tile)
@@ -953,6 +1048,19 @@ void gemm_launch(const double *r, int64_t nlat, int nr, const double *f64, const
             pl.wait_tries, done);
 }
 
+// Calls f with the smallest instantiated number of columns (1, 2, 4, 6, 8) that holds nr right-hand sides.
+// The kernels form every column of their instantiation: a test per column and step (8 columns for any nr) kept
+// the double-float chains of a thread from overlapping (six right-hand sides, 24^3 p = 3: 5.57 -> 3.66 ms).
+template <class F>
+void with_columns(int nr, F &&f)
+{
+    if (nr <= 1) f(std::integral_constant<int, 1>());
+    else if (nr <= 2) f(std::integral_constant<int, 2>());
+    else if (nr <= 4) f(std::integral_constant<int, 4>());
+    else if (nr <= 6) f(std::integral_constant<int, 6>());
+    else f(std::integral_constant<int, 8>());
+}
+
 template <int P, int NR>
 void cols_launch(const double *r, int64_t nlat, int nr, const double *f64, const float *f32, const SchwarzPlan &pl,
                  double *zb, int64_t zsize, const int *done, cudaStream_t s)
@@ -962,6 +1070,19 @@ void cols_launch(const double *r, int64_t nlat, int nr, const double *f64, const
         r, nlat, nr, f64, f32, pl.slots, pl.col_items, pl.g, pl.rule, zb, pl.zs, zsize, pl.pairs, done);
 }
 
+template <int P, int NR>
+void fold_launch(const double *r, int64_t nlat, int nr, const float *f32, const SchwarzPlan &pl, double *zb,
+                 int64_t zsize, const int *done, cudaStream_t s)
+{
+    if (pl.n_fold32 > 0)
+        schwarz_fold_kernel<P, NR, float><<<pl.n_fold32, fold_threads(P), 0, s>>>(
+            r, nlat, nr, f32, pl.fold_items, pl.g, zb, pl.zs, zsize, pl.pairs, pl.err, pl.wait_tries, done);
+    if (pl.n_fold_ff > 0)
+        schwarz_fold_kernel<P, NR, float2><<<pl.n_fold_ff, fold_threads(P), 0, s>>>(
+            r, nlat, nr, f32, pl.fold_items + pl.n_fold32, pl.g, zb, pl.zs, zsize, pl.pairs, pl.err, pl.wait_tries,
+            done);
+}
+
 template <int P>
 void apply_p(const double *r, double *z, int64_t nlat, int nr, const double *f64, const float *f32,
              const SchwarzPlan &pl, double *zb, const int *done, cudaStream_t s)
@@ -969,7 +1090,7 @@ void apply_p(const double *r, double *z, int64_t nlat, int nr, const double *f64
     const int64_t zsize = (int64_t)pl.nslots * pl.zs;
     const bool gemm = pl.n_tiles32 + pl.n_tiles64 + (nr == 1 ? pl.n_tc_tiles : 0) > 0;
     const bool own = nr == 1 && P == 3 ? pl.n_row_items > 0 : pl.n_col_items > 0;
-    const bool side = pl.concurrent && gemm && own && pl.side;
+    const bool side = pl.concurrent && gemm && (own || pl.n_fold32 + pl.n_fold_ff > 0) && pl.side;
     if (side) {
         // the shared-factor products on the second stream, beside the streamed factors
         cudaEventRecord(pl.ev_fork, s);
@@ -979,17 +1100,18 @@ void apply_p(const double *r, double *z, int64_t nlat, int nr, const double *f64
     } else if (gemm) {
         gemm_launch<P>(r, nlat, nr, f64, f32, pl, zb, zsize, done, s);
     }
+    if constexpr (P <= 2)
+        with_columns(nr, [&](auto c) { fold_launch<P, decltype(c)::value>(r, nlat, nr, f32, pl, zb, zsize, done, s); });
     if (own) {
-        if constexpr (P == 3) {
-            if (nr == 1)
+        if (P == 3 && nr == 1) {
+            if constexpr (P == 3)
                 schwarz_rows_kernel<P><<<pl.n_row_items, kRowsThreads, 0, s>>>(
                     r, f64, f32, pl.slots, pl.row_items, pl.rows, pl.g, pl.rule, zb, pl.zs, pl.pairs, done);
-            else
-                cols_launch<P, 8>(r, nlat, nr, f64, f32, pl, zb, zsize, done, s);
-        } else if (nr == 1)
-            cols_launch<P, 1>(r, nlat, nr, f64, f32, pl, zb, zsize, done, s);
-        else
-            cols_launch<P, 8>(r, nlat, nr, f64, f32, pl, zb, zsize, done, s);
+        } else {
+            with_columns(nr, [&](auto c) {
+                cols_launch<P, decltype(c)::value>(r, nlat, nr, f64, f32, pl, zb, zsize, done, s);
+            });
+        }
     }
     if (side) cudaStreamWaitEvent(s, pl.ev_join, 0);
     if (pl.pairs)
@@ -1011,12 +1133,12 @@ cudaError_t prepare_p()
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(schwarz_gemm_kernel<P, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  gemm_smem_bytes<P, double>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(schwarz_cols_kernel<P, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 factor_ld<double>(sbox_max(P)) * 8 * 8);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(schwarz_cols_kernel<P, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 factor_ld<double>(sbox_max(P)) * 8);
+    for (int nr = 1; nr <= 8 && e == cudaSuccess; ++nr)
+        with_columns(nr, [&](auto c) {
+            constexpr int NR = decltype(c)::value;
+            e = cudaFuncSetAttribute(schwarz_cols_kernel<P, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     factor_ld<double>(sbox_max(P)) * NR * 8);
+        });
     return e;
 }
 
@@ -1065,6 +1187,18 @@ cudaError_t schwarz_tc_factor(int p, const double *F, int n, float *ft, cudaStre
     if (p == 3) tc_factor_kernel<3><<<grid, 256, 0, s>>>(F, n, ft);
     else if (p == 2) tc_factor_kernel<2><<<grid, 256, 0, s>>>(F, n, ft);
     else return cudaErrorInvalidValue;
+    return cudaGetLastError();
+}
+
+bool schwarz_folds(int p) { return p <= 2; }
+
+int64_t schwarz_fold_floats(int n, int prec) { return (int64_t)fold_entries(n) * (prec == 2 ? 2 : 1); }
+
+cudaError_t schwarz_fold_factor(const double *F, int n, int prec, float *out, cudaStream_t s)
+{
+    const int grid = (fold_entries(n) + 255) / 256;
+    if (prec == 2) fold_factor_kernel<float2><<<grid, 256, 0, s>>>(F, reinterpret_cast<float2 *>(out), n);
+    else fold_factor_kernel<float><<<grid, 256, 0, s>>>(F, out, n);
     return cudaGetLastError();
 }
 

@@ -144,9 +144,9 @@ __device__ __forceinline__ void fold_dot(const float *m, int n, int t0, int t, c
         });
 }
 
-// the same for a double-float F; nr <= NR of the right-hand sides are formed
+// the same for a double-float F
 template <int N, int NR>
-__device__ __forceinline__ void fold_dot(const float2 *m, int n, int t0, int t, const float2 *xs, int nr, float (&S)[NR],
+__device__ __forceinline__ void fold_dot(const float2 *m, int n, int t0, int t, const float2 *xs, float (&S)[NR],
                                          float (&C)[NR])
 {
     float2 xv[NR == 1 ? 4 : 1];
@@ -169,11 +169,10 @@ __device__ __forceinline__ void fold_dot(const float2 *m, int n, int t0, int t, 
                 ff_fma(f.x, f.y, xv[k].x, xv[k].y, S[0], C[0]);
             } else {
 #pragma unroll
-                for (int r = 0; r < NR; ++r)
-                    if (r < nr) {
-                        const float2 v = xj[k * NR + r];
-                        ff_fma(f.x, f.y, v.x, v.y, S[r], C[r]);
-                    }
+                for (int r = 0; r < NR; ++r) {
+                    const float2 v = xj[k * NR + r];
+                    ff_fma(f.x, f.y, v.x, v.y, S[r], C[r]);
+                }
             }
         });
 }
