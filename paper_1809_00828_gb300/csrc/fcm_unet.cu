@@ -9,137 +9,363 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
+#include <cstring>
 #include <string>
 #include <vector>
 
 #include "fcm_device.cuh"
+#include "fcm_tma.cuh"
 
 namespace fcm {
 namespace {
 
-constexpr int kConvThreads = 128;
-constexpr int kCiChunk = 16;
+// ---- 3x3x3 convolution on the tensor cores
+//
+// out[b][co][p] = bias[co] + sum_{ci, tap} w[co][ci][tap] in[b][ci][p + off(tap)], zero padding, as a product
+// D[voxel][co] += A[voxel][ci] B[co][ci] per tap (tcgen05 kind::f16, BF16 operands, FP32 accumulators in tensor
+// memory).  The weights are BF16; an FP32 activation is the exact sum of three BF16 values (8 significant bits
+// each, cut from the top), so three products give what FP32 multiplications of the same weights give.
+//
+// A CTA makes 8 x 16 x ZT voxels (x, y, z) of up to 64 output channels.  Per 16 input channels it writes the
+// tile with its halo of one voxel to shared memory, [split][8 channels][z][y][x] with 16 bytes per voxel:
+// eight voxels along x are a core matrix of the canonical K-major layout without swizzle and a row of them a
+// fixed stride, so each of the 27 taps is the same tile at another start address, and no input is gathered
+// twice.  Forward pass on 80^3 cells, channels 16 to 64 (75 GFLOP of convolutions): 1.19 ms, 5.76 ms with FP32
+// arithmetic on the CUDA cores (13 TFLOP/s); bound by the rate at which one thread issues products, 81 per 128
+// voxels and 16 input channels.  Two CTAs per SM overlap one's halo loads with the other's products.
+//
+// The tensor core adds into its FP32 accumulators by truncation: with one accumulator over all 81 products of
+// 16 input channels the outputs were 5.6e-6 off (relative, 2-norm), 10 times the FP32 multiply-adds' error.  So
+// the leading parts of each plane of taps (dz) have an accumulator of their own, the two small parts share a
+// fourth, and after every 16 channels the four are added in registers with rounding to nearest.  That is also
+// four independent chains of products instead of one.
+//
+// Around it, the loader reads the decoder's concatenation from its two sources (upsampled and skip), the
+// gradient through a ReLU from the gradient and the ReLU's output, and the epilogue adds the bias and applies
+// the ReLU: no pass over an activation is left between two convolutions but the pooling.
+constexpr int kConvThreads = 256;
+constexpr int kTX = 8, kTY = 16, kHX = kTX + 2, kHY = kTY + 2;
+constexpr int kCoMax = 64;   // output channels of a CTA
 
-// out[b][co][p] = bias[co] + sum_{ci, tap} w[co][ci][tap] in[b][ci][p + off(tap)], zero padding.
-// One thread per output voxel and COB output channels; a chunk of weights is staged in shared memory.
-template <int COB>
-__global__ void __launch_bounds__(kConvThreads)
-    conv3_fwd_kernel(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ bias,
-                     float *__restrict__ out, int Cin, int Cout, int nx, int ny, int nz)
+__host__ __device__ constexpr int conv_hv(int ZT) { return kHX * kHY * (ZT + 2); }        // voxels with halo
+__host__ __device__ constexpr int conv_a_bytes(int ZT) { return 3 * 2 * 16 * conv_hv(ZT); }
+__host__ __device__ constexpr int conv_smem(int ZT, int nb) { return 1024 + conv_a_bytes(ZT) + 27 * 32 * nb; }
+__host__ __device__ constexpr int up16(int n) { return (n + 15) / 16 * 16; }
+// columns (output channels) of a CTA, CTAs per voxel tile, and BF16 entries of a layer's weight tiles
+__host__ __device__ constexpr int conv_nb(int n) { return n <= kCoMax ? up16(n) : kCoMax; }
+__host__ __device__ constexpr int conv_blocks(int n) { return (n + kCoMax - 1) / kCoMax; }
+__host__ __device__ constexpr int64_t conv_tile_entries(int cin, int cout)
 {
-    __shared__ float ws[COB][kCiChunk][27];
-    const int S = nx * ny * nz;
-    const int b = blockIdx.z;
-    const int co0 = blockIdx.y * COB;
-    const int p = blockIdx.x * kConvThreads + threadIdx.x;
-    const int x = p % nx, y = (p / nx) % ny, z = p / (nx * ny);
-    float acc[COB];
+    return (int64_t)conv_blocks(cout) * (up16(cin) / 16) * 27 * 16 * conv_nb(cout);
+}
+
+// Source of a convolution or of its weight gradient: channels 0 .. c0 - 1 at half resolution (nearest
+// upsampling), then those of `full`, set to 0 where the same entry of `gate` is not positive (gate may be null).
+struct ConvSrc {
+    const float *half, *full, *gate;
+    int c0, c1;
+};
+
+__device__ __forceinline__ float conv_load(const ConvSrc &s, int b, int ci, int x, int y, int z, int nx, int ny, int nz)
+{
+    if (ci < s.c0) {
+        const int hx = nx >> 1, hy = ny >> 1, hz = nz >> 1;
+        return __ldg(s.half + (((int64_t)b * s.c0 + ci) * hz + (z >> 1)) * hy * hx + (y >> 1) * hx + (x >> 1));
+    }
+    const int64_t at = (((int64_t)b * s.c1 + ci - s.c0) * nz + z) * ny * nx + (int64_t)y * nx + x;
+    const float v = __ldg(s.full + at);
+    return s.gate && !(__ldg(s.gate + at) > 0.f) ? 0.f : v;
+}
+
+// x = hi + mid + lo, each with 8 significant bits in its upper half word; infinities and NaN in hi alone
+__device__ __forceinline__ void split3(float x, uint32_t &hi, uint32_t &mid, uint32_t &lo)
+{
+    const uint32_t u = __float_as_uint(x);
+    hi = u & 0xFFFF0000u;
+    const float r = __fsub_rn(x, __uint_as_float(hi));
+    mid = __float_as_uint(r) & 0xFFFF0000u;
+    lo = __float_as_uint(__fsub_rn(r, __uint_as_float(mid)));
+    if ((u & 0x7F800000u) == 0x7F800000u) {
+        if (u & 0x7FFFFFu) hi |= 0x00400000u;
+        mid = lo = 0u;
+    }
+}
+
+template <int ZT>
+__global__ void __launch_bounds__(kConvThreads)
+    conv3_tc_kernel(ConvSrc src, const uint4 *__restrict__ w, const float *__restrict__ bias, float *__restrict__ out,
+                    int cin, int cout, int nx, int ny, int nz, int relu, int *err)
+{
+    constexpr int HV = conv_hv(ZT);
+    extern __shared__ __align__(1024) unsigned char csm[];
+    uint64_t *bar = reinterpret_cast<uint64_t *>(csm);
+    uint32_t *slot = reinterpret_cast<uint32_t *>(csm + 8);
+    unsigned char *A = csm + 1024, *W = A + conv_a_bytes(ZT);
+    const int nb = conv_nb(cout), nch = up16(cin) / 16;
+    const int tx = (nx + kTX - 1) / kTX, ty = (ny + kTY - 1) / kTY;
+    const int x0 = (blockIdx.x % tx) * kTX, y0 = (blockIdx.x / tx % ty) * kTY, z0 = (blockIdx.x / (tx * ty)) * ZT;
+    const int b = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t S = (int64_t)nx * ny * nz, S2 = (int64_t)(nx >> 1) * (ny >> 1) * (nz >> 1);
+    const uint32_t cols = 4 * ZT * nb <= 64 ? 64 : 4 * ZT * nb <= 128 ? 128 : 256;
+    if (tid == 0) mbar_init(bar);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *slot;
+    // warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (rows y of four, 8 voxels along x each) of the items
+    // (z, 16 channels) w / 4, w / 4 + 2
+    const int items = ZT * (nb / 16);
+    float sum[2][16];
 #pragma unroll
-    for (int k = 0; k < COB; ++k) acc[k] = (bias && co0 + k < Cout) ? bias[co0 + k] : 0.f;
-    const float *inb = in + (size_t)b * Cin * S;
-    for (int ci0 = 0; ci0 < Cin; ci0 += kCiChunk) {
-        const int nci = min(kCiChunk, Cin - ci0);
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int k = 0; k < 16; ++k) sum[i][k] = 0.f;
+    for (int ch = 0; ch < nch; ++ch) {
+        for (int e = tid; e < 2 * HV; e += kConvThreads) {
+            const int kc = e >= HV, v = e - kc * HV, hx = v % kHX, hy = v / kHX % kHY, hz = v / (kHX * kHY);
+            const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
+            const bool in = x >= 0 && y >= 0 && z >= 0 && x < nx && y < ny && z < nz;
+            const int ci = 16 * ch + 8 * kc;
+            float f[8];
+            if (in && ci >= src.c0 && ci + 8 <= cin) {
+                const int64_t at = ((int64_t)b * src.c1 + ci - src.c0) * S + ((int64_t)z * ny + y) * nx + x;
+                const float *p = src.full + at;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) f[k] = __ldg(p + k * S);
+                if (src.gate) {
+                    const float *q = src.gate + at;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        if (!(__ldg(q + k * S) > 0.f)) f[k] = 0.f;
+                }
+            } else if (in && ci + 8 <= src.c0) {
+                const float *p = src.half + ((int64_t)b * src.c0 + ci) * S2 + ((int64_t)(z >> 1) * (ny >> 1) + (y >> 1)) * (nx >> 1) + (x >> 1);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) f[k] = __ldg(p + k * S2);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) f[k] = in && ci + k < cin ? conv_load(src, b, ci + k, x, y, z, nx, ny, nz) : 0.f;
+            }
+            uint32_t s[3][8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) split3(f[k], s[0][k], s[1][k], s[2][k]);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                uint4 o;  // the upper half words, channel k at bytes 2 k
+                o.x = __byte_perm(s[q][0], s[q][1], 0x7632);
+                o.y = __byte_perm(s[q][2], s[q][3], 0x7632);
+                o.z = __byte_perm(s[q][4], s[q][5], 0x7632);
+                o.w = __byte_perm(s[q][6], s[q][7], 0x7632);
+                reinterpret_cast<uint4 *>(A)[(2 * q + kc) * HV + v] = o;
+            }
+        }
+        const uint4 *wc = w + ((int64_t)blockIdx.y * nch + ch) * 27 * 2 * nb;
+        for (int e = tid; e < 27 * 2 * nb; e += kConvThreads) reinterpret_cast<uint4 *>(W)[e] = __ldg(wc + e);
+        // the tensor core reads shared memory through the async proxy
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        for (int e = threadIdx.x; e < COB * kCiChunk * 27; e += kConvThreads) {
-            const int k = e / (kCiChunk * 27), r = e % (kCiChunk * 27), ci = r / 27, t = r % 27;
-            ws[k][ci][t] = (co0 + k < Cout && ci < nci) ? __bfloat162float(w[((size_t)(co0 + k) * Cin + ci0 + ci) * 27 + t]) : 0.f;
+        if (tid == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            // FP32 accumulator, BF16 A and B, both K-major, M = 128, N = nb
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nb >> 3) << 17) | (8u << 24);
+            const uint32_t a0 = smem_u32(A), w0 = smem_u32(W);
+            const int zn = min(ZT, nz - z0);
+            // accumulator 4 z + dz: the leading parts of the taps of plane dz; 4 z + 3: the small parts
+            for (int t = 0; t < 9; ++t)
+                for (int dz = 0; dz < 3; ++dz) {
+                    const uint64_t bd = smem_desc(w0 + (9 * dz + t) * 32 * nb, 128, 256);
+                    const int at = dz * kHX * kHY + t / 3 * kHX + t % 3;
+                    for (int z = 0; z < zn; ++z) {
+                        const uint32_t a = a0 + 16 * (at + z * kHX * kHY), d = tmem + 4 * z * nb;
+                        tc_mma_bf16(d + dz * nb, smem_desc(a, 16 * HV, 16 * kHX), bd, idesc, t > 0);
+                        tc_mma_bf16(d + 3 * nb, smem_desc(a + 64 * HV, 16 * HV, 16 * kHX), bd, idesc, t > 0 || dz > 0);
+                        tc_mma_bf16(d + 3 * nb, smem_desc(a + 32 * HV, 16 * HV, 16 * kHX), bd, idesc, 1);
+                    }
+                }
+            tc_commit(bar);
+        }
+        if (!mbar_wait(bar, ch & 1, kWaitTries)) {
+            atomicExch(err, 1);  // the products still in flight land before shared memory is written again
+            mbar_wait(bar, ch & 1, kDrainTries);
+        }
+        __syncwarp();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int it = (warp >> 2) + 2 * i;
+            if (it >= items) break;  // uniform across the warp
+            const uint32_t at = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 4 * (it / (nb / 16)) * nb + it % (nb / 16) * 16;
+            float part[16];
+#pragma unroll
+            for (int q = 3; q >= 0; --q) {
+                uint32_t v[16];
+                tc_load16(at + q * nb, v);
+#pragma unroll
+                for (int k = 0; k < 16; ++k)
+                    part[k] = q == 3 ? __uint_as_float(v[k]) : __fadd_rn(part[k], __uint_as_float(v[k]));
+            }
+#pragma unroll
+            for (int k = 0; k < 16; ++k) sum[i][k] = __fadd_rn(sum[i][k], part[k]);
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    }
+    const int vx = x0 + (lane & 7), vy = y0 + 4 * (warp & 3) + (lane >> 3);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int it = (warp >> 2) + 2 * i, vz = z0 + it / (nb / 16);
+        if (it >= items || vx >= nx || vy >= ny || vz >= nz) continue;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int co = blockIdx.y * kCoMax + it % (nb / 16) * 16 + k;
+            if (co < cout) {
+                float f = sum[i][k];
+                if (bias) f = __fadd_rn(f, bias[co]);
+                if (relu) f = fmaxf(f, 0.f);
+                out[((int64_t)b * cout + co) * S + ((int64_t)vz * ny + vy) * nx + vx] = f;
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
+}
+
+// Weight tiles of one layer in the tensor core's layout, from the BF16 weights w[co][ci][27]: per block of 64
+// output channels, 16 input channels and tap, [channel / 8][K / 8][8 channels][8 K] (zeros beyond the layer).
+// flip: the tiles of the data-gradient convolution, w'[ci][co][26 - tap] (cin, cout: those of that convolution).
+__global__ void conv_tiles_kernel(const __nv_bfloat16 *__restrict__ w, __nv_bfloat16 *__restrict__ t, int cin, int cout,
+                                  int flip)
+{
+    const int nb = conv_nb(cout), nch = up16(cin) / 16;
+    const int64_t n = conv_tile_entries(cin, cout);
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const int k = (int)(e & 7), r = (int)(e >> 3 & 7), kc = (int)(e >> 6 & 1);
+        int64_t q = e >> 7;
+        const int n8 = (int)(q % (nb / 8));
+        q /= nb / 8;
+        const int tap = (int)(q % 27);
+        q /= 27;
+        const int ci = 16 * (int)(q % nch) + 8 * kc + k, co = kCoMax * (int)(q / nch) + 8 * n8 + r;
+        __nv_bfloat16 v = __float2bfloat16(0.f);
+        if (ci < cin && co < cout)
+            v = flip ? w[((int64_t)ci * cout + co) * 27 + 26 - tap] : w[((int64_t)co * cin + ci) * 27 + tap];
+        t[e] = v;
+    }
+}
+
+// ---- weight gradients: gw[co][ci][tap] += sum_{b,p} gout[b][co][p] in[b][ci][p + off(tap)], gb[co] += sum gout
+//
+// A CTA owns 16 output x 8 input channels and walks tiles of 8 x 8 x 4 voxels; a thread owns one (co, ci) pair
+// of half of the voxels with its 27 taps (and the bias) in registers, so four voxels along x cost 19 vector
+// reads of shared memory and 112 multiply-adds: bound by the FP32 pipe.  The tiles are dealt to enough CTAs to
+// fill the GPU, each writes its sums to `part`, and wgrad_sum_kernel adds them in a fixed order in FP64
+// (deterministic).  One CTA per (co, ci) pair with 27 unshared global reads per multiply-add row took 4.9 ms
+// for the gradients of the 16-to-64-channel network on four 32^3 cubes; this 1.08 + 0.29 ms.
+constexpr int kWC = 8, kWO = 16, kWX = 8, kWY = 8, kWZ = 4, kWPitch = 12, kWGo = kWX * kWY * kWZ + 4;
+constexpr int kWTaps = 28;
+constexpr int kSumParts = 16;  // parts of the slabs that wgrad_sum_kernel adds side by side
+
+__global__ void __launch_bounds__(256)
+    conv3_wgrad_kernel(ConvSrc in, ConvSrc go, int cin, int cout, int B, int nx, int ny, int nz, float *__restrict__ part)
+{
+    __shared__ __align__(16) float si[kWC][kWZ + 2][kWY + 2][kWPitch];
+    __shared__ __align__(16) float sg[kWO][kWGo];
+    const int ci0 = blockIdx.x * kWC, co0 = blockIdx.y * kWO, tid = threadIdx.x;
+    const int co = tid & 15, ci = tid >> 4 & 7, zh = tid >> 7;  // zh: z planes 2 zh, 2 zh + 1 of the tile
+    const int tx = (nx + kWX - 1) / kWX, ty = (ny + kWY - 1) / kWY, tz = (nz + kWZ - 1) / kWZ;
+    const int64_t tiles = (int64_t)B * tx * ty * tz;
+    float acc[kWTaps];
+#pragma unroll
+    for (int t = 0; t < kWTaps; ++t) acc[t] = 0.f;
+    for (int64_t tile = blockIdx.z; tile < tiles; tile += gridDim.z) {
+        const int b = (int)(tile / ((int64_t)tx * ty * tz)), q = (int)(tile % ((int64_t)tx * ty * tz));
+        const int x0 = q % tx * kWX, y0 = q / tx % ty * kWY, z0 = q / (tx * ty) * kWZ;
+        __syncthreads();
+        for (int e = tid; e < kWC * (kWZ + 2) * (kWY + 2) * (kWX + 2); e += 256) {
+            const int hx = e % (kWX + 2), hy = e / (kWX + 2) % (kWY + 2), hz = e / ((kWX + 2) * (kWY + 2)) % (kWZ + 2),
+                      c = e / ((kWX + 2) * (kWY + 2) * (kWZ + 2));
+            const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
+            const bool on = ci0 + c < cin && x >= 0 && y >= 0 && z >= 0 && x < nx && y < ny && z < nz;
+            si[c][hz][hy][hx] = on ? conv_load(in, b, ci0 + c, x, y, z, nx, ny, nz) : 0.f;
+        }
+        for (int e = tid; e < kWO * kWX * kWY * kWZ; e += 256) {
+            const int v = e % (kWX * kWY * kWZ), c = e / (kWX * kWY * kWZ);
+            const int x = x0 + v % kWX, y = y0 + v / kWX % kWY, z = z0 + v / (kWX * kWY);
+            const bool on = co0 + c < cout && x < nx && y < ny && z < nz;
+            sg[c][v] = on ? conv_load(go, b, co0 + c, x, y, z, nx, ny, nz) : 0.f;
         }
         __syncthreads();
-        if (p < S) {
-            for (int ci = 0; ci < nci; ++ci) {
-                const float *src = inb + (size_t)(ci0 + ci) * S;
-                for (int dz = -1; dz <= 1; ++dz) {
-                    const int zz = z + dz;
-                    if (zz < 0 || zz >= nz) continue;
-                    for (int dy = -1; dy <= 1; ++dy) {
-                        const int yy = y + dy;
-                        if (yy < 0 || yy >= ny) continue;
-                        for (int dx = -1; dx <= 1; ++dx) {
-                            const int xx = x + dx;
-                            if (xx < 0 || xx >= nx) continue;
-                            const float v = src[(zz * ny + yy) * nx + xx];
-                            const int t = (dz + 1) * 9 + (dy + 1) * 3 + (dx + 1);
+#pragma unroll 1
+        for (int zy = 0; zy < 2 * kWY; ++zy) {
+            const int z = 2 * zh + zy / kWY, y = zy % kWY;
 #pragma unroll
-                            for (int k = 0; k < COB; ++k) acc[k] = fmaf(ws[k][ci][t], v, acc[k]);
-                        }
-                    }
+            for (int xr = 0; xr < kWX; xr += 4) {
+                const float4 g4 = *reinterpret_cast<const float4 *>(&sg[co][(z * kWY + y) * kWX + xr]);
+                const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+                acc[27] += (g[0] + g[1]) + (g[2] + g[3]);
+#pragma unroll
+                for (int d = 0; d < 9; ++d) {
+                    const float *row = &si[ci][z + d / 3][y + d % 3][xr];
+                    const float4 a = *reinterpret_cast<const float4 *>(row);
+                    const float2 c = *reinterpret_cast<const float2 *>(row + 4);
+                    const float v[6] = {a.x, a.y, a.z, a.w, c.x, c.y};
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) acc[3 * d + dx] = fmaf(g[k], v[k + dx], acc[3 * d + dx]);
                 }
             }
         }
     }
-    if (p < S)
+    // the two halves of the voxels, then this CTA's sums: part[z][co][ci][tap]
+    __syncthreads();
+    float *red = &si[0][0][0][0];  // 128 x 28 floats
+    static_assert(128 * kWTaps <= kWC * (kWZ + 2) * (kWY + 2) * kWPitch, "reduction buffer");
+    if (zh == 1)
 #pragma unroll
-        for (int k = 0; k < COB; ++k)
-            if (co0 + k < Cout) out[((size_t)b * Cout + co0 + k) * S + p] = acc[k];
+        for (int t = 0; t < kWTaps; ++t) red[t * 128 + (tid & 127)] = acc[t];
+    __syncthreads();
+    if (zh == 0) {
+        float *p = part + ((((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * kWO + co) * (gridDim.x * kWC) + ci0 + ci) * kWTaps;
+#pragma unroll
+        for (int t = 0; t < kWTaps; ++t) p[t] = acc[t] + red[t * 128 + tid];
+    }
 }
 
-// gw[co][ci][tap] += sum_{b,p} gout[b][co][p] in[b][ci][p + off(tap)];  gb[co] += sum gout (ci == 0 block).
-// One block per (ci, co); fixed-order block reduction (deterministic).
-__global__ void __launch_bounds__(256)
-    conv3_wgrad_kernel(const float *__restrict__ in, const float *__restrict__ gout, int Cin, int Cout, int B, int nx,
-                       int ny, int nz, float *__restrict__ gw, float *__restrict__ gb)
+__global__ void __launch_bounds__(32 * kSumParts)
+    wgrad_sum_kernel(const float *__restrict__ part, int nslab, int cin, int cout, int cip, int cop, float *__restrict__ gw,
+                     float *__restrict__ gb)
 {
-    __shared__ float red[28][256];
-    const int ci = blockIdx.x, co = blockIdx.y;
-    const int S = nx * ny * nz;
-    float acc[28];
-#pragma unroll
-    for (int t = 0; t < 28; ++t) acc[t] = 0.f;
-    for (int b = 0; b < B; ++b) {
-        const float *src = in + ((size_t)b * Cin + ci) * S;
-        const float *go = gout + ((size_t)b * Cout + co) * S;
-        for (int p = threadIdx.x; p < S; p += blockDim.x) {
-            const float g = go[p];
-            const int x = p % nx, y = (p / nx) % ny, z = p / (nx * ny);
-            acc[27] += g;
-#pragma unroll
-            for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-                for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-                    for (int dx = -1; dx <= 1; ++dx) {
-                        const int zz = z + dz, yy = y + dy, xx = x + dx;
-                        const bool ok = zz >= 0 && zz < nz && yy >= 0 && yy < ny && xx >= 0 && xx < nx;
-                        const float v = ok ? src[(zz * ny + yy) * nx + xx] : 0.f;
-                        acc[(dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)] = fmaf(g, v, acc[(dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)]);
-                    }
+    const int64_t n = (int64_t)cout * cin * kWTaps, slab = (int64_t)cop * cip * kWTaps;
+    __shared__ double sh[kSumParts][32];
+    for (int64_t e0 = blockIdx.x * (int64_t)32; e0 < n; e0 += (int64_t)gridDim.x * 32) {
+        const int64_t e = e0 + threadIdx.x;
+        const int t = (int)(e % kWTaps), ci = (int)(e / kWTaps % cin), co = (int)(e / ((int64_t)kWTaps * cin));
+        const bool on = e < n && (t < 27 || ci == 0);
+        double s = 0.0;
+        if (on) {
+            const float *p = part + ((int64_t)co * cip + ci) * kWTaps + t;
+#pragma unroll 8
+            for (int k = threadIdx.y; k < nslab; k += kSumParts) s += p[k * slab];
         }
-    }
+        sh[threadIdx.y][threadIdx.x] = s;
+        __syncthreads();
+        if (threadIdx.y == 0 && on) {
 #pragma unroll
-    for (int t = 0; t < 28; ++t) red[t][threadIdx.x] = acc[t];
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int t = 0; t < 28; ++t) red[t][threadIdx.x] += red[t][threadIdx.x + o];
+            for (int q = 1; q < kSumParts; ++q) s += sh[q][threadIdx.x];
+            if (t < 27) gw[((int64_t)co * cin + ci) * 27 + t] += (float)s;
+            else gb[co] += (float)s;
+        }
         __syncthreads();
     }
-    if (threadIdx.x < 27) gw[((size_t)co * Cin + ci) * 27 + threadIdx.x] += red[threadIdx.x][0];
-    if (threadIdx.x == 27 && ci == 0) gb[co] += red[27][0];
-}
-
-// wt[ci][co][26 - t] = w[co][ci][t] (the weights of the data-gradient convolution)
-__global__ void transpose_flip_kernel(const __nv_bfloat16 *w, __nv_bfloat16 *wt, int Cin, int Cout)
-{
-    const int64_t n = (int64_t)Cin * Cout * 27;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int t = (int)(e % 27);
-        const int64_t r = e / 27;
-        const int ci = (int)(r % Cin), co = (int)(r / Cin);
-        wt[((int64_t)ci * Cout + co) * 27 + (26 - t)] = w[e];
-    }
-}
-
-__global__ void relu_fwd_kernel(const float *a, float *b, int64_t n)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        b[i] = fmaxf(a[i], 0.f);
-}
-
-__global__ void relu_bwd_kernel(const float *pre, const float *g, float *gpre, int64_t n)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        gpre[i] = pre[i] > 0.f ? g[i] : 0.f;
 }
 
 // coarse[bc][Z][Y][X] = mean of the 8 children (2x average pooling); bc = batch * channels
@@ -165,19 +391,6 @@ __global__ void pool_bwd_kernel(const float *gcoarse, float *gfine, int64_t bc, 
         const int x = (int)(e % nx), y = (int)((e / nx) % ny), z = (int)((e / ((int64_t)nx * ny)) % nz);
         const int64_t c = e / ((int64_t)nx * ny * nz);
         gfine[e] += 0.125f * gcoarse[((c * (nz / 2) + z / 2) * (ny / 2) + y / 2) * (nx / 2) + x / 2];
-    }
-}
-
-// dst[b][c0 + c][p] = nearest-upsampled src[b][c][p/2]  (src at half resolution, C channels)
-__global__ void up_fwd_kernel(const float *src, float *dst, int B, int C, int Cdst, int c0, int nx, int ny, int nz)
-{
-    const int64_t S = (int64_t)nx * ny * nz, n = (int64_t)B * C * S;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = e % S, bc = e / S;
-        const int c = (int)(bc % C), b = (int)(bc / C);
-        const int x = (int)(p % nx), y = (int)((p / nx) % ny), z = (int)(p / ((int64_t)nx * ny));
-        dst[((int64_t)b * Cdst + c0 + c) * S + p] =
-            src[(((int64_t)b * C + c) * (nz / 2) + z / 2) * (ny / 2) * (nx / 2) + (y / 2) * (nx / 2) + x / 2];
     }
 }
 
@@ -210,11 +423,6 @@ __global__ void chan_copy_kernel(const float *src, int Csrc, int cs0, float *dst
         float &d = dst[((int64_t)b * Cdst + c0 + c) * S + p];
         d = accumulate ? d + v : v;
     }
-}
-
-__global__ void fill_kernel(float *a, int64_t n, float v)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) a[i] = v;
 }
 
 __global__ void to_bf16_kernel(const float *a, __nv_bfloat16 *b, int64_t n)
@@ -250,25 +458,29 @@ using namespace fcm;
 struct UConv {
     int cin, cout;
     int64_t woff, boff;  // offsets in the parameter arrays
+    int64_t toff, doff;  // offsets of its weight tiles and of its data-gradient convolution's
 };
 
 struct fcm_unet {
     cudaStream_t stream = nullptr;
     int in_ch = 0, out_ch = 0, base = 0, levels = 0;
     std::vector<UConv> conv;  // enc (2 per level), dec (2 per level above the bottom, top-down), out
-    int64_t nparam = 0, max_w = 0;
+    int64_t nparam = 0;
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
-    __nv_bfloat16 *w16 = nullptr, *wt16 = nullptr;
+    __nv_bfloat16 *w16 = nullptr;
+    __nv_bfloat16 *tiles = nullptr;  // weight tiles of every layer (conv_tiles_kernel), made with w16
+    float *part = nullptr;           // partial sums of a weight gradient
+    float *host = nullptr;           // pinned copy of parameters and gradients for fcm_unet_get (made on first use)
+    int *err = nullptr;              // set by a convolution whose wait for the tensor core ran out
     // activations for the current shape
     int B = 0, n[3] = {0, 0, 0};
     std::vector<float *> act;  // owned buffers
     const float *input = nullptr;
     float *output = nullptr;
-    // per level l
-    std::vector<float *> xin, ea, eA, eb, eB, cat, da, dA, db, dB;
-    std::vector<float *> gxin, gea, geA, geb, geB, gcat, gda, gdA, gdb, gdB;
+    // per level l: the pooled input, the ReLU outputs of the four convolutions, and their gradients
+    std::vector<float *> xin, eA, eB, dA, dB;
+    std::vector<float *> gxin, geA, geB, gcat, gdA, gdB;
     std::vector<int64_t> S;   // voxels per level
-    std::vector<int> dim;     // nx >> l etc. (cube not required: stored per axis below)
     std::vector<int> lx, ly, lz;
     // identity of this network and of its activation buffers, for graphs that captured its launches
     uint64_t serial = 0, act_gen = 0;
@@ -302,10 +514,8 @@ cudaError_t ensure_shape(fcm_unet *N, int B, int nx, int ny, int nz)
     free_acts(N);
     ++N->act_gen;
     const int L = N->levels;
-    auto resize = [&](std::vector<float *> &v) { v.assign(L, nullptr); };
-    for (auto *v : {&N->xin, &N->ea, &N->eA, &N->eb, &N->eB, &N->cat, &N->da, &N->dA, &N->db, &N->dB, &N->gxin, &N->gea,
-                    &N->geA, &N->geb, &N->geB, &N->gcat, &N->gda, &N->gdA, &N->gdb, &N->gdB})
-        resize(*v);
+    for (auto *v : {&N->xin, &N->eA, &N->eB, &N->dA, &N->dB, &N->gxin, &N->geA, &N->geB, &N->gcat, &N->gdA, &N->gdB})
+        v->assign(L, nullptr);
     N->S.assign(L, 0);
     N->lx.assign(L, 0);
     N->ly.assign(L, 0);
@@ -323,20 +533,12 @@ cudaError_t ensure_shape(fcm_unet *N, int B, int nx, int ny, int nz)
             if ((e = falloc(N, &N->xin[l], (int64_t)B * N->ch(l - 1) * S)) != cudaSuccess) return e;
             if ((e = falloc(N, &N->gxin[l], (int64_t)B * N->ch(l - 1) * S)) != cudaSuccess) return e;
         }
-        for (auto pr : {std::make_pair(&N->ea, &N->gea), std::make_pair(&N->eA, &N->geA), std::make_pair(&N->eb, &N->geb),
-                        std::make_pair(&N->eB, &N->geB)}) {
-            if ((e = falloc(N, &(*pr.first)[l], bs)) != cudaSuccess) return e;
-            if ((e = falloc(N, &(*pr.second)[l], bs)) != cudaSuccess) return e;
-        }
+        for (auto *v : {&N->eA, &N->eB, &N->geA, &N->geB})
+            if ((e = falloc(N, &(*v)[l], bs)) != cudaSuccess) return e;
         if (l <= L - 2) {
-            const int64_t cs = (int64_t)B * (N->ch(l + 1) + c) * S;
-            if ((e = falloc(N, &N->cat[l], cs)) != cudaSuccess) return e;
-            if ((e = falloc(N, &N->gcat[l], cs)) != cudaSuccess) return e;
-            for (auto pr : {std::make_pair(&N->da, &N->gda), std::make_pair(&N->dA, &N->gdA), std::make_pair(&N->db, &N->gdb),
-                            std::make_pair(&N->dB, &N->gdB)}) {
-                if ((e = falloc(N, &(*pr.first)[l], bs)) != cudaSuccess) return e;
-                if ((e = falloc(N, &(*pr.second)[l], bs)) != cudaSuccess) return e;
-            }
+            if ((e = falloc(N, &N->gcat[l], (int64_t)B * (N->ch(l + 1) + c) * S)) != cudaSuccess) return e;
+            for (auto *v : {&N->dA, &N->dB, &N->gdA, &N->gdB})
+                if ((e = falloc(N, &(*v)[l], bs)) != cudaSuccess) return e;
         }
     }
     N->B = B;
@@ -346,47 +548,67 @@ cudaError_t ensure_shape(fcm_unet *N, int B, int nx, int ny, int nz)
     return cudaSuccess;
 }
 
-void conv_fwd(fcm_unet *N, int layer, const float *in, float *out, int l)
+// CTAs of a weight gradient's partial sums: about four per SM over the channel tiles
+int wgrad_slabs(int cin, int cout, int64_t tiles)
 {
-    const UConv &c = N->conv[layer];
-    const int64_t S = N->S[l];
-    const dim3 blk(kConvThreads);
-    if (c.cout <= 4) {
-        const dim3 grid((unsigned)((S + kConvThreads - 1) / kConvThreads), (c.cout + 3) / 4, N->B);
-        conv3_fwd_kernel<4><<<grid, blk, 0, N->stream>>>(in, N->w16 + c.woff, N->w + c.boff, out, c.cin, c.cout, N->lx[l],
-                                                         N->ly[l], N->lz[l]);
-    } else {
-        const dim3 grid((unsigned)((S + kConvThreads - 1) / kConvThreads), (c.cout + 15) / 16, N->B);
-        conv3_fwd_kernel<16><<<grid, blk, 0, N->stream>>>(in, N->w16 + c.woff, N->w + c.boff, out, c.cin, c.cout,
-                                                          N->lx[l], N->ly[l], N->lz[l]);
-    }
+    const int64_t ch = (int64_t)((cin + kWC - 1) / kWC) * ((cout + kWO - 1) / kWO);
+    return (int)std::max<int64_t>(1, std::min<int64_t>({tiles, 608 / ch, (int64_t)65535}));
 }
 
-// weight gradients of `layer` and, if gin != NULL, the data gradient (overwritten)
-void conv_bwd(fcm_unet *N, int layer, const float *in, const float *gout, float *gin, int l)
+// out = [relu](bias + conv(src)) at level l with the tiles of a convolution cin -> cout
+void conv_launch(fcm_unet *N, const ConvSrc &src, int64_t tiles, const float *bias, float *out, int cin, int cout, int l,
+                 bool relu)
 {
-    const UConv &c = N->conv[layer];
-    conv3_wgrad_kernel<<<dim3(c.cin, c.cout), 256, 0, N->stream>>>(in, gout, c.cin, c.cout, N->B, N->lx[l], N->ly[l],
-                                                                     N->lz[l], N->g + c.woff, N->g + c.boff);
-    if (!gin) return;
-    const int64_t nw = (int64_t)c.cin * c.cout * 27;
-    transpose_flip_kernel<<<blocks_for(nw), 256, 0, N->stream>>>(N->w16 + c.woff, N->wt16, c.cin, c.cout);
-    const int64_t S = N->S[l];
-    const dim3 grid((unsigned)((S + kConvThreads - 1) / kConvThreads), (c.cin + 15) / 16, N->B);
-    if (c.cin <= 4) {
-        const dim3 g4((unsigned)((S + kConvThreads - 1) / kConvThreads), (c.cin + 3) / 4, N->B);
-        conv3_fwd_kernel<4><<<g4, kConvThreads, 0, N->stream>>>(gout, N->wt16, nullptr, gin, c.cout, c.cin, N->lx[l],
-                                                                N->ly[l], N->lz[l]);
-    } else {
-        conv3_fwd_kernel<16><<<grid, kConvThreads, 0, N->stream>>>(gout, N->wt16, nullptr, gin, c.cout, c.cin, N->lx[l],
-                                                                   N->ly[l], N->lz[l]);
-    }
+    const int nx = N->lx[l], ny = N->ly[l], nz = N->lz[l], nb = conv_nb(cout);
+    const int64_t txy = (int64_t)((nx + kTX - 1) / kTX) * ((ny + kTY - 1) / kTY);
+    const uint4 *w = reinterpret_cast<const uint4 *>(N->tiles + tiles);
+    // two z planes per CTA read 2.8 instead of 4.2 halo voxels per output; with 48 or 64 columns two such CTAs do
+    // not fit an SM, and a small grid has too few of them
+    const bool two = nb <= 32 && txy * ((nz + 1) / 2) * N->B >= 304;
+    const dim3 grid((unsigned)(txy * (two ? (nz + 1) / 2 : nz)), conv_blocks(cout), N->B);
+    if (two)
+        conv3_tc_kernel<2><<<grid, kConvThreads, conv_smem(2, nb), N->stream>>>(src, w, bias, out, cin, cout, nx, ny, nz,
+                                                                              relu, N->err);
+    else
+        conv3_tc_kernel<1><<<grid, kConvThreads, conv_smem(1, nb), N->stream>>>(src, w, bias, out, cin, cout, nx, ny, nz,
+                                                                              relu, N->err);
 }
 
-void relu_f(fcm_unet *N, const float *a, float *b, int64_t n) { relu_fwd_kernel<<<blocks_for(n), 256, 0, N->stream>>>(a, b, n); }
-void relu_b(fcm_unet *N, const float *pre, const float *g, float *gp, int64_t n)
+void conv_fwd(fcm_unet *N, int layer, const ConvSrc &src, float *out, int l, bool relu)
 {
-    relu_bwd_kernel<<<blocks_for(n), 256, 0, N->stream>>>(pre, g, gp, n);
+    const UConv &c = N->conv[layer];
+    conv_launch(N, src, c.toff, N->w + c.boff, out, c.cin, c.cout, l, relu);
+}
+
+// weight gradients of `layer` and, if gin != NULL, the data gradient (overwritten); gout is read through the
+// gate (the ReLU's output; null: none)
+void conv_bwd(fcm_unet *N, int layer, const ConvSrc &in, const float *gout, const float *gate, float *gin, int l)
+{
+    const UConv &c = N->conv[layer];
+    const int nx = N->lx[l], ny = N->ly[l], nz = N->lz[l];
+    const ConvSrc go{nullptr, gout, gate, 0, c.cout};
+    const int64_t tiles = (int64_t)N->B * ((nx + kWX - 1) / kWX) * ((ny + kWY - 1) / kWY) * ((nz + kWZ - 1) / kWZ);
+    const int cit = (c.cin + kWC - 1) / kWC, cot = (c.cout + kWO - 1) / kWO, ns = wgrad_slabs(c.cin, c.cout, tiles);
+    conv3_wgrad_kernel<<<dim3(cit, cot, ns), 256, 0, N->stream>>>(in, go, c.cin, c.cout, N->B, nx, ny, nz, N->part);
+    wgrad_sum_kernel<<<blocks_for((int64_t)c.cin * c.cout * kWTaps * 8), dim3(32, kSumParts), 0, N->stream>>>(
+        N->part, ns, c.cin, c.cout, cit * kWC, cot * kWO, N->g + c.woff, N->g + c.boff);
+    if (gin) conv_launch(N, go, c.doff, nullptr, gin, c.cout, c.cin, l, false);
+}
+
+ConvSrc plain(const float *a, int c) { return ConvSrc{nullptr, a, nullptr, 0, c}; }
+
+// BF16 copy of the parameters and every layer's weight tiles
+void refresh_weights(fcm_unet *N)
+{
+    to_bf16_kernel<<<blocks_for(N->nparam), 256, 0, N->stream>>>(N->w, N->w16, N->nparam);
+    for (const UConv &c : N->conv) {
+        conv_tiles_kernel<<<blocks_for(conv_tile_entries(c.cin, c.cout)), 256, 0, N->stream>>>(N->w16 + c.woff,
+                                                                                             N->tiles + c.toff, c.cin,
+                                                                                             c.cout, 0);
+        conv_tiles_kernel<<<blocks_for(conv_tile_entries(c.cout, c.cin)), 256, 0, N->stream>>>(N->w16 + c.woff,
+                                                                                             N->tiles + c.doff, c.cout,
+                                                                                             c.cin, 1);
+    }
 }
 
 uint64_t splitmix(uint64_t &s)
@@ -446,21 +668,26 @@ fcm_status fcm_unet_create(const fcm_unet_desc *d, void *cuda_stream, fcm_unet *
     N->levels = d->levels;
     const int L = d->levels;
     for (int l = 0; l < L; ++l) {
-        N->conv.push_back({l == 0 ? d->in_ch : N->ch(l - 1), N->ch(l), 0, 0});
-        N->conv.push_back({N->ch(l), N->ch(l), 0, 0});
+        N->conv.push_back({l == 0 ? d->in_ch : N->ch(l - 1), N->ch(l), 0, 0, 0, 0});
+        N->conv.push_back({N->ch(l), N->ch(l), 0, 0, 0, 0});
     }
     for (int l = L - 2; l >= 0; --l) {
-        N->conv.push_back({N->ch(l + 1) + N->ch(l), N->ch(l), 0, 0});
-        N->conv.push_back({N->ch(l), N->ch(l), 0, 0});
+        N->conv.push_back({N->ch(l + 1) + N->ch(l), N->ch(l), 0, 0, 0, 0});
+        N->conv.push_back({N->ch(l), N->ch(l), 0, 0, 0, 0});
     }
-    N->conv.push_back({N->ch(0), d->out_ch, 0, 0});
-    int64_t off = 0;
+    N->conv.push_back({N->ch(0), d->out_ch, 0, 0, 0, 0});
+    int64_t off = 0, toff = 0, npart = 0;
     for (UConv &c : N->conv) {
         c.woff = off;
         off += (int64_t)c.cout * c.cin * 27;
         c.boff = off;
         off += c.cout;
-        N->max_w = std::max<int64_t>(N->max_w, (int64_t)c.cout * c.cin * 27);
+        c.toff = toff;
+        toff += conv_tile_entries(c.cin, c.cout);
+        c.doff = toff;
+        toff += conv_tile_entries(c.cout, c.cin);
+        const int64_t pairs = (int64_t)((c.cin + kWC - 1) / kWC * kWC) * ((c.cout + kWO - 1) / kWO * kWO);
+        npart = std::max(npart, pairs * kWTaps * wgrad_slabs(c.cin, c.cout, INT64_MAX));
     }
     N->nparam = off;
     // Kaiming-uniform weights (bound sqrt(6 / fan_in)), zero biases; the output layer 10x smaller
@@ -487,10 +714,18 @@ fcm_status fcm_unet_create(const fcm_unet_desc *d, void *cuda_stream, fcm_unet *
         if ((e = cudaMemsetAsync(*a, 0, sizeof(float) * off, N->stream)) != cudaSuccess) return fail(e);
     }
     if ((e = cudaMalloc((void **)&N->w16, sizeof(__nv_bfloat16) * off)) != cudaSuccess) return fail(e);
-    if ((e = cudaMalloc((void **)&N->wt16, sizeof(__nv_bfloat16) * N->max_w)) != cudaSuccess) return fail(e);
+    if ((e = cudaMalloc((void **)&N->tiles, sizeof(__nv_bfloat16) * toff)) != cudaSuccess) return fail(e);
+    if ((e = cudaMalloc((void **)&N->part, sizeof(float) * npart)) != cudaSuccess) return fail(e);
+    if ((e = cudaMalloc((void **)&N->err, sizeof(int))) != cudaSuccess) return fail(e);
+    if ((e = cudaMemsetAsync(N->err, 0, sizeof(int), N->stream)) != cudaSuccess) return fail(e);
+    if ((e = cudaFuncSetAttribute(conv3_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  conv_smem(1, kCoMax))) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(conv3_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, conv_smem(2, 32))) !=
+            cudaSuccess)
+        return fail(e);
     if ((e = cudaMemcpyAsync(N->w, h.data(), sizeof(float) * off, cudaMemcpyHostToDevice, N->stream)) != cudaSuccess)
         return fail(e);
-    to_bf16_kernel<<<blocks_for(off), 256, 0, N->stream>>>(N->w, N->w16, off);
+    refresh_weights(N);
     if ((e = cudaStreamSynchronize(N->stream)) != cudaSuccess) return fail(e);
     *out = N;
     return FCM_OK;
@@ -506,9 +741,21 @@ fcm_status fcm_unet_params(const fcm_unet *N, int64_t *count)
 fcm_status fcm_unet_get(fcm_unet *N, float *w_host, float *g_host)
 {
     if (!N || !w_host) return FCM_EINVAL;
-    UN_CUDA(cudaMemcpyAsync(w_host, N->w, sizeof(float) * N->nparam, cudaMemcpyDeviceToHost, N->stream));
-    if (g_host) UN_CUDA(cudaMemcpyAsync(g_host, N->g, sizeof(float) * N->nparam, cudaMemcpyDeviceToHost, N->stream));
+    // through pinned memory: a copy to the caller's pageable buffers runs at 3.4 GB/s (2 MB each, 1.2 ms)
+    const size_t bytes = sizeof(float) * N->nparam;
+    if (!N->host) UN_CUDA(cudaMallocHost((void **)&N->host, 2 * bytes + sizeof(int)));
+    int &err = *reinterpret_cast<int *>(N->host + 2 * N->nparam);
+    UN_CUDA(cudaMemcpyAsync(N->host, N->w, bytes, cudaMemcpyDeviceToHost, N->stream));
+    if (g_host) UN_CUDA(cudaMemcpyAsync(N->host + N->nparam, N->g, bytes, cudaMemcpyDeviceToHost, N->stream));
+    UN_CUDA(cudaMemcpyAsync(&err, N->err, sizeof(int), cudaMemcpyDeviceToHost, N->stream));
     UN_CUDA(cudaStreamSynchronize(N->stream));
+    std::memcpy(w_host, N->host, bytes);
+    if (g_host) std::memcpy(g_host, N->host + N->nparam, bytes);
+    if (err) {
+        UN_CUDA(cudaMemsetAsync(N->err, 0, sizeof(int), N->stream));
+        fcm_unet_last_error() = "a convolution gave up waiting for the tensor core (bounded wait); its output is not valid";
+        return FCM_ETIMEOUT;
+    }
     return FCM_OK;
 }
 
@@ -516,7 +763,7 @@ fcm_status fcm_unet_set(fcm_unet *N, const float *w_host)
 {
     if (!N || !w_host) return FCM_EINVAL;
     UN_CUDA(cudaMemcpyAsync(N->w, w_host, sizeof(float) * N->nparam, cudaMemcpyHostToDevice, N->stream));
-    to_bf16_kernel<<<blocks_for(N->nparam), 256, 0, N->stream>>>(N->w, N->w16, N->nparam);
+    refresh_weights(N);
     UN_CUDA(cudaStreamSynchronize(N->stream));
     return FCM_OK;
 }
@@ -534,31 +781,19 @@ fcm_status fcm_unet_forward(fcm_unet *N, const float *in, int B, int nx, int ny,
     N->input = in;
     N->output = out;
     for (int l = 0; l < L; ++l) {
-        const int64_t bs = (int64_t)B * N->ch(l) * N->S[l];
         if (l > 0)
             pool_fwd_kernel<<<blocks_for((int64_t)B * N->ch(l - 1) * N->S[l]), 256, 0, N->stream>>>(
                 N->eB[l - 1], N->xin[l], (int64_t)B * N->ch(l - 1), N->lx[l - 1], N->ly[l - 1], N->lz[l - 1]);
-        conv_fwd(N, N->enc_a(l), l == 0 ? in : N->xin[l], N->ea[l], l);
-        relu_f(N, N->ea[l], N->eA[l], bs);
-        conv_fwd(N, N->enc_b(l), N->eA[l], N->eb[l], l);
-        relu_f(N, N->eb[l], N->eB[l], bs);
+        conv_fwd(N, N->enc_a(l), l == 0 ? plain(in, N->in_ch) : plain(N->xin[l], N->ch(l - 1)), N->eA[l], l, true);
+        conv_fwd(N, N->enc_b(l), plain(N->eA[l], N->ch(l)), N->eB[l], l, true);
     }
     const float *prev = N->eB[L - 1];
     for (int l = L - 2; l >= 0; --l) {
-        const int cu = N->ch(l + 1), cs = N->ch(l), cc = cu + cs;
-        const int64_t S = N->S[l];
-        up_fwd_kernel<<<blocks_for((int64_t)B * cu * S), 256, 0, N->stream>>>(prev, N->cat[l], B, cu, cc, 0, N->lx[l],
-                                                                             N->ly[l], N->lz[l]);
-        chan_copy_kernel<<<blocks_for((int64_t)B * cs * S), 256, 0, N->stream>>>(N->eB[l], cs, 0, N->cat[l], cc, cu, B, cs,
-                                                                                S, 0);
-        const int64_t bs = (int64_t)B * cs * S;
-        conv_fwd(N, N->dec_a(l), N->cat[l], N->da[l], l);
-        relu_f(N, N->da[l], N->dA[l], bs);
-        conv_fwd(N, N->dec_b(l), N->dA[l], N->db[l], l);
-        relu_f(N, N->db[l], N->dB[l], bs);
+        conv_fwd(N, N->dec_a(l), ConvSrc{prev, N->eB[l], nullptr, N->ch(l + 1), N->ch(l)}, N->dA[l], l, true);
+        conv_fwd(N, N->dec_b(l), plain(N->dA[l], N->ch(l)), N->dB[l], l, true);
         prev = N->dB[l];
     }
-    conv_fwd(N, N->out_layer(), prev, out, 0);
+    conv_fwd(N, N->out_layer(), plain(prev, N->ch(0)), out, 0, false);
     UN_CUDA(cudaGetLastError());
     return FCM_OK;
 }
@@ -570,40 +805,30 @@ fcm_status fcm_unet_backward(fcm_unet *N, const float *gout, float *gin)
         return N ? FCM_ESTATE : FCM_EINVAL;
     }
     const int L = N->levels, B = N->B;
-    // skip/encoder-output gradients accumulate from two consumers
-    for (int l = 0; l < L; ++l) {
-        const int64_t bs = (int64_t)B * N->ch(l) * N->S[l];
-        fill_kernel<<<blocks_for(bs), 256, 0, N->stream>>>(N->geB[l], bs, 0.f);
-    }
     float *gtop = (L >= 2) ? N->gdB[0] : N->geB[0];
     const float *top = (L >= 2) ? N->dB[0] : N->eB[0];
-    conv_bwd(N, N->out_layer(), top, gout, gtop, 0);
+    conv_bwd(N, N->out_layer(), plain(top, N->ch(0)), gout, nullptr, gtop, 0);
     for (int l = 0; l <= L - 2; ++l) {
         const int cu = N->ch(l + 1), cs = N->ch(l), cc = cu + cs;
         const int64_t S = N->S[l], bs = (int64_t)B * cs * S;
-        relu_b(N, N->db[l], N->gdB[l], N->gdb[l], bs);
-        conv_bwd(N, N->dec_b(l), N->dA[l], N->gdb[l], N->gdA[l], l);
-        relu_b(N, N->da[l], N->gdA[l], N->gda[l], bs);
-        conv_bwd(N, N->dec_a(l), N->cat[l], N->gda[l], N->gcat[l], l);
-        // skip part -> encoder output of level l
-        chan_copy_kernel<<<blocks_for(bs), 256, 0, N->stream>>>(N->gcat[l], cc, cu, N->geB[l], cs, 0, B, cs, S, 1);
+        const float *prev = l + 1 == L - 1 ? N->eB[L - 1] : N->dB[l + 1];
+        conv_bwd(N, N->dec_b(l), plain(N->dA[l], cs), N->gdB[l], N->dB[l], N->gdA[l], l);
+        conv_bwd(N, N->dec_a(l), ConvSrc{prev, N->eB[l], nullptr, cu, cs}, N->gdA[l], N->dA[l], N->gcat[l], l);
+        // skip part -> encoder output of level l (the pooling adds the other part below)
+        chan_copy_kernel<<<blocks_for(bs), 256, 0, N->stream>>>(N->gcat[l], cc, cu, N->geB[l], cs, 0, B, cs, S, 0);
         // upsampled part -> the level below
         float *gprev = (l + 1 == L - 1) ? N->geB[L - 1] : N->gdB[l + 1];
-        const int acc = (l + 1 == L - 1) ? 1 : 0;
         up_bwd_kernel<<<blocks_for((int64_t)B * cu * N->S[l + 1]), 256, 0, N->stream>>>(
-            N->gcat[l], gprev, B, cu, cc, 0, N->lx[l], N->ly[l], N->lz[l], acc);
+            N->gcat[l], gprev, B, cu, cc, 0, N->lx[l], N->ly[l], N->lz[l], 0);
     }
     for (int l = L - 1; l >= 0; --l) {
-        const int64_t bs = (int64_t)B * N->ch(l) * N->S[l];
-        relu_b(N, N->eb[l], N->geB[l], N->geb[l], bs);
-        conv_bwd(N, N->enc_b(l), N->eA[l], N->geb[l], N->geA[l], l);
-        relu_b(N, N->ea[l], N->geA[l], N->gea[l], bs);
+        conv_bwd(N, N->enc_b(l), plain(N->eA[l], N->ch(l)), N->geB[l], N->eB[l], N->geA[l], l);
         if (l > 0) {
-            conv_bwd(N, N->enc_a(l), N->xin[l], N->gea[l], N->gxin[l], l);
+            conv_bwd(N, N->enc_a(l), plain(N->xin[l], N->ch(l - 1)), N->geA[l], N->eA[l], N->gxin[l], l);
             pool_bwd_kernel<<<blocks_for((int64_t)B * N->ch(l - 1) * N->S[l - 1]), 256, 0, N->stream>>>(
                 N->gxin[l], N->geB[l - 1], (int64_t)B * N->ch(l - 1), N->lx[l - 1], N->ly[l - 1], N->lz[l - 1]);
         } else {
-            conv_bwd(N, N->enc_a(0), N->input, N->gea[0], gin, 0);
+            conv_bwd(N, N->enc_a(0), plain(N->input, N->in_ch), N->geA[0], N->eA[0], gin, 0);
         }
     }
     UN_CUDA(cudaGetLastError());
@@ -622,7 +847,7 @@ fcm_status fcm_unet_adam(fcm_unet *N, float lr, float b1, float b2, float eps, i
     if (!N || step < 1) return FCM_EINVAL;
     const float c1 = 1.f - std::pow(b1, (float)step), c2 = 1.f - std::pow(b2, (float)step);
     adam_kernel<<<blocks_for(N->nparam), 256, 0, N->stream>>>(N->w, N->g, N->m, N->v, N->nparam, lr, b1, b2, eps, c1, c2);
-    to_bf16_kernel<<<blocks_for(N->nparam), 256, 0, N->stream>>>(N->w, N->w16, N->nparam);
+    refresh_weights(N);
     UN_CUDA(cudaGetLastError());
     return FCM_OK;
 }
@@ -632,9 +857,10 @@ void fcm_unet_destroy(fcm_unet *N)
     if (!N) return;
     if (N->stream) cudaStreamSynchronize(N->stream);
     free_acts(N);
-    void *ptrs[] = {N->w, N->g, N->m, N->v, N->w16, N->wt16};
+    void *ptrs[] = {N->w, N->g, N->m, N->v, N->w16, N->tiles, N->part, N->err};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+    if (N->host) cudaFreeHost(N->host);
     delete N;
 }
 
