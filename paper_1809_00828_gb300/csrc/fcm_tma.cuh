@@ -60,6 +60,15 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
 }
 
+// One thread of a converged warp.
+__device__ __forceinline__ bool tc_elect()
+{
+    uint32_t on;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(on)::"memory");
+    return on != 0;
+}
+
 // D (tensor memory) (+)= A B, kind::f16 (BF16 operands by `idesc`); one thread issues it
 __device__ __forceinline__ void tc_mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, int acc)
 {

@@ -32,9 +32,12 @@ namespace {
 // tile with its halo of one voxel to shared memory, [split][8 channels][z][y][x] with 16 bytes per voxel:
 // eight voxels along x are a core matrix of the canonical K-major layout without swizzle and a row of them a
 // fixed stride, so each of the 27 taps is the same tile at another start address, and no input is gathered
-// twice.  Forward pass on 80^3 cells, channels 16 to 64 (75 GFLOP of convolutions): 1.19 ms, 5.76 ms with FP32
-// arithmetic on the CUDA cores (13 TFLOP/s); bound by the rate at which one thread issues products, 81 per 128
-// voxels and 16 input channels.  Two CTAs per SM overlap one's halo loads with the other's products.
+// twice.  A halo plane goes through the taps of up to three output planes in one product (N up to 3 x the
+// columns: the accumulators of the tile's planes lie side by side), since one thread issues the products at a
+// rate that does not depend on N: 27 (ZT + 2) of them per 16 input channels instead of 81 ZT.  Forward pass on
+// 80^3 cells, channels 16 to 64 (75 GFLOP of convolutions): 0.90 ms; 1.19 ms with a product per plane, and
+// 5.76 ms with FP32 arithmetic on the CUDA cores (13 TFLOP/s).  Two CTAs per SM overlap one's halo loads with
+// the other's products.
 //
 // The tensor core adds into its FP32 accumulators by truncation: with one accumulator over all 81 products of
 // 16 input channels the outputs were 5.6e-6 off (relative, 2-norm), 10 times the FP32 multiply-adds' error.  So
@@ -53,6 +56,16 @@ __host__ __device__ constexpr int conv_hv(int ZT) { return kHX * kHY * (ZT + 2);
 __host__ __device__ constexpr int conv_a_bytes(int ZT) { return 3 * 2 * 16 * conv_hv(ZT); }
 __host__ __device__ constexpr int conv_smem(int ZT, int nb) { return 1024 + conv_a_bytes(ZT) + 27 * 32 * nb; }
 __host__ __device__ constexpr int up16(int n) { return (n + 15) / 16 * 16; }
+// A halo plane i reaches the tile's planes z = i - 2 + s in [0, ZT) by the taps of dz = 2 - s ("slots" s): first slot,
+// number of slots, and slots of the planes before it
+__host__ __device__ constexpr int conv_s0(int i) { return i < 2 ? 2 - i : 0; }
+__host__ __device__ constexpr int conv_ns(int ZT, int i) { return (ZT + 1 - i < 2 ? ZT + 1 - i : 2) - conv_s0(i) + 1; }
+__host__ __device__ constexpr int conv_at(int ZT, int i)
+{
+    int n = 0;
+    for (int k = 0; k < i; ++k) n += conv_ns(ZT, k);
+    return n;
+}
 // columns (output channels) of a CTA, CTAs per voxel tile, and BF16 entries of a layer's weight tiles
 __host__ __device__ constexpr int conv_nb(int n) { return n <= kCoMax ? up16(n) : kCoMax; }
 __host__ __device__ constexpr int conv_blocks(int n) { return (n + kCoMax - 1) / kCoMax; }
@@ -171,26 +184,31 @@ __global__ void __launch_bounds__(kConvThreads)
         // the tensor core reads shared memory through the async proxy
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0 && tc_elect()) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // FP32 accumulator, BF16 A and B, both K-major, M = 128, N = nb
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nb >> 3) << 17) | (8u << 24);
-            const uint32_t a0 = smem_u32(A), w0 = smem_u32(W);
-            const int zn = min(ZT, nz - z0);
-            // accumulator 4 z + dz: the leading parts of the taps of plane dz; 4 z + 3: the small parts
-            for (int t = 0; t < 9; ++t)
-                for (int dz = 0; dz < 3; ++dz) {
-                    const uint64_t bd = smem_desc(w0 + (9 * dz + t) * 32 * nb, 128, 256);
-                    const int at = dz * kHX * kHY + t / 3 * kHX + t % 3;
-                    for (int z = 0; z < zn; ++z) {
-                        const uint32_t a = a0 + 16 * (at + z * kHX * kHY), d = tmem + 4 * z * nb;
-                        tc_mma_bf16(d + dz * nb, smem_desc(a, 16 * HV, 16 * kHX), bd, idesc, t > 0);
-                        tc_mma_bf16(d + 3 * nb, smem_desc(a + 64 * HV, 16 * HV, 16 * kHX), bd, idesc, t > 0 || dz > 0);
-                        tc_mma_bf16(d + 3 * nb, smem_desc(a + 32 * HV, 16 * HV, 16 * kHX), bd, idesc, 1);
+            // FP32 accumulator, BF16 A and B, both K-major, M = 128, N = nb .. 3 nb
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24), in8 = (uint32_t)(nb >> 3) << 17;
+            const uint64_t a0 = smem_desc(smem_u32(A), 16 * HV, 16 * kHX);
+            uint64_t bt = smem_desc(smem_u32(W), 128, 256);
+            const uint32_t small = tmem + 3 * ZT * nb;
+#pragma unroll
+            for (int t = 0; t < 9; ++t, bt += 6 * nb)
+#pragma unroll
+                for (int q = 2; q >= 0; --q)
+#pragma unroll
+                    for (int k = 0; k < ZT + 2; ++k) {
+                        // planes 2, 5, .. first: together they write each small accumulator once
+                        constexpr int n3 = (ZT + 2) / 3;
+                        const int i = k < n3 ? 3 * k + 2 : (k - n3) / 2 * 3 + (k - n3) % 2;
+                        const uint64_t ad = a0 + (uint64_t)(2 * q * HV + i * kHX * kHY + t / 3 * kHX + t % 3);
+                        const uint64_t bd = bt + (uint64_t)(2 * conv_s0(i) * nb);
+                        const uint32_t id = idesc + conv_ns(ZT, i) * in8;
+                        if (q == 0) tc_mma_bf16(tmem + conv_at(ZT, i) * nb, ad, bd, id, t > 0);
+                        else tc_mma_bf16(small + (i < 2 ? 0 : i - 2) * nb, ad, bd, id, t > 0 || q < 2 || k >= n3);
                     }
-                }
             tc_commit(bar);
         }
+        __syncwarp();
         if (!mbar_wait(bar, ch & 1, kWaitTries)) {
             atomicExch(err, 1);  // the products still in flight land before shared memory is written again
             mbar_wait(bar, ch & 1, kDrainTries);
@@ -201,12 +219,18 @@ __global__ void __launch_bounds__(kConvThreads)
         for (int i = 0; i < 2; ++i) {
             const int it = (warp >> 2) + 2 * i;
             if (it >= items) break;  // uniform across the warp
-            const uint32_t at = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 4 * (it / (nb / 16)) * nb + it % (nb / 16) * 16;
+            const int z = it / (nb / 16);
+            const uint32_t at = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + it % (nb / 16) * 16;
             float part[16];
 #pragma unroll
             for (int q = 3; q >= 0; --q) {
+                int blk = 3 * ZT + z;  // the small parts, then the leading ones of dz = 2, 1, 0
+                if (q < 3) {
+                    blk = 2 - q - conv_s0(z + q);
+                    for (int k = 0; k < z + q; ++k) blk += conv_ns(ZT, k);
+                }
                 uint32_t v[16];
-                tc_load16(at + q * nb, v);
+                tc_load16(at + blk * nb, v);
 #pragma unroll
                 for (int k = 0; k < 16; ++k)
                     part[k] = q == 3 ? __uint_as_float(v[k]) : __fadd_rn(part[k], __uint_as_float(v[k]));
@@ -239,7 +263,8 @@ __global__ void __launch_bounds__(kConvThreads)
 }
 
 // Weight tiles of one layer in the tensor core's layout, from the BF16 weights w[co][ci][27]: per block of 64
-// output channels, 16 input channels and tap, [channel / 8][K / 8][8 channels][8 K] (zeros beyond the layer).
+// output channels, 16 input channels, (dy, dx) and slot 2 - dz, [channel / 8][K / 8][8 channels][8 K] (zeros beyond
+// the layer).
 // flip: the tiles of the data-gradient convolution, w'[ci][co][26 - tap] (cin, cout: those of that convolution).
 __global__ void conv_tiles_kernel(const __nv_bfloat16 *__restrict__ w, __nv_bfloat16 *__restrict__ t, int cin, int cout,
                                   int flip)
@@ -251,7 +276,7 @@ __global__ void conv_tiles_kernel(const __nv_bfloat16 *__restrict__ w, __nv_bflo
         int64_t q = e >> 7;
         const int n8 = (int)(q % (nb / 8));
         q /= nb / 8;
-        const int tap = (int)(q % 27);
+        const int tap = 9 * (2 - (int)(q % 3)) + (int)(q / 3 % 9);
         q /= 27;
         const int ci = 16 * (int)(q % nch) + 8 * kc + k, co = kCoMax * (int)(q / nch) + 8 * n8 + r;
         __nv_bfloat16 v = __float2bfloat16(0.f);
@@ -263,28 +288,30 @@ __global__ void conv_tiles_kernel(const __nv_bfloat16 *__restrict__ w, __nv_bflo
 
 // ---- weight gradients: gw[co][ci][tap] += sum_{b,p} gout[b][co][p] in[b][ci][p + off(tap)], gb[co] += sum gout
 //
-// A CTA owns 16 output x 8 input channels and walks tiles of 8 x 8 x 4 voxels; a thread owns one (co, ci) pair
-// of half of the voxels with its 27 taps (and the bias) in registers, so four voxels along x cost 19 vector
-// reads of shared memory and 112 multiply-adds: bound by the FP32 pipe.  The tiles are dealt to enough CTAs to
-// fill the GPU, each writes its sums to `part`, and wgrad_sum_kernel adds them in a fixed order in FP64
-// (deterministic).  One CTA per (co, ci) pair with 27 unshared global reads per multiply-add row took 4.9 ms
-// for the gradients of the 16-to-64-channel network on four 32^3 cubes; this 1.08 + 0.29 ms.
-constexpr int kWC = 8, kWO = 16, kWX = 8, kWY = 8, kWZ = 4, kWPitch = 12, kWGo = kWX * kWY * kWZ + 4;
+// A CTA owns 16 output x 8 input channels and walks tiles of 8 x 8 x 4 voxels; a thread owns two output channels
+// and one input channel of one plane of the tile, with their 27 taps (and the bias) in registers: eight voxels
+// along x cost 31 vector reads of shared memory and 448 multiply-adds (one output channel and four voxels a time
+// cost 19 reads for 112).  The tiles are dealt to enough CTAs to fill the GPU, each
+// writes its sums to `part`, and wgrad_sum_kernel adds them in a fixed order in FP64 (deterministic).  One CTA per
+// (co, ci) pair with 27 unshared global reads per multiply-add row took 4.9 ms for the gradients of the
+// 16-to-64-channel network on four 32^3 cubes, one channel a thread 1.08 + 0.29 ms; this 1.00 + 0.12 ms.
+constexpr int kWC = 8, kWO = 16, kWX = 8, kWY = 8, kWZ = 4, kWGo = kWX * kWY * kWZ + 4;
+constexpr int kWRow = 12, kWPlane = kWRow * (kWY + 2), kWCh = kWPlane * (kWZ + 2) + 4;  // 4 channels: distinct banks
 constexpr int kWTaps = 28;
 constexpr int kSumParts = 16;  // parts of the slabs that wgrad_sum_kernel adds side by side
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
     conv3_wgrad_kernel(ConvSrc in, ConvSrc go, int cin, int cout, int B, int nx, int ny, int nz, float *__restrict__ part)
 {
-    __shared__ __align__(16) float si[kWC][kWZ + 2][kWY + 2][kWPitch];
+    __shared__ __align__(16) float si[kWC * kWCh];
     __shared__ __align__(16) float sg[kWO][kWGo];
     const int ci0 = blockIdx.x * kWC, co0 = blockIdx.y * kWO, tid = threadIdx.x;
-    const int co = tid & 15, ci = tid >> 4 & 7, zh = tid >> 7;  // zh: z planes 2 zh, 2 zh + 1 of the tile
+    const int co = tid & 7, ci = tid >> 3 & 7, zq = tid >> 6;  // output channels co, co + 8; plane zq of the tile
     const int tx = (nx + kWX - 1) / kWX, ty = (ny + kWY - 1) / kWY, tz = (nz + kWZ - 1) / kWZ;
     const int64_t tiles = (int64_t)B * tx * ty * tz;
-    float acc[kWTaps];
+    float acc[2][kWTaps];
 #pragma unroll
-    for (int t = 0; t < kWTaps; ++t) acc[t] = 0.f;
+    for (int t = 0; t < kWTaps; ++t) acc[0][t] = acc[1][t] = 0.f;
     for (int64_t tile = blockIdx.z; tile < tiles; tile += gridDim.z) {
         const int b = (int)(tile / ((int64_t)tx * ty * tz)), q = (int)(tile % ((int64_t)tx * ty * tz));
         const int x0 = q % tx * kWX, y0 = q / tx % ty * kWY, z0 = q / (tx * ty) * kWZ;
@@ -294,7 +321,7 @@ __global__ void __launch_bounds__(256)
                       c = e / ((kWX + 2) * (kWY + 2) * (kWZ + 2));
             const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
             const bool on = ci0 + c < cin && x >= 0 && y >= 0 && z >= 0 && x < nx && y < ny && z < nz;
-            si[c][hz][hy][hx] = on ? conv_load(in, b, ci0 + c, x, y, z, nx, ny, nz) : 0.f;
+            si[c * kWCh + hz * kWPlane + hy * kWRow + hx] = on ? conv_load(in, b, ci0 + c, x, y, z, nx, ny, nz) : 0.f;
         }
         for (int e = tid; e < kWO * kWX * kWY * kWZ; e += 256) {
             const int v = e % (kWX * kWY * kWZ), c = e / (kWX * kWY * kWZ);
@@ -304,42 +331,57 @@ __global__ void __launch_bounds__(256)
         }
         __syncthreads();
 #pragma unroll 1
-        for (int zy = 0; zy < 2 * kWY; ++zy) {
-            const int z = 2 * zh + zy / kWY, y = zy % kWY;
+        for (int y = 0; y < kWY; ++y) {
+            float g[2][8];
 #pragma unroll
-            for (int xr = 0; xr < kWX; xr += 4) {
-                const float4 g4 = *reinterpret_cast<const float4 *>(&sg[co][(z * kWY + y) * kWX + xr]);
-                const float g[4] = {g4.x, g4.y, g4.z, g4.w};
-                acc[27] += (g[0] + g[1]) + (g[2] + g[3]);
+            for (int o = 0; o < 2; ++o) {
+                const float4 *p = reinterpret_cast<const float4 *>(&sg[co + 8 * o][(zq * kWY + y) * kWX]);
+                const float4 a = p[0], c = p[1];
+                g[o][0] = a.x, g[o][1] = a.y, g[o][2] = a.z, g[o][3] = a.w;
+                g[o][4] = c.x, g[o][5] = c.y, g[o][6] = c.z, g[o][7] = c.w;
+                acc[o][27] += ((a.x + a.y) + (a.z + a.w)) + ((c.x + c.y) + (c.z + c.w));
+            }
 #pragma unroll
-                for (int d = 0; d < 9; ++d) {
-                    const float *row = &si[ci][z + d / 3][y + d % 3][xr];
-                    const float4 a = *reinterpret_cast<const float4 *>(row);
-                    const float2 c = *reinterpret_cast<const float2 *>(row + 4);
-                    const float v[6] = {a.x, a.y, a.z, a.w, c.x, c.y};
+            for (int d = 0; d < 9; ++d) {
+                const float *row = si + ci * kWCh + (zq + d / 3) * kWPlane + (y + d % 3) * kWRow;
+                const float4 a = *reinterpret_cast<const float4 *>(row), c = *reinterpret_cast<const float4 *>(row + 4);
+                const float2 f = *reinterpret_cast<const float2 *>(row + 8);
+                const float v[10] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w, f.x, f.y};
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
 #pragma unroll
                     for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) acc[3 * d + dx] = fmaf(g[k], v[k + dx], acc[3 * d + dx]);
-                }
+                        for (int o = 0; o < 2; ++o) acc[o][3 * d + dx] = fmaf(g[o][k], v[k + dx], acc[o][3 * d + dx]);
             }
         }
     }
-    // the two halves of the voxels, then this CTA's sums: part[z][co][ci][tap]
-    __syncthreads();
-    float *red = &si[0][0][0][0];  // 128 x 28 floats
-    static_assert(128 * kWTaps <= kWC * (kWZ + 2) * (kWY + 2) * kWPitch, "reduction buffer");
-    if (zh == 1)
+    // the four planes, then this CTA's sums: part[z][co][ci][tap]
+    float *red = si;  // 64 x 2 x 28 floats
+    static_assert(64 * 2 * kWTaps <= kWC * kWCh, "reduction buffer");
+#pragma unroll 1
+    for (int w = 1; w < kWZ; ++w) {
+        __syncthreads();
+        if (zq == w)
 #pragma unroll
-        for (int t = 0; t < kWTaps; ++t) red[t * 128 + (tid & 127)] = acc[t];
-    __syncthreads();
-    if (zh == 0) {
-        float *p = part + ((((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * kWO + co) * (gridDim.x * kWC) + ci0 + ci) * kWTaps;
+            for (int t = 0; t < 2 * kWTaps; ++t) red[t * 64 + (tid & 63)] = acc[t / kWTaps][t % kWTaps];
+        __syncthreads();
+        if (zq == 0)
 #pragma unroll
-        for (int t = 0; t < kWTaps; ++t) p[t] = acc[t] + red[t * 128 + tid];
+            for (int t = 0; t < 2 * kWTaps; ++t) acc[t / kWTaps][t % kWTaps] += red[t * 64 + tid];
+    }
+    if (zq == 0) {
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+            float4 *p = reinterpret_cast<float4 *>(
+                part + ((((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * kWO + co + 8 * o) * (gridDim.x * kWC) + ci0 + ci) * kWTaps);
+#pragma unroll
+            for (int t = 0; t < kWTaps; t += 4) p[t / 4] = make_float4(acc[o][t], acc[o][t + 1], acc[o][t + 2], acc[o][t + 3]);
+        }
     }
 }
 
+// one warp per 32 entries and part of the slabs; blockDim.y parts, so that a thread adds about eight slabs
 __global__ void __launch_bounds__(32 * kSumParts)
     wgrad_sum_kernel(const float *__restrict__ part, int nslab, int cin, int cout, int cip, int cop, float *__restrict__ gw,
                      float *__restrict__ gb)
@@ -354,17 +396,18 @@ __global__ void __launch_bounds__(32 * kSumParts)
         if (on) {
             const float *p = part + ((int64_t)co * cip + ci) * kWTaps + t;
 #pragma unroll 8
-            for (int k = threadIdx.y; k < nslab; k += kSumParts) s += p[k * slab];
+            for (int k = threadIdx.y; k < nslab; k += blockDim.y) s += p[k * slab];
         }
-        sh[threadIdx.y][threadIdx.x] = s;
-        __syncthreads();
+        if (blockDim.y > 1) {
+            sh[threadIdx.y][threadIdx.x] = s;
+            __syncthreads();
+        }
         if (threadIdx.y == 0 && on) {
-#pragma unroll
-            for (int q = 1; q < kSumParts; ++q) s += sh[q][threadIdx.x];
+            for (int q = 1; q < blockDim.y; ++q) s += sh[q][threadIdx.x];
             if (t < 27) gw[((int64_t)co * cin + ci) * 27 + t] += (float)s;
             else gb[co] += (float)s;
         }
-        __syncthreads();
+        if (blockDim.y > 1) __syncthreads();
     }
 }
 
@@ -548,11 +591,11 @@ cudaError_t ensure_shape(fcm_unet *N, int B, int nx, int ny, int nz)
     return cudaSuccess;
 }
 
-// CTAs of a weight gradient's partial sums: about four per SM over the channel tiles
+// CTAs of a weight gradient's partial sums: two per SM over the channel tiles
 int wgrad_slabs(int cin, int cout, int64_t tiles)
 {
     const int64_t ch = (int64_t)((cin + kWC - 1) / kWC) * ((cout + kWO - 1) / kWO);
-    return (int)std::max<int64_t>(1, std::min<int64_t>({tiles, 608 / ch, (int64_t)65535}));
+    return (int)std::max<int64_t>(1, std::min<int64_t>({tiles, 304 / ch, (int64_t)65535}));
 }
 
 // out = [relu](bias + conv(src)) at level l with the tiles of a convolution cin -> cout
@@ -562,16 +605,14 @@ void conv_launch(fcm_unet *N, const ConvSrc &src, int64_t tiles, const float *bi
     const int nx = N->lx[l], ny = N->ly[l], nz = N->lz[l], nb = conv_nb(cout);
     const int64_t txy = (int64_t)((nx + kTX - 1) / kTX) * ((ny + kTY - 1) / kTY);
     const uint4 *w = reinterpret_cast<const uint4 *>(N->tiles + tiles);
-    // two z planes per CTA read 2.8 instead of 4.2 halo voxels per output; with 48 or 64 columns two such CTAs do
-    // not fit an SM, and a small grid has too few of them
-    const bool two = nb <= 32 && txy * ((nz + 1) / 2) * N->B >= 304;
-    const dim3 grid((unsigned)(txy * (two ? (nz + 1) / 2 : nz)), conv_blocks(cout), N->B);
-    if (two)
-        conv3_tc_kernel<2><<<grid, kConvThreads, conv_smem(2, nb), N->stream>>>(src, w, bias, out, cin, cout, nx, ny, nz,
-                                                                              relu, N->err);
-    else
-        conv3_tc_kernel<1><<<grid, kConvThreads, conv_smem(1, nb), N->stream>>>(src, w, bias, out, cin, cout, nx, ny, nz,
-                                                                              relu, N->err);
+    // More planes per CTA take fewer products and halo voxels per output (27 (ZT + 2) and 1.4 (ZT + 2), over ZT);
+    // with 16 columns three and with 32 two still leave room for two CTAs per SM (256 of 512 tensor-memory columns
+    // each), and a small grid has too few of them.
+    const auto ctas = [&](int zt) { return txy * ((nz + zt - 1) / zt) * N->B * conv_blocks(cout); };
+    const int zt = nb == 16 && ctas(3) >= 304 ? 3 : nb <= 32 && ctas(2) >= 304 ? 2 : 1;
+    const auto kernel = zt == 3 ? conv3_tc_kernel<3> : zt == 2 ? conv3_tc_kernel<2> : conv3_tc_kernel<1>;
+    const dim3 grid((unsigned)(txy * ((nz + zt - 1) / zt)), conv_blocks(cout), N->B);
+    kernel<<<grid, kConvThreads, conv_smem(zt, nb), N->stream>>>(src, w, bias, out, cin, cout, nx, ny, nz, relu, N->err);
 }
 
 void conv_fwd(fcm_unet *N, int layer, const ConvSrc &src, float *out, int l, bool relu)
@@ -590,7 +631,8 @@ void conv_bwd(fcm_unet *N, int layer, const ConvSrc &in, const float *gout, cons
     const int64_t tiles = (int64_t)N->B * ((nx + kWX - 1) / kWX) * ((ny + kWY - 1) / kWY) * ((nz + kWZ - 1) / kWZ);
     const int cit = (c.cin + kWC - 1) / kWC, cot = (c.cout + kWO - 1) / kWO, ns = wgrad_slabs(c.cin, c.cout, tiles);
     conv3_wgrad_kernel<<<dim3(cit, cot, ns), 256, 0, N->stream>>>(in, go, c.cin, c.cout, N->B, nx, ny, nz, N->part);
-    wgrad_sum_kernel<<<blocks_for((int64_t)c.cin * c.cout * kWTaps * 8), dim3(32, kSumParts), 0, N->stream>>>(
+    const int np = std::max(1, std::min(ns / 8, kSumParts));
+    wgrad_sum_kernel<<<blocks_for((int64_t)c.cin * c.cout * kWTaps * 8), dim3(32, np), 0, N->stream>>>(
         N->part, ns, c.cin, c.cout, cit * kWC, cot * kWO, N->g + c.woff, N->g + c.boff);
     if (gin) conv_launch(N, go, c.doff, nullptr, gin, c.cout, c.cin, l, false);
 }
@@ -721,6 +763,8 @@ fcm_status fcm_unet_create(const fcm_unet_desc *d, void *cuda_stream, fcm_unet *
     if ((e = cudaFuncSetAttribute(conv3_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   conv_smem(1, kCoMax))) != cudaSuccess ||
         (e = cudaFuncSetAttribute(conv3_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, conv_smem(2, 32))) !=
+            cudaSuccess ||
+        (e = cudaFuncSetAttribute(conv3_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, conv_smem(3, 16))) !=
             cudaSuccess)
         return fail(e);
     if ((e = cudaMemcpyAsync(N->w, h.data(), sizeof(float) * off, cudaMemcpyHostToDevice, N->stream)) != cudaSuccess)
