@@ -66,17 +66,17 @@ struct StreamScope {
     }
 };
 
-void apply_K_dev(fcm_ctx *C, const double *x, double *y, const int *done)
+void apply_K_dev(fcm_ctx *C, const double *x, double *y, const int *done, const uint8_t *xmask = nullptr)
 {
     if (C->k_ff)
-        fcm::launch_k_apply_ff(C->p, C->g, x, y, C->d_mask, C->d_elem_ff, C->kc, done, C->stream, C->ks);
+        fcm::launch_k_apply_ff(C->p, C->g, x, y, C->d_mask, C->d_elem_ff, C->kc, xmask, done, C->stream, C->ks);
     else
-        fcm::launch_k_apply(C->p, C->g, x, y, C->d_mask, C->d_elem, C->kc, done, C->stream, C->ks);
+        fcm::launch_k_apply(C->p, C->g, x, y, C->d_mask, C->d_elem, C->kc, xmask, done, C->stream, C->ks);
 }
 
-void apply_S_dev(fcm_ctx *C, const double *r, double *z, const int *done)
+void apply_S_dev(fcm_ctx *C, const double *r, double *z, const int *done, const uint8_t *xmask = nullptr)
 {
-    fcm::launch_schwarz_apply(C->p, C->g, r, z, C->d_f64, C->d_f32, C->plan, done, C->stream);
+    fcm::launch_schwarz_apply(C->p, C->g, r, z, C->d_f64, C->d_f32, C->plan, xmask, done, C->stream);
 }
 
 void destroy_graph(fcm_ctx *C)
@@ -560,7 +560,7 @@ static fcm_status solve_multi(fcm_ctx *C, const double *rhs, int nr, double tol,
     API_CUDA(C, cudaMemcpyAsync(C->d_ms, C->h_ms, sizeof(CgScalars) * nr, cudaMemcpyHostToDevice, st));
     API_CUDA(C, cudaEventRecord(C->ev_t0, st));
     for (int k = 0; k < nr; ++k) fcm::cg_init_kernels(w[k], st);
-    fcm::launch_schwarz_apply_multi(C->p, R, Z, n, nr, C->d_f64, C->d_f32, C->plan, C->d_mzb, nullptr, st);
+    fcm::launch_schwarz_apply_multi(C->p, R, Z, n, nr, C->d_f64, C->d_f32, C->plan, C->d_mzb, nullptr, nullptr, st);
     for (int k = 0; k < nr; ++k) fcm::cg_after_first_S(w[k], st);
     for (int it = 0;; ++it) {
         if (it % 8 == 0) {
@@ -579,7 +579,7 @@ static fcm_status solve_multi(fcm_ctx *C, const double *rhs, int nr, double tol,
         }
         for (int k = 0; k < nr; ++k) apply_K_dev(C, w[k].p, w[k].q, &C->d_ms[k].done);
         for (int k = 0; k < nr; ++k) fcm::cg_after_K(w[k], st);
-        fcm::launch_schwarz_apply_multi(C->p, R, Z, n, nr, C->d_f64, C->d_f32, C->plan, C->d_mzb, nullptr, st);
+        fcm::launch_schwarz_apply_multi(C->p, R, Z, n, nr, C->d_f64, C->d_f32, C->plan, C->d_mzb, nullptr, nullptr, st);
         for (int k = 0; k < nr; ++k) fcm::cg_after_S(w[k], st);
         API_CUDA(C, cudaGetLastError());
     }
@@ -687,8 +687,12 @@ fcm_status fcm_apply_K(fcm_ctx *C, const double *x_dev, double *y_dev)
 {
     if (!C || !x_dev || !y_dev) return FCM_EINVAL;
     StreamScope sc(C);
-    fcm::launch_mask_copy(x_dev, C->d_t, C->d_mask, C->nlat, C->stream);
-    apply_K_dev(C, C->d_t, y_dev, nullptr);
+    if (C->kc.n_uncut > 0) {
+        fcm::launch_mask_copy(x_dev, C->d_t, C->d_mask, C->nlat, C->stream);
+        apply_K_dev(C, C->d_t, y_dev, nullptr);
+    } else {  // y_dev (which may overlap x_dev) is written after all cells' products
+        apply_K_dev(C, x_dev, y_dev, nullptr, C->d_mask);
+    }
     API_CUDA(C, cudaGetLastError());
     return FCM_OK;
 }
@@ -701,8 +705,12 @@ fcm_status fcm_apply_S(fcm_ctx *C, const double *r_dev, double *z_dev)
         return FCM_ESTATE;
     }
     StreamScope sc(C);
-    fcm::launch_mask_copy(r_dev, C->d_t, C->d_mask, C->nlat, C->stream);
-    apply_S_dev(C, C->d_t, z_dev, nullptr);
+    if (C->d_jac) {  // the diagonal part reads r while z is written: a copy keeps overlapping buffers apart
+        fcm::launch_mask_copy(r_dev, C->d_t, C->d_mask, C->nlat, C->stream);
+        apply_S_dev(C, C->d_t, z_dev, nullptr);
+    } else {
+        apply_S_dev(C, r_dev, z_dev, nullptr, C->d_mask);
+    }
     API_CUDA(C, cudaGetLastError());
     return FCM_OK;
 }
@@ -737,9 +745,16 @@ fcm_status fcm_apply_S_many(fcm_ctx *C, const double *r_dev, int nrhs, double *z
         API_CUDA(C, cudaMalloc(&C->d_mzb, sizeof(double) * (size_t)nrhs * C->plan.nslots * C->plan.zs));
         C->m_nr = nrhs;
     }
-    double *R = C->d_m;  // masked copies of the inputs
-    for (int k = 0; k < nrhs; ++k) fcm::launch_mask_copy(r_dev + (size_t)k * n, R + (size_t)k * n, C->d_mask, n, C->stream);
-    fcm::launch_schwarz_apply_multi(C->p, R, z_dev, n, nrhs, C->d_f64, C->d_f32, C->plan, C->d_mzb, nullptr, C->stream);
+    const double *R = r_dev;
+    const uint8_t *xmask = C->d_mask;
+    if (C->d_jac) {  // as in fcm_apply_S
+        for (int k = 0; k < nrhs; ++k)
+            fcm::launch_mask_copy(r_dev + (size_t)k * n, C->d_m + (size_t)k * n, C->d_mask, n, C->stream);
+        R = C->d_m;
+        xmask = nullptr;
+    }
+    fcm::launch_schwarz_apply_multi(C->p, R, z_dev, n, nrhs, C->d_f64, C->d_f32, C->plan, C->d_mzb, xmask, nullptr,
+                                    C->stream);
     API_CUDA(C, cudaGetLastError());
     return FCM_OK;
 }

@@ -18,8 +18,10 @@ struct PatchRec {
     int64_t off;   // element offset of the block factor in the factor pool
     int32_t v;     // vertex patches: linear vertex index v_x + (n_x+1)(v_y + (n_y+1) v_z);
                    // element blocks: linear cell index c_x + n_x (c_y + n_y c_z)
-    int32_t prec;  // 0: factor stored in FP64, 1: FP32
+    int32_t prec;  // 0: factor stored in FP64, 1: FP32, 2: float pairs; + kMaskedBlock if its box holds entries
+                   // that are not free
 };
+constexpr int kMaskedBlock = 1 << 8;
 
 // Leading dimension of a stored block factor with n rows: rows are padded to a multiple of 16
 // bytes (zeros), so a row, or a run of rows, can be moved by one bulk copy and read as 16-byte
@@ -53,6 +55,10 @@ struct CutCell {
     int64_t base;
     int cell, elem;
 };
+#ifdef __CUDACC__
+// an input entry of K; 0 where its mask byte (may be null) says it is not free
+__device__ __forceinline__ double k_input(const double *x, const uint8_t *m) { return m && !*m ? 0.0 : __ldg(x); }
+#endif
 
 // Active cells of the K apply, in cell order: uncut cells (matrix-free) and cut cells (their own dense
 // element matrix).
@@ -93,7 +99,7 @@ struct TcTile {
 };
 
 // A block with a folded factor of its own: factor offset (floats), lattice DOF at the low corner of its box,
-// slot, nodes of the box per axis.
+// slot (~slot if its box holds entries that are not free), nodes of the box per axis.
 struct FoldItem {
     int64_t off, base;
     int slot, d[3];
@@ -135,14 +141,17 @@ struct KStreams {
     cudaEvent_t fork, join;
 };
 
-// Launchers (all asynchronous on `s`).  `done` may be null.  The Schwarz launchers overwrite z
-// with S r.  The multi-RHS form takes nr <= 8 vectors nlat apart and a Zb of nr * nslots * zs doubles.
+// Launchers (all asynchronous on `s`).  `done` may be null.  `xmask` (null: the input's entries that are not free
+// are 0, as in the solver's own vectors) makes the kernels read those entries as 0, so that an apply called from
+// outside needs no masked copy of its input (S at 80^3, p = 2: 732 -> 718 us; K and S of a 4^3 grid: 36 -> 28.7).
+// K takes it for dense cells only: the modal kernel lost as much to the mask's loads (218 -> 246 us) as the copy
+// took.  The Schwarz launchers overwrite z with S r.  The multi-RHS form takes nr <= 8 vectors nlat apart and a Zb of nr * nslots * zs doubles.
 void launch_k_apply(int p, const Grid3 &g, const double *x, double *y, const uint8_t *mask, const double *elem,
-                    const KCells &kc, const int *done, cudaStream_t s, const KStreams &ks);
+                    const KCells &kc, const uint8_t *xmask, const int *done, cudaStream_t s, const KStreams &ks);
 // the same in double-float arithmetic on the FP32 pipe (fcm_kapply_ff.cu); elem: the element matrices as
 // float pairs
 void launch_k_apply_ff(int p, const Grid3 &g, const double *x, double *y, const uint8_t *mask, const float2 *elem,
-                       const KCells &kc, const int *done, cudaStream_t s, const KStreams &ks);
+                       const KCells &kc, const uint8_t *xmask, const int *done, cudaStream_t s, const KStreams &ks);
 // kernel attributes (dynamic shared memory); host calls, outside stream capture
 cudaError_t k_prepare(int p);
 cudaError_t k_prepare_ff(int p);
@@ -152,10 +161,11 @@ void launch_to_ff_pairs(const double *in, float2 *out, int64_t n, cudaStream_t s
 int64_t element_ff_entries(int p, int64_t nelem);
 void launch_element_ff(int p, const double *in, float2 *out, int64_t nelem, cudaStream_t s);
 void launch_schwarz_apply(int p, const Grid3 &g, const double *r, double *z, const double *fpool64,
-                          const float *fpool32, const SchwarzPlan &plan, const int *done, cudaStream_t s);
+                          const float *fpool32, const SchwarzPlan &plan, const uint8_t *xmask, const int *done,
+                          cudaStream_t s);
 void launch_schwarz_apply_multi(int p, const double *r, double *z, int64_t nlat, int nr, const double *f64,
-                                const float *f32, const SchwarzPlan &plan, double *zb, const int *done,
-                                cudaStream_t s);
+                                const float *f32, const SchwarzPlan &plan, double *zb, const uint8_t *xmask,
+                                const int *done, cudaStream_t s);
 // columns of a GEMM tile for FP32 (prec 1) or FP64 (prec 0) factors; rows per col_items work item;
 // whether single right-hand sides stream through row_items; threads of a row_items CTA
 int schwarz_gemm_cols(int p, int prec);

@@ -43,7 +43,8 @@ struct FFAcc {
 template <int P>
 __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
     ebe_apply_ff_kernel(const double *__restrict__ x, float2 *__restrict__ zk, const float2 *__restrict__ elem,
-                        const CutCell *__restrict__ cells, Grid3 g, int64_t nc, const int *__restrict__ done)
+                        const CutCell *__restrict__ cells, Grid3 g, int64_t nc, const uint8_t *__restrict__ xmask,
+                        const int *__restrict__ done)
 {
     constexpr int Q = P + 1, NE = 3 * Q * Q * Q;
     if (done && *done) return;
@@ -51,7 +52,8 @@ __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
     const CutCell ce = cells[blockIdx.x];
     for (int t = threadIdx.x; t < NE; t += blockDim.x) {
         const int l = t / 3, ix = l % Q, iy = (l / Q) % Q, iz = l / (Q * Q);
-        xe[t] = split_ff(x[ce.base + 3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3]);
+        const int64_t at = ce.base + 3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3;
+        xe[t] = split_ff(k_input(x + at, xmask ? xmask + at : nullptr));
     }
     __syncthreads();
     const float2 *__restrict__ K = elem + (size_t)ce.elem * NE * NE;
@@ -69,8 +71,8 @@ __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
 template <int P>
 __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
     ebe_fold_ff_kernel(const double *__restrict__ x, float2 *__restrict__ zk, const float2 *__restrict__ elem,
-                       const CutCell *__restrict__ cells, Grid3 g, int64_t nc, int *err, int wait_tries,
-                       const int *__restrict__ done)
+                       const CutCell *__restrict__ cells, Grid3 g, int64_t nc, const uint8_t *__restrict__ xmask,
+                       int *err, int wait_tries, const int *__restrict__ done)
 {
     constexpr int Q = P + 1, NE = 3 * Q * Q * Q;
     if (done && *done) return;
@@ -83,7 +85,10 @@ __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
         mbar_expect(&bar, fold_entries(NE) * 8);
         bulk_g2s(m, elem + (size_t)ce.elem * fold_entries(NE), fold_entries(NE) * 8, &bar);
     }
-    if (t < NE) xe[t] = split_ff(__ldg(x + ce.base + 3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3));
+    if (t < NE) {
+        const int64_t at = ce.base + 3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3;
+        xe[t] = split_ff(k_input(x + at, xmask ? xmask + at : nullptr));
+    }
     __syncthreads();
     if (!mbar_wait(&bar, 0, wait_tries)) {
         atomicExch(err, 1);
@@ -241,7 +246,7 @@ void uncut_launch_ff(const Grid3 &g, const double *x, float2 *zk, const KCells &
 
 template <int P>
 void k_launch_ff(const Grid3 &g, const double *x, double *y, const uint8_t *mask, const float2 *elem,
-                 const KCells &kc, const int *done, cudaStream_t s, const KStreams &ks)
+                 const KCells &kc, const uint8_t *xmask, const int *done, cudaStream_t s, const KStreams &ks)
 {
     constexpr int NE = 3 * (P + 1) * (P + 1) * (P + 1);
     const int64_t nc = (int64_t)g.n[0] * g.n[1] * g.n[2];
@@ -254,10 +259,11 @@ void k_launch_ff(const Grid3 &g, const double *x, double *y, const uint8_t *mask
     }
     if (kc.n_cut > 0) {
         if constexpr (P <= 2)
-            ebe_fold_ff_kernel<P><<<kc.n_cut, ebe_threads(NE), 0, fork ? ks.side : s>>>(x, zk, elem, kc.cut, g, nc, kc.err,
-                                                                                     kc.wait_tries, done);
+            ebe_fold_ff_kernel<P><<<kc.n_cut, ebe_threads(NE), 0, fork ? ks.side : s>>>(x, zk, elem, kc.cut, g, nc, xmask,
+                                                                                     kc.err, kc.wait_tries, done);
         else
-            ebe_apply_ff_kernel<P><<<kc.n_cut, ebe_threads(NE), 0, fork ? ks.side : s>>>(x, zk, elem, kc.cut, g, nc, done);
+            ebe_apply_ff_kernel<P><<<kc.n_cut, ebe_threads(NE), 0, fork ? ks.side : s>>>(x, zk, elem, kc.cut, g, nc, xmask,
+                                                                                      done);
     }
     if (kc.n_uncut > 0) uncut_launch_ff<P>(g, x, zk, kc, done, s);
     if (fork) {
@@ -303,13 +309,13 @@ __global__ void fold_ff_pairs_kernel(const double *__restrict__ in, float2 *__re
 }  // namespace
 
 void launch_k_apply_ff(int p, const Grid3 &g, const double *x, double *y, const uint8_t *mask, const float2 *elem,
-                       const KCells &kc, const int *done, cudaStream_t s, const KStreams &ks)
+                       const KCells &kc, const uint8_t *xmask, const int *done, cudaStream_t s, const KStreams &ks)
 {
     switch (p) {
-    case 1: k_launch_ff<1>(g, x, y, mask, elem, kc, done, s, ks); break;
-    case 2: k_launch_ff<2>(g, x, y, mask, elem, kc, done, s, ks); break;
-    case 3: k_launch_ff<3>(g, x, y, mask, elem, kc, done, s, ks); break;
-    case 4: k_launch_ff<4>(g, x, y, mask, elem, kc, done, s, ks); break;
+    case 1: k_launch_ff<1>(g, x, y, mask, elem, kc, xmask, done, s, ks); break;
+    case 2: k_launch_ff<2>(g, x, y, mask, elem, kc, xmask, done, s, ks); break;
+    case 3: k_launch_ff<3>(g, x, y, mask, elem, kc, xmask, done, s, ks); break;
+    case 4: k_launch_ff<4>(g, x, y, mask, elem, kc, xmask, done, s, ks); break;
     default: break;
     }
 }

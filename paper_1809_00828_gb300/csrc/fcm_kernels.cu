@@ -29,7 +29,8 @@ __host__ __device__ constexpr int ebe_threads(int P) { return round32(ebe_rows(P
 template <int P>
 __global__ void __launch_bounds__(ebe_threads(P))
     ebe_apply_kernel(const double *__restrict__ x, double *__restrict__ zk, const double *__restrict__ elem,
-                     const CutCell *__restrict__ cells, Grid3 g, int64_t nc, const int *__restrict__ done)
+                     const CutCell *__restrict__ cells, Grid3 g, int64_t nc, const uint8_t *__restrict__ xmask,
+                     const int *__restrict__ done)
 {
     constexpr int Q = P + 1, NE = 3 * Q * Q * Q, R32 = round32(NE), PARTS = ebe_parts(P), JP = (NE + PARTS - 1) / PARTS;
     if (done && *done) return;
@@ -38,7 +39,8 @@ __global__ void __launch_bounds__(ebe_threads(P))
     const double *xc = x + ce.base;
     for (int t = threadIdx.x; t < NE; t += blockDim.x) {
         const int l = t / 3, ix = l % Q, iy = (l / Q) % Q, iz = l / (Q * Q);
-        xe[t] = xc[3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3];
+        const int64_t at = 3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3;
+        xe[t] = k_input(xc + at, xmask ? xmask + ce.base + at : nullptr);
     }
     __syncthreads();
     const int t = threadIdx.x % R32, pt = threadIdx.x / R32;
@@ -224,7 +226,7 @@ void uncut_launch(const Grid3 &g, const double *x, double *zk, const KCells &kc,
 
 template <int P>
 void k_launch(const Grid3 &g, const double *x, double *y, const uint8_t *mask, const double *elem, const KCells &kc,
-              const int *done, cudaStream_t s, const KStreams &ks)
+              const uint8_t *xmask, const int *done, cudaStream_t s, const KStreams &ks)
 {
     const int64_t nc = (int64_t)g.n[0] * g.n[1] * g.n[2];
     double *zk = reinterpret_cast<double *>(kc.zk);
@@ -234,7 +236,7 @@ void k_launch(const Grid3 &g, const double *x, double *y, const uint8_t *mask, c
         cudaStreamWaitEvent(ks.side, ks.fork, 0);
     }
     if (kc.n_cut > 0)
-        ebe_apply_kernel<P><<<kc.n_cut, ebe_threads(P), 0, fork ? ks.side : s>>>(x, zk, elem, kc.cut, g, nc, done);
+        ebe_apply_kernel<P><<<kc.n_cut, ebe_threads(P), 0, fork ? ks.side : s>>>(x, zk, elem, kc.cut, g, nc, xmask, done);
     if (kc.n_uncut > 0) uncut_launch<P>(g, x, zk, kc, done, s);
     if (fork) {
         cudaEventRecord(ks.join, ks.side);
@@ -262,13 +264,13 @@ int grid_for(int64_t n, int threads)
 }  // namespace
 
 void launch_k_apply(int p, const Grid3 &g, const double *x, double *y, const uint8_t *mask, const double *elem,
-                    const KCells &kc, const int *done, cudaStream_t s, const KStreams &ks)
+                    const KCells &kc, const uint8_t *xmask, const int *done, cudaStream_t s, const KStreams &ks)
 {
     switch (p) {
-    case 1: k_launch<1>(g, x, y, mask, elem, kc, done, s, ks); break;
-    case 2: k_launch<2>(g, x, y, mask, elem, kc, done, s, ks); break;
-    case 3: k_launch<3>(g, x, y, mask, elem, kc, done, s, ks); break;
-    case 4: k_launch<4>(g, x, y, mask, elem, kc, done, s, ks); break;
+    case 1: k_launch<1>(g, x, y, mask, elem, kc, xmask, done, s, ks); break;
+    case 2: k_launch<2>(g, x, y, mask, elem, kc, xmask, done, s, ks); break;
+    case 3: k_launch<3>(g, x, y, mask, elem, kc, xmask, done, s, ks); break;
+    case 4: k_launch<4>(g, x, y, mask, elem, kc, xmask, done, s, ks); break;
     default: break;
     }
 }

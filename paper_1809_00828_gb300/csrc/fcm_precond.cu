@@ -594,6 +594,19 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
     for (size_t f = 0; f < fac.size(); ++f)
         tc[f] = mixed && !o.simt_shared && shared[f] && prec[f] == 1 && schwarz_tc_supported(p) &&
                 fac[f].cond <= kTcCondMax;
+    // DOFs in some block, and the blocks whose box holds entries that are not free
+    std::vector<uint8_t> covered(hp.nlat, 0), block_masked(npatch, 0);
+    for (int64_t v = 0; v < npatch; ++v) {
+        if (patch_factor[v] < 0) continue;
+        const BoxInfo bx = block_box_of(rule, p, g, (int)v);
+        for (int t = 0; t < bx.n; ++t) {
+            const int nl = t / 3;
+            const int x = bx.lo[0] + nl % bx.d[0], y = bx.lo[1] + (nl / bx.d[0]) % bx.d[1], z = bx.lo[2] + nl / (bx.d[0] * bx.d[1]);
+            const int64_t l = 3 * (x + (int64_t)g.M[0] * (y + (int64_t)g.M[1] * z)) + t % 3;
+            covered[l] = 1;
+            block_masked[v] |= !hp.mask[l];
+        }
+    }
     std::vector<PatchRec> slots;
     std::vector<int> slot_of(npatch, -1);
     std::vector<int2> tiles32, tiles64;
@@ -609,7 +622,7 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
             const int first = (int)slots.size();
             for (int v : blocks_of[f]) {
                 slot_of[v] = (int)slots.size();
-                slots.push_back({off[f], v, prec[f]});
+                slots.push_back({off[f], v, prec[f] | (block_masked[v] ? kMaskedBlock : 0)});
             }
             const int cnt = (int)blocks_of[f].size();
             for (int s0 = 0; s0 < cnt; s0 += nc) (want == 1 ? tiles32 : tiles64).push_back(make_int2(first + s0, std::min(nc, cnt - s0)));
@@ -645,11 +658,12 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
             if (folded[f]) {
                 const BoxInfo bx = block_box_of(rule, p, g, v);
                 fold_items[prec[f]].push_back({off[f], 3 * (bx.lo[0] + (int64_t)g.M[0] * (bx.lo[1] + (int64_t)g.M[1] * bx.lo[2])),
-                                               (int)slots.size(), {bx.d[0], bx.d[1], bx.d[2]}});
+                                               block_masked[v] ? ~(int)slots.size() : (int)slots.size(),
+                                               {bx.d[0], bx.d[1], bx.d[2]}});
             } else {
                 own_slots[prec[f]].push_back((int)slots.size());
             }
-            slots.push_back({off[f], v, prec[f]});
+            slots.push_back({off[f], v, prec[f] | (block_masked[v] ? kMaskedBlock : 0)});
         }
     }
     const int n_fold32 = (int)fold_items[1].size(), n_fold_ff = (int)fold_items[2].size();
@@ -735,7 +749,7 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
     // the pair format stores FP32 slots as floats: their slot_of entries carry the flag the sum kernel reads
     if (mixed)
         for (int64_t v = 0; v < npatch; ++v)
-            if (slot_of[v] >= 0 && slots[slot_of[v]].prec == 1) slot_of[v] |= 1 << 30;
+            if (slot_of[v] >= 0 && (slots[slot_of[v]].prec & (kMaskedBlock - 1)) == 1) slot_of[v] |= 1 << 30;
     PC_CUDA(cudaMemcpyAsync(C->d_slot_of, slot_of.data(), sizeof(int) * slot_of.size(), cudaMemcpyHostToDevice, st));
     int2 *d_col = C->d_items + max_rows_items, *d_tiles = d_col + col_items.size();
     PC_CUDA(cudaMemcpyAsync(d_col, col_items.data(), sizeof(int2) * col_items.size(), cudaMemcpyHostToDevice, st));
@@ -793,16 +807,6 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
         return cudaSuccess;
     };
     // ---- Algorithm 1's diagonal part: 1 / K_ll for the free DOFs in no block
-    std::vector<uint8_t> covered(hp.nlat, 0);
-    for (int64_t v = 0; v < npatch; ++v) {
-        if (patch_factor[v] < 0) continue;
-        const BoxInfo bx = block_box_of(rule, p, g, (int)v);
-        for (int t = 0; t < bx.n; ++t) {
-            const int nl = t / 3;
-            const int x = bx.lo[0] + nl % bx.d[0], y = bx.lo[1] + (nl / bx.d[0]) % bx.d[1], z = bx.lo[2] + nl / (bx.d[0] * bx.d[1]);
-            covered[3 * (x + (int64_t)g.M[0] * (y + (int64_t)g.M[1] * z)) + t % 3] = 1;
-        }
-    }
     int64_t nuncovered = 0;
     for (int64_t l = 0; l < hp.nlat; ++l) nuncovered += hp.mask[l] && !covered[l];
     if (C->d_jac) cudaFree(C->d_jac);
@@ -835,9 +839,9 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o)
                 fail = "autotune upload";
                 break;
             }
-            for (int w = 0; w < 2; ++w) launch_schwarz_apply(p, g, C->d_rhs, C->d_z, C->d_f64, C->d_f32, plan, nullptr, st);
+            for (int w = 0; w < 2; ++w) launch_schwarz_apply(p, g, C->d_rhs, C->d_z, C->d_f64, C->d_f32, plan, nullptr, nullptr, st);
             cudaEventRecord(e0, st);
-            for (int w = 0; w < 5; ++w) launch_schwarz_apply(p, g, C->d_rhs, C->d_z, C->d_f64, C->d_f32, plan, nullptr, st);
+            for (int w = 0; w < 5; ++w) launch_schwarz_apply(p, g, C->d_rhs, C->d_z, C->d_f64, C->d_f32, plan, nullptr, nullptr, st);
             cudaEventRecord(e1, st);
             if (cudaEventSynchronize(e1) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
                 fail = "autotune run";

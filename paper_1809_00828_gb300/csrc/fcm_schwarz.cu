@@ -68,6 +68,15 @@ __device__ __forceinline__ SBox sbox(int rule, int P, const Grid3 &g, int id)
     return b;
 }
 
+// r[i], 0 where the mask m (may be null) says the entry is not free
+__device__ __forceinline__ double masked(const double *__restrict__ r, const uint8_t *__restrict__ m, int64_t i)
+{
+    const double v = __ldg(r + i);  // without a branch: loads of a loop stay in flight together
+    return m && !m[i] ? 0.0 : v;
+}
+
+__device__ __forceinline__ int fold_slot(const FoldItem &it) { return it.slot < 0 ? ~it.slot : it.slot; }
+
 // offset of box entry t from the box's first lattice DOF
 __device__ __forceinline__ int box_rel(const SBox &b, const Grid3 &g, int t)
 {
@@ -134,7 +143,8 @@ constexpr int kRowsThreads = 256;
 
 // rows [row0, row0 + rows) of Zb = F r_B, F in T (FP32 or FP64), rows of ld entries padded to 16 bytes
 template <int P, typename T>
-__device__ __forceinline__ void rows_plain(const double *__restrict__ r, const T *__restrict__ F, const SBox &b,
+__device__ __forceinline__ void rows_plain(const double *__restrict__ r, const uint8_t *__restrict__ xm,
+                                           const T *__restrict__ F, const SBox &b,
                                            const Grid3 &g, int row0, int rows, double *__restrict__ zout,
                                            bool pairs, unsigned char *smem)
 {
@@ -145,7 +155,7 @@ __device__ __forceinline__ void rows_plain(const double *__restrict__ r, const T
     T *rb = reinterpret_cast<T *>(smem);
     const int n = b.n, ld = factor_ld<T>(n), nv = ld / V;
     const int64_t base = box_base(b, g);
-    for (int t = threadIdx.x; t < ld; t += blockDim.x) rb[t] = t < n ? gathered<T>(r[base + box_rel(b, g, t)]) : (T)0;
+    for (int t = threadIdx.x; t < ld; t += blockDim.x) rb[t] = t < n ? gathered<T>(masked(r, xm, base + box_rel(b, g, t))) : (T)0;
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     VT xr[KV];
@@ -184,7 +194,8 @@ __device__ __forceinline__ void rows_plain(const double *__restrict__ r, const T
 
 // the same for a double-float factor: entry j of a row is the float pair at 2j, 2j+1
 template <int P>
-__device__ __forceinline__ void rows_ff(const double *__restrict__ r, const float *__restrict__ F, const SBox &b,
+__device__ __forceinline__ void rows_ff(const double *__restrict__ r, const uint8_t *__restrict__ xm,
+                                        const float *__restrict__ F, const SBox &b,
                                         const Grid3 &g, int row0, int rows, double *__restrict__ zout, bool pairs,
                                         unsigned char *smem)
 {
@@ -194,7 +205,7 @@ __device__ __forceinline__ void rows_ff(const double *__restrict__ r, const floa
     const int n = b.n, ld = factor_ld<double>(n), nv = ld / 2;
     const int64_t base = box_base(b, g);
     for (int t = threadIdx.x; t < ld; t += blockDim.x)
-        rb[t] = t < n ? split_ff(r[base + box_rel(b, g, t)]) : make_float2(0.f, 0.f);
+        rb[t] = t < n ? split_ff(masked(r, xm, base + box_rel(b, g, t))) : make_float2(0.f, 0.f);
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     float4 xr[KV];
@@ -248,7 +259,8 @@ template <int P>
 __global__ void __launch_bounds__(kRowsThreads)
     schwarz_rows_kernel(const double *__restrict__ r, const double *__restrict__ f64, const float *__restrict__ f32,
                         const PatchRec *__restrict__ slots, const int2 *__restrict__ items, int rows, Grid3 g, int rule,
-                        double *__restrict__ zb, int zs, int pairs, const int *__restrict__ done)
+                        double *__restrict__ zb, int zs, int pairs, const uint8_t *__restrict__ xmask,
+                        const int *__restrict__ done)
 {
     __shared__ __align__(16) double smem_d[factor_ld<double>(sbox_max(P))];
     if (done && *done) return;
@@ -257,9 +269,11 @@ __global__ void __launch_bounds__(kRowsThreads)
     const PatchRec pr = slots[it.x];
     const SBox b = sbox(rule, P, g, pr.v);
     double *zout = zb + (size_t)it.x * zs;
-    if (pr.prec == 1) rows_plain<P, float>(r, f32 + pr.off, b, g, it.y, rows, zout, pairs, smem);
-    else if (pr.prec == 2) rows_ff<P>(r, f32 + pr.off, b, g, it.y, rows, zout, pairs, smem);
-    else rows_plain<P, double>(r, f64 + pr.off, b, g, it.y, rows, zout, pairs, smem);
+    const uint8_t *xm = pr.prec & kMaskedBlock ? xmask : nullptr;
+    const int prec = pr.prec & (kMaskedBlock - 1);
+    if (prec == 1) rows_plain<P, float>(r, xm, f32 + pr.off, b, g, it.y, rows, zout, pairs, smem);
+    else if (prec == 2) rows_ff<P>(r, xm, f32 + pr.off, b, g, it.y, rows, zout, pairs, smem);
+    else rows_plain<P, double>(r, xm, f64 + pr.off, b, g, it.y, rows, zout, pairs, smem);
 }
 
 // ---- phase 1b: own factors, a thread per row (small blocks; several right-hand sides)
@@ -272,7 +286,8 @@ __global__ void __launch_bounds__(kRowsThreads)
 __host__ __device__ constexpr int cols_threads(int P) { return P >= 3 ? 128 : rnd32(sbox_max(P)); }
 
 template <int P, int NR, typename T>
-__device__ __forceinline__ void cols_plain(const double *__restrict__ r, int64_t nlat, int nr, const T *__restrict__ F,
+__device__ __forceinline__ void cols_plain(const double *__restrict__ r, const uint8_t *__restrict__ xm, int64_t nlat,
+                                           int nr, const T *__restrict__ F,
                                            const SBox &b, const Grid3 &g, int row0, double *__restrict__ zout,
                                            int64_t zsize, bool pairs, unsigned char *smem)
 {
@@ -281,7 +296,7 @@ __device__ __forceinline__ void cols_plain(const double *__restrict__ r, int64_t
     const int64_t base = box_base(b, g);
     for (int e = threadIdx.x; e < n * NR; e += blockDim.x) {
         const int t = e / NR, k = e % NR;
-        rbT[t][k] = k < nr ? gathered<T>(r[(int64_t)k * nlat + base + box_rel(b, g, t)]) : (T)0;
+        rbT[t][k] = k < nr ? gathered<T>(masked(r + (int64_t)k * nlat, xm, base + box_rel(b, g, t))) : (T)0;
     }
     __syncthreads();
     const int row = row0 + threadIdx.x;
@@ -302,7 +317,8 @@ __device__ __forceinline__ void cols_plain(const double *__restrict__ r, int64_t
 }
 
 template <int P, int NR>
-__device__ __forceinline__ void cols_ff(const double *__restrict__ r, int64_t nlat, int nr, const float *__restrict__ F,
+__device__ __forceinline__ void cols_ff(const double *__restrict__ r, const uint8_t *__restrict__ xm, int64_t nlat,
+                                        int nr, const float *__restrict__ F,
                                         const SBox &b, const Grid3 &g, int row0, double *__restrict__ zout, int64_t zsize,
                                         bool pairs, unsigned char *smem)
 {
@@ -311,7 +327,7 @@ __device__ __forceinline__ void cols_ff(const double *__restrict__ r, int64_t nl
     const int64_t base = box_base(b, g);
     for (int e = threadIdx.x; e < n * NR; e += blockDim.x) {
         const int t = e / NR, k = e % NR;
-        rbT[t][k] = k < nr ? split_ff(r[(int64_t)k * nlat + base + box_rel(b, g, t)]) : make_float2(0.f, 0.f);
+        rbT[t][k] = k < nr ? split_ff(masked(r + (int64_t)k * nlat, xm, base + box_rel(b, g, t))) : make_float2(0.f, 0.f);
     }
     __syncthreads();
     const int row = row0 + threadIdx.x;
@@ -336,7 +352,7 @@ __global__ void __launch_bounds__(cols_threads(P))
     schwarz_cols_kernel(const double *__restrict__ r, int64_t nlat, int nr, const double *__restrict__ f64,
                         const float *__restrict__ f32, const PatchRec *__restrict__ slots,
                         const int2 *__restrict__ items, Grid3 g, int rule, double *__restrict__ zb, int zs,
-                        int64_t zsize, int pairs, const int *__restrict__ done)
+                        int64_t zsize, int pairs, const uint8_t *__restrict__ xmask, const int *__restrict__ done)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     if (done && *done) return;
@@ -344,9 +360,11 @@ __global__ void __launch_bounds__(cols_threads(P))
     const PatchRec pr = slots[it.x];
     const SBox b = sbox(rule, P, g, pr.v);
     double *zout = zb + (size_t)it.x * zs;
-    if (pr.prec == 1) cols_plain<P, NR, float>(r, nlat, nr, f32 + pr.off, b, g, it.y, zout, zsize, pairs, smem);
-    else if (pr.prec == 2) cols_ff<P, NR>(r, nlat, nr, f32 + pr.off, b, g, it.y, zout, zsize, pairs, smem);
-    else cols_plain<P, NR, double>(r, nlat, nr, f64 + pr.off, b, g, it.y, zout, zsize, pairs, smem);
+    const uint8_t *xm = pr.prec & kMaskedBlock ? xmask : nullptr;
+    const int prec = pr.prec & (kMaskedBlock - 1);
+    if (prec == 1) cols_plain<P, NR, float>(r, xm, nlat, nr, f32 + pr.off, b, g, it.y, zout, zsize, pairs, smem);
+    else if (prec == 2) cols_ff<P, NR>(r, xm, nlat, nr, f32 + pr.off, b, g, it.y, zout, zsize, pairs, smem);
+    else cols_plain<P, NR, double>(r, xm, nlat, nr, f64 + pr.off, b, g, it.y, zout, zsize, pairs, smem);
 }
 
 // ---- phase 1b': own FP32 and double-float factors of small blocks (p <= 2), folded (fcm_sym.cuh)
@@ -361,7 +379,8 @@ template <int P, int NR, class T>
 __global__ void __launch_bounds__(fold_threads(P))
     schwarz_fold_kernel(const double *__restrict__ r, int64_t nlat, int nr, const float *__restrict__ f32,
                         const FoldItem *__restrict__ items, Grid3 g, double *__restrict__ zb, int zs, int64_t zsize,
-                        int pairs, int *err, int wait_tries, const int *__restrict__ done)
+                        int pairs, const uint8_t *__restrict__ xmask, int *err, int wait_tries,
+                        const int *__restrict__ done)
 {
     constexpr int NM = sbox_max(P);
     if (done && *done) return;
@@ -387,10 +406,11 @@ __global__ void __launch_bounds__(fold_threads(P))
             iy = (l / it.d[0]) % it.d[1];
             iz = l / (it.d[0] * it.d[1]);
         }
-        const double *rt = r + it.base + 3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3;
+        const int64_t at = it.base + 3 * (ix + g.M[0] * (iy + (int64_t)g.M[1] * iz)) + t % 3;
+        const bool on = !(xmask && it.slot < 0) || xmask[at];
 #pragma unroll
         for (int k = 0; k < NR; ++k) {
-            const double v = k < nr ? __ldg(rt + k * nlat) : 0.0;
+            const double v = k < nr && on ? __ldg(r + at + k * nlat) : 0.0;
             if constexpr (sizeof(T) == 4) xs[t * NR + k] = to_f32(v);
             else xs[t * NR + k] = split_ff(v);
         }
@@ -404,7 +424,7 @@ __global__ void __launch_bounds__(fold_threads(P))
     const int t0 = threadIdx.x & ~31;
     if (t0 >= n) return;
     const int row = threadIdx.x, t = min(row, n - 1);
-    double *zout = zb + (size_t)it.slot * zs;
+    double *zout = zb + (size_t)fold_slot(it) * zs;
     if constexpr (sizeof(T) == 4) {
         float acc[NR];
 #pragma unroll
@@ -511,8 +531,8 @@ template <int P, typename T>
 __global__ void __launch_bounds__(gemm_threads(P))
     schwarz_gemm_kernel(const double *__restrict__ r, int64_t nlat, int nr, const T *__restrict__ pool,
                         const PatchRec *__restrict__ slots, const int2 *__restrict__ tiles, Grid3 g, int rule,
-                        double *__restrict__ zb, int zs, int64_t zsize, int pairs, int *err, int wait_tries,
-                        const int *__restrict__ done)
+                        double *__restrict__ zb, int zs, int64_t zsize, int pairs, const uint8_t *__restrict__ xmask,
+                        int *err, int wait_tries, const int *__restrict__ done)
 {
     constexpr int NC = GemmCfg<T, P>::NC, KC = GemmCfg<T, P>::KC, CPT = NC / 8, HALF = CPT / 2;
     constexpr int SE = gemm_stage_elems<P, T>();
@@ -574,7 +594,9 @@ __global__ void __launch_bounds__(gemm_threads(P))
         for (int e = tid; e < n * NC; e += blockDim.x) {
             const int t = e / NC, c = e % NC;
             const int64_t s = src[c];
-            panel[e] = s >= 0 ? gathered<T>(r[s + rel[t]]) : (T)0;
+            double v = s >= 0 ? r[s + rel[t]] : 0.0;
+            if (xmask && s >= 0 && !xmask[s + rel[t] - (int64_t)(c % nr) * nlat]) v = 0.0;
+            panel[e] = gathered<T>(v);
         }
         __syncthreads();
         for (int pass = 0; pass < passes; ++pass) {
@@ -831,7 +853,7 @@ template <int P>
 __global__ void __launch_bounds__(TcCfg<P>::THREADS, TcCfg<P>::CTAS_PER_SM)
     tc_gemm_kernel(const double *__restrict__ r, const PatchRec *__restrict__ slots, const TcTile *__restrict__ tiles,
                    Grid3 g, int rule, const float *__restrict__ ft, double *__restrict__ zb, int zs, int pairs,
-                   int *err, int wait_tries, const int *__restrict__ done)
+                   const uint8_t *__restrict__ xmask, int *err, int wait_tries, const int *__restrict__ done)
 {
     using Cfg = TcCfg<P>;
     constexpr int S = Cfg::STAGES;
@@ -925,6 +947,7 @@ __global__ void __launch_bounds__(TcCfg<P>::THREADS, TcCfg<P>::CTAS_PER_SM)
         // producers: column m, K values 8 kh .. 8 kh + 7 of each chunk
         const int p = threadIdx.x - 32, m = p & 127, kh = p >> 7;
         const int64_t bm = base[m];
+        const uint8_t *xm = xmask && bm >= 0 && slots[tl.first + m].prec & kMaskedBlock ? xmask : nullptr;
         double cur[8], nxt[8];
         auto load = [&](int c, double *v) {
 #pragma unroll
@@ -933,6 +956,12 @@ __global__ void __launch_bounds__(TcCfg<P>::THREADS, TcCfg<P>::CTAS_PER_SM)
                 const int rk = k < Cfg::NRP ? rel[k] : -1;
                 v[i] = (bm >= 0 && rk >= 0) ? r[bm + rk] : 0.0;
             }
+            if (xm)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int k = 16 * c + 8 * kh + i, rk = k < Cfg::NRP ? rel[k] : -1;
+                    if (rk >= 0 && !xm[bm + rk]) v[i] = 0.0;
+                }
         };
         load(0, cur);
         for (int c = 0; c < nch; ++c) {
@@ -999,7 +1028,7 @@ dim3 sum_grid(const Grid3 &g) { return dim3((g.M[0] + 31) / 32, (g.M[1] + 7) / 8
 
 template <int P>
 void gemm_launch(const double *r, int64_t nlat, int nr, const double *f64, const float *f32, const SchwarzPlan &pl,
-                 double *zb, int64_t zsize, const int *done, cudaStream_t s)
+                 double *zb, int64_t zsize, const uint8_t *xm, const int *done, cudaStream_t s)
 {
     const Grid3 &g = pl.g;
     // one right-hand side: the FP32 shared factors that have tensor-core tiles go through tcgen05
@@ -1007,15 +1036,15 @@ void gemm_launch(const double *r, int64_t nlat, int nr, const double *f64, const
     if constexpr (P == 2 || P == 3) {
         if (tc)
             tc_gemm_kernel<P><<<pl.n_tc_tiles, TcCfg<P>::THREADS, TcCfg<P>::SMEM, s>>>(
-                r, pl.slots, pl.tc_tiles, g, pl.rule, pl.tc_ft, zb, pl.zs, pl.pairs, pl.err, pl.wait_tries, done);
+                r, pl.slots, pl.tc_tiles, g, pl.rule, pl.tc_ft, zb, pl.zs, pl.pairs, xm, pl.err, pl.wait_tries, done);
     }
     const int n32 = tc ? pl.n_tiles32_plain : pl.n_tiles32;
     if (n32 > 0)
         schwarz_gemm_kernel<P, float><<<n32, gemm_threads(P), gemm_smem_bytes<P, float>(), s>>>(
-            r, nlat, nr, f32, pl.slots, pl.tiles, g, pl.rule, zb, pl.zs, zsize, pl.pairs, pl.err, pl.wait_tries, done);
+            r, nlat, nr, f32, pl.slots, pl.tiles, g, pl.rule, zb, pl.zs, zsize, pl.pairs, xm, pl.err, pl.wait_tries, done);
     if (pl.n_tiles64 > 0)
         schwarz_gemm_kernel<P, double><<<pl.n_tiles64, gemm_threads(P), gemm_smem_bytes<P, double>(), s>>>(
-            r, nlat, nr, f64, pl.slots, pl.tiles + pl.n_tiles32, g, pl.rule, zb, pl.zs, zsize, pl.pairs, pl.err,
+            r, nlat, nr, f64, pl.slots, pl.tiles + pl.n_tiles32, g, pl.rule, zb, pl.zs, zsize, pl.pairs, xm, pl.err,
             pl.wait_tries, done);
 }
 
@@ -1034,29 +1063,29 @@ void with_columns(int nr, F &&f)
 
 template <int P, int NR>
 void cols_launch(const double *r, int64_t nlat, int nr, const double *f64, const float *f32, const SchwarzPlan &pl,
-                 double *zb, int64_t zsize, const int *done, cudaStream_t s)
+                 double *zb, int64_t zsize, const uint8_t *xm, const int *done, cudaStream_t s)
 {
     const int smem = factor_ld<double>(sbox_max(P)) * NR * 8;
     schwarz_cols_kernel<P, NR><<<pl.n_col_items, cols_threads(P), smem, s>>>(
-        r, nlat, nr, f64, f32, pl.slots, pl.col_items, pl.g, pl.rule, zb, pl.zs, zsize, pl.pairs, done);
+        r, nlat, nr, f64, f32, pl.slots, pl.col_items, pl.g, pl.rule, zb, pl.zs, zsize, pl.pairs, xm, done);
 }
 
 template <int P, int NR>
 void fold_launch(const double *r, int64_t nlat, int nr, const float *f32, const SchwarzPlan &pl, double *zb,
-                 int64_t zsize, const int *done, cudaStream_t s)
+                 int64_t zsize, const uint8_t *xm, const int *done, cudaStream_t s)
 {
     if (pl.n_fold32 > 0)
         schwarz_fold_kernel<P, NR, float><<<pl.n_fold32, fold_threads(P), 0, s>>>(
-            r, nlat, nr, f32, pl.fold_items, pl.g, zb, pl.zs, zsize, pl.pairs, pl.err, pl.wait_tries, done);
+            r, nlat, nr, f32, pl.fold_items, pl.g, zb, pl.zs, zsize, pl.pairs, xm, pl.err, pl.wait_tries, done);
     if (pl.n_fold_ff > 0)
         schwarz_fold_kernel<P, NR, float2><<<pl.n_fold_ff, fold_threads(P), 0, s>>>(
-            r, nlat, nr, f32, pl.fold_items + pl.n_fold32, pl.g, zb, pl.zs, zsize, pl.pairs, pl.err, pl.wait_tries,
+            r, nlat, nr, f32, pl.fold_items + pl.n_fold32, pl.g, zb, pl.zs, zsize, pl.pairs, xm, pl.err, pl.wait_tries,
             done);
 }
 
 template <int P>
 void apply_p(const double *r, double *z, int64_t nlat, int nr, const double *f64, const float *f32,
-             const SchwarzPlan &pl, double *zb, const int *done, cudaStream_t s)
+             const SchwarzPlan &pl, double *zb, const uint8_t *xm, const int *done, cudaStream_t s)
 {
     const int64_t zsize = (int64_t)pl.nslots * pl.zs;
     const bool gemm = pl.n_tiles32 + pl.n_tiles64 + (nr == 1 ? pl.n_tc_tiles : 0) > 0;
@@ -1066,21 +1095,21 @@ void apply_p(const double *r, double *z, int64_t nlat, int nr, const double *f64
         // the shared-factor products on the second stream, beside the streamed factors
         cudaEventRecord(pl.ev_fork, s);
         cudaStreamWaitEvent(pl.side, pl.ev_fork, 0);
-        gemm_launch<P>(r, nlat, nr, f64, f32, pl, zb, zsize, done, pl.side);
+        gemm_launch<P>(r, nlat, nr, f64, f32, pl, zb, zsize, xm, done, pl.side);
         cudaEventRecord(pl.ev_join, pl.side);
     } else if (gemm) {
-        gemm_launch<P>(r, nlat, nr, f64, f32, pl, zb, zsize, done, s);
+        gemm_launch<P>(r, nlat, nr, f64, f32, pl, zb, zsize, xm, done, s);
     }
     if constexpr (P <= 2)
-        with_columns(nr, [&](auto c) { fold_launch<P, decltype(c)::value>(r, nlat, nr, f32, pl, zb, zsize, done, s); });
+        with_columns(nr, [&](auto c) { fold_launch<P, decltype(c)::value>(r, nlat, nr, f32, pl, zb, zsize, xm, done, s); });
     if (own) {
         if (P == 3 && nr == 1) {
             if constexpr (P == 3)
                 schwarz_rows_kernel<P><<<pl.n_row_items, kRowsThreads, 0, s>>>(
-                    r, f64, f32, pl.slots, pl.row_items, pl.rows, pl.g, pl.rule, zb, pl.zs, pl.pairs, done);
+                    r, f64, f32, pl.slots, pl.row_items, pl.rows, pl.g, pl.rule, zb, pl.zs, pl.pairs, xm, done);
         } else {
             with_columns(nr, [&](auto c) {
-                cols_launch<P, decltype(c)::value>(r, nlat, nr, f64, f32, pl, zb, zsize, done, s);
+                cols_launch<P, decltype(c)::value>(r, nlat, nr, f64, f32, pl, zb, zsize, xm, done, s);
             });
         }
     }
@@ -1186,22 +1215,23 @@ cudaError_t schwarz_prepare(int p)
 }
 
 void launch_schwarz_apply_multi(int p, const double *r, double *z, int64_t nlat, int nr, const double *f64,
-                                const float *f32, const SchwarzPlan &plan, double *zb, const int *done, cudaStream_t s)
+                                const float *f32, const SchwarzPlan &plan, double *zb, const uint8_t *xmask,
+                                const int *done, cudaStream_t s)
 {
     switch (p) {
-    case 1: apply_p<1>(r, z, nlat, nr, f64, f32, plan, zb, done, s); break;
-    case 2: apply_p<2>(r, z, nlat, nr, f64, f32, plan, zb, done, s); break;
-    case 3: apply_p<3>(r, z, nlat, nr, f64, f32, plan, zb, done, s); break;
-    case 4: apply_p<4>(r, z, nlat, nr, f64, f32, plan, zb, done, s); break;
+    case 1: apply_p<1>(r, z, nlat, nr, f64, f32, plan, zb, xmask, done, s); break;
+    case 2: apply_p<2>(r, z, nlat, nr, f64, f32, plan, zb, xmask, done, s); break;
+    case 3: apply_p<3>(r, z, nlat, nr, f64, f32, plan, zb, xmask, done, s); break;
+    case 4: apply_p<4>(r, z, nlat, nr, f64, f32, plan, zb, xmask, done, s); break;
     default: break;
     }
 }
 
 void launch_schwarz_apply(int p, const Grid3 &g, const double *r, double *z, const double *f64, const float *f32,
-                          const SchwarzPlan &plan, const int *done, cudaStream_t s)
+                          const SchwarzPlan &plan, const uint8_t *xmask, const int *done, cudaStream_t s)
 {
     const int64_t nlat = 3 * (int64_t)g.M[0] * g.M[1] * g.M[2];
-    launch_schwarz_apply_multi(p, r, z, nlat, 1, f64, f32, plan, plan.zb, done, s);
+    launch_schwarz_apply_multi(p, r, z, nlat, 1, f64, f32, plan, plan.zb, xmask, done, s);
 }
 
 }  // namespace fcm
