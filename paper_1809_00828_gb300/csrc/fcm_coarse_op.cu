@@ -505,39 +505,43 @@ __global__ void __launch_bounds__(RT) mg_interp_kernel(const float *__restrict__
     }
 }
 
-// fc = P2^T rf, one thread per coarse cell (up to 4 fine cells per axis)
+// fc = P2^T rf, one thread per coarse cell (up to 4 fine cells per axis).  The weights are made first and the
+// 192 loads carry no branches (cells of weight 0 read the cell 2 J, in bounds), so a plane's 48 are in flight
+// together (four levels from 80^3 cells: 33 us; with a test before each load, a chain of latencies, 64).
 __global__ void __launch_bounds__(RT) mg_restrict_kernel(const float *__restrict__ rf, float *__restrict__ fc, LvDims d,
                                                           const int *stop)
 {
     STOP_RETURN;
     for (int64_t q = blockIdx.x * (int64_t)RT + threadIdx.x; q < d.ncc; q += (int64_t)gridDim.x * RT) {
         const int J[3] = {(int)(q % d.nc[0]), (int)((q / d.nc[0]) % d.nc[1]), (int)(q / ((int64_t)d.nc[0] * d.nc[1]))};
-        int lo[3], cnt[3];
+        int at[3][4];
+        float w[3][4];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = d.f[a] == 1 ? J[a] : 2 * J[a] - 1;
-            cnt[a] = d.f[a] == 1 ? 1 : 4;
-        }
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = d.f[a] == 1 ? J[a] + k : 2 * J[a] - 1 + k;
+                const bool on = (d.f[a] != 1 || k == 0) && i >= 0 && i < d.nf[a];
+                w[a][k] = on ? axis_w(i, J[a], d.nc[a], d.f[a]) : 0.f;
+                at[a][k] = on ? i : d.f[a] * J[a];
+            }
         float acc[3] = {0.f, 0.f, 0.f};
-        for (int kz = 0; kz < cnt[2]; ++kz) {
-            const int iz = lo[2] + kz;
-            if (iz < 0 || iz >= d.nf[2]) continue;
-            const float wz = axis_w(iz, J[2], d.nc[2], d.f[2]);
-            if (wz == 0.f) continue;
-            for (int ky = 0; ky < cnt[1]; ++ky) {
-                const int iy = lo[1] + ky;
-                if (iy < 0 || iy >= d.nf[1]) continue;
-                const float wy = wz * axis_w(iy, J[1], d.nc[1], d.f[1]);
-                if (wy == 0.f) continue;
-                for (int kx = 0; kx < cnt[0]; ++kx) {
-                    const int ix = lo[0] + kx;
-                    if (ix < 0 || ix >= d.nf[0]) continue;
-                    const float wt = wy * axis_w(ix, J[0], d.nc[0], d.f[0]);
-                    if (wt == 0.f) continue;
-                    const int64_t c = ix + (int64_t)d.nf[0] * (iy + (int64_t)d.nf[1] * iz);
+#pragma unroll 1
+        for (int kz = 0; kz < 4; ++kz) {
+            const float wz = kz == 0 ? w[2][0] : kz == 1 ? w[2][1] : kz == 2 ? w[2][2] : w[2][3];
+            const int iz = kz == 0 ? at[2][0] : kz == 1 ? at[2][1] : kz == 2 ? at[2][2] : at[2][3];
+            float v[16][3];
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) acc[a] = fmaf(wt, rf[a * d.ncf + c], acc[a]);
-                }
+            for (int k = 0; k < 16; ++k) {
+                const int64_t c = at[0][k & 3] + (int64_t)d.nf[0] * (at[1][k >> 2] + (int64_t)d.nf[1] * iz);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) v[k][a] = __ldg(rf + a * d.ncf + c);
+            }
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const float wt = wz * w[1][k >> 2] * w[0][k & 3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) acc[a] = wt != 0.f ? fmaf(wt, v[k][a], acc[a]) : acc[a];
             }
         }
 #pragma unroll
