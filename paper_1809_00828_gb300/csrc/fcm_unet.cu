@@ -35,7 +35,7 @@ namespace {
 // twice.  A halo plane goes through the taps of up to three output planes in one product (N up to 3 x the
 // columns: the accumulators of the tile's planes lie side by side), since one thread issues the products at a
 // rate that does not depend on N: 27 (ZT + 2) of them per 16 input channels instead of 81 ZT.  Forward pass on
-// 80^3 cells, channels 16 to 64 (75 GFLOP of convolutions): 0.90 ms; 1.19 ms with a product per plane, and
+// 80^3 cells, channels 16 to 64 (75 GFLOP of convolutions): 0.85 ms; 1.19 ms with a product per plane, and
 // 5.76 ms with FP32 arithmetic on the CUDA cores (13 TFLOP/s).  Two CTAs per SM overlap one's halo loads with
 // the other's products.
 //
@@ -294,7 +294,7 @@ __global__ void conv_tiles_kernel(const __nv_bfloat16 *__restrict__ w, __nv_bflo
 // cost 19 reads for 112).  The tiles are dealt to enough CTAs to fill the GPU, each
 // writes its sums to `part`, and wgrad_sum_kernel adds them in a fixed order in FP64 (deterministic).  One CTA per
 // (co, ci) pair with 27 unshared global reads per multiply-add row took 4.9 ms for the gradients of the
-// 16-to-64-channel network on four 32^3 cubes, one channel a thread 1.08 + 0.29 ms; this 1.00 + 0.12 ms.
+// 16-to-64-channel network on four 32^3 cubes, one channel a thread 1.08 + 0.29 ms; this 0.90 + 0.12 ms.
 constexpr int kWC = 8, kWO = 16, kWX = 8, kWY = 8, kWZ = 4, kWGo = kWX * kWY * kWZ + 4;
 constexpr int kWRow = 12, kWPlane = kWRow * (kWY + 2), kWCh = kWPlane * (kWZ + 2) + 4;  // 4 channels: distinct banks
 constexpr int kWTaps = 28;
@@ -316,6 +316,7 @@ __global__ void __launch_bounds__(256, 2)
         const int b = (int)(tile / ((int64_t)tx * ty * tz)), q = (int)(tile % ((int64_t)tx * ty * tz));
         const int x0 = q % tx * kWX, y0 = q / tx % ty * kWY, z0 = q / (tx * ty) * kWZ;
         __syncthreads();
+#pragma unroll 10  // that many loads in flight
         for (int e = tid; e < kWC * (kWZ + 2) * (kWY + 2) * (kWX + 2); e += 256) {
             const int hx = e % (kWX + 2), hy = e / (kWX + 2) % (kWY + 2), hz = e / ((kWX + 2) * (kWY + 2)) % (kWZ + 2),
                       c = e / ((kWX + 2) * (kWY + 2) * (kWZ + 2));
@@ -323,6 +324,7 @@ __global__ void __launch_bounds__(256, 2)
             const bool on = ci0 + c < cin && x >= 0 && y >= 0 && z >= 0 && x < nx && y < ny && z < nz;
             si[c * kWCh + hz * kWPlane + hy * kWRow + hx] = on ? conv_load(in, b, ci0 + c, x, y, z, nx, ny, nz) : 0.f;
         }
+#pragma unroll 8
         for (int e = tid; e < kWO * kWX * kWY * kWZ; e += 256) {
             const int v = e % (kWX * kWY * kWZ), c = e / (kWX * kWY * kWZ);
             const int x = x0 + v % kWX, y = y0 + v / kWX % kWY, z = z0 + v / (kWX * kWY);
@@ -607,9 +609,13 @@ void conv_launch(fcm_unet *N, const ConvSrc &src, int64_t tiles, const float *bi
     const uint4 *w = reinterpret_cast<const uint4 *>(N->tiles + tiles);
     // More planes per CTA take fewer products and halo voxels per output (27 (ZT + 2) and 1.4 (ZT + 2), over ZT);
     // with 16 columns three and with 32 two still leave room for two CTAs per SM (256 of 512 tensor-memory columns
-    // each), and a small grid has too few of them.
+    // each).  The choice is the least number of waves of 304 CTAs times ZT + 2 (40^3 cells, 32 channels: two planes
+    // are one wave, one plane two).
     const auto ctas = [&](int zt) { return txy * ((nz + zt - 1) / zt) * N->B * conv_blocks(cout); };
-    const int zt = nb == 16 && ctas(3) >= 304 ? 3 : nb <= 32 && ctas(2) >= 304 ? 2 : 1;
+    const auto cost = [&](int zt) { return (ctas(zt) + 303) / 304 * (zt + 2); };
+    int zt = 1;
+    for (int k = 2; k <= (nb == 16 ? 3 : nb <= 32 ? 2 : 1); ++k)
+        if (cost(k) < cost(zt)) zt = k;
     const auto kernel = zt == 3 ? conv3_tc_kernel<3> : zt == 2 ? conv3_tc_kernel<2> : conv3_tc_kernel<1>;
     const dim3 grid((unsigned)(txy * ((nz + zt - 1) / zt)), conv_blocks(cout), N->B);
     kernel<<<grid, kConvThreads, conv_smem(zt, nb), N->stream>>>(src, w, bias, out, cin, cout, nx, ny, nz, relu, N->err);
