@@ -33,11 +33,12 @@ namespace {
 // eight voxels along x are a core matrix of the canonical K-major layout without swizzle and a row of them a
 // fixed stride, so each of the 27 taps is the same tile at another start address, and no input is gathered
 // twice.  A halo plane goes through the taps of up to three output planes in one product (N up to 3 x the
-// columns: the accumulators of the tile's planes lie side by side), since one thread issues the products at a
-// rate that does not depend on N: 27 (ZT + 2) of them per 16 input channels instead of 81 ZT.  Forward pass on
-// 80^3 cells, channels 16 to 64 (75 GFLOP of convolutions): 0.85 ms; 1.19 ms with a product per plane, and
-// 5.76 ms with FP32 arithmetic on the CUDA cores (13 TFLOP/s).  Two CTAs per SM overlap one's halo loads with
-// the other's products.
+// columns: the accumulators of the tile's planes lie side by side): an MMA takes 48 clocks for N <= 96 and N / 2
+// beyond, so 27 (ZT + 2) of them per 16 input channels are cheaper than 81 ZT narrow ones.  Two CTAs of 512 threads
+// per SM overlap one's halo loads (latency-bound: 16 warps rather than 8 took the forward pass from 0.85 to 0.75
+// ms) with the other's products (half of the time).  Forward pass on 80^3 cells, channels 16 to 64 (75 GFLOP of
+// convolutions): 0.75 ms; 1.19 ms with a product per plane, and 5.76 ms with FP32 arithmetic on the CUDA cores (13
+// TFLOP/s).
 //
 // The tensor core adds into its FP32 accumulators by truncation: with one accumulator over all 81 products of
 // 16 input channels the outputs were 5.6e-6 off (relative, 2-norm), 10 times the FP32 multiply-adds' error.  So
@@ -48,7 +49,7 @@ namespace {
 // Around it, the loader reads the decoder's concatenation from its two sources (upsampled and skip), the
 // gradient through a ReLU from the gradient and the ReLU's output, and the epilogue adds the bias and applies
 // the ReLU: no pass over an activation is left between two convolutions but the pooling.
-constexpr int kConvThreads = 256;
+constexpr int kConvThreads = 512;
 constexpr int kTX = 8, kTY = 16, kHX = kTX + 2, kHY = kTY + 2;
 constexpr int kCoMax = 64;   // output channels of a CTA
 
@@ -107,7 +108,7 @@ __device__ __forceinline__ void split3(float x, uint32_t &hi, uint32_t &mid, uin
 }
 
 template <int ZT>
-__global__ void __launch_bounds__(kConvThreads)
+__global__ void __launch_bounds__(kConvThreads, 2)
     conv3_tc_kernel(ConvSrc src, const uint4 *__restrict__ w, const float *__restrict__ bias, float *__restrict__ out,
                     int cin, int cout, int nx, int ny, int nz, int relu, int *err)
 {
@@ -132,14 +133,12 @@ __global__ void __launch_bounds__(kConvThreads)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *slot;
-    // warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (rows y of four, 8 voxels along x each) of the items
-    // (z, 16 channels) w / 4, w / 4 + 2
-    const int items = ZT * (nb / 16);
-    float sum[2][16];
+    // warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (rows y of four, 8 voxels along x each) of item w / 4:
+    // (z, 16 channels)
+    const int items = ZT * (nb / 16), it = warp >> 2, zi = it / (nb / 16), col = it % (nb / 16) * 16;
+    float sum[16];
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int k = 0; k < 16; ++k) sum[i][k] = 0.f;
+    for (int k = 0; k < 16; ++k) sum[k] = 0.f;
     for (int ch = 0; ch < nch; ++ch) {
         for (int e = tid; e < 2 * HV; e += kConvThreads) {
             const int kc = e >= HV, v = e - kc * HV, hx = v % kHX, hy = v / kHX % kHY, hz = v / (kHX * kHY);
@@ -215,19 +214,15 @@ __global__ void __launch_bounds__(kConvThreads)
         }
         __syncwarp();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int it = (warp >> 2) + 2 * i;
-            if (it >= items) break;  // uniform across the warp
-            const int z = it / (nb / 16);
-            const uint32_t at = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + it % (nb / 16) * 16;
+        if (it < items) {  // uniform across the warp
+            const uint32_t at = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + col;
             float part[16];
 #pragma unroll
             for (int q = 3; q >= 0; --q) {
-                int blk = 3 * ZT + z;  // the small parts, then the leading ones of dz = 2, 1, 0
+                int blk = 3 * ZT + zi;  // the small parts, then the leading ones of dz = 2, 1, 0
                 if (q < 3) {
-                    blk = 2 - q - conv_s0(z + q);
-                    for (int k = 0; k < z + q; ++k) blk += conv_ns(ZT, k);
+                    blk = 2 - q - conv_s0(zi + q);
+                    for (int k = 0; k < zi + q; ++k) blk += conv_ns(ZT, k);
                 }
                 uint32_t v[16];
                 tc_load16(at + blk * nb, v);
@@ -236,20 +231,17 @@ __global__ void __launch_bounds__(kConvThreads)
                     part[k] = q == 3 ? __uint_as_float(v[k]) : __fadd_rn(part[k], __uint_as_float(v[k]));
             }
 #pragma unroll
-            for (int k = 0; k < 16; ++k) sum[i][k] = __fadd_rn(sum[i][k], part[k]);
+            for (int k = 0; k < 16; ++k) sum[k] = __fadd_rn(sum[k], part[k]);
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     }
-    const int vx = x0 + (lane & 7), vy = y0 + 4 * (warp & 3) + (lane >> 3);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int it = (warp >> 2) + 2 * i, vz = z0 + it / (nb / 16);
-        if (it >= items || vx >= nx || vy >= ny || vz >= nz) continue;
+    const int vx = x0 + (lane & 7), vy = y0 + 4 * (warp & 3) + (lane >> 3), vz = z0 + zi;
+    if (it < items && vx < nx && vy < ny && vz < nz) {
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-            const int co = blockIdx.y * kCoMax + it % (nb / 16) * 16 + k;
+            const int co = blockIdx.y * kCoMax + col + k;
             if (co < cout) {
-                float f = sum[i][k];
+                float f = sum[k];
                 if (bias) f = __fadd_rn(f, bias[co]);
                 if (relu) f = fmaxf(f, 0.f);
                 out[((int64_t)b * cout + co) * S + ((int64_t)vz * ny + vy) * nx + vx] = f;

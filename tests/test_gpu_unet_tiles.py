@@ -39,10 +39,10 @@ def _layers(base, levels):
     return conv + [(ch[0], 3)]
 
 
-# (levels, base, (z, y, x), batch); the fifth runs the two-plane tiles (>= 304 of them), the sixth the three-plane ones
+# (levels, base, (z, y, x), batch); the fifth runs the two-plane tiles, the sixth the three-plane ones (288 blocks each)
 @pytest.mark.parametrize("levels,base,shape,batch", [(1, 5, (3, 17, 9), 2), (2, 12, (6, 18, 10), 1), (1, 70, (2, 5, 3), 1),
-                                                     (3, 17, (4, 8, 12), 3), (1, 20, (33, 34, 41), 1),
-                                                     (1, 12, (50, 34, 41), 1)])
+                                                     (3, 17, (4, 8, 12), 3), (1, 20, (31, 34, 41), 1),
+                                                     (1, 12, (47, 34, 41), 1)])
 def test_unet_tile_edges(levels, base, shape, batch):
     from paper_1809_00828_gb300 import fcm
     net = fcm.UNet(in_ch=4, out_ch=3, base=base, levels=levels, seed=1)
