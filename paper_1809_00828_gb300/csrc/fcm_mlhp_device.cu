@@ -69,11 +69,32 @@ __global__ void __launch_bounds__(kThreads) mlhp_spmv_kernel(int n, const int64_
     if (row >= n) return;  // uniform across the warp
     float S = 0.f, C = 0.f;
     const int64_t e1 = rowptr[row + 1];
-#pragma unroll 4
-    for (int64_t e = rowptr[row] + lane; e < e1; e += 32) {
-        const float2 v = __ldcs(vals + e);
-        const float2 xv = x[cols[e]];
-        ff_fma(v.x, v.y, xv.x, xv.y, S, C);
+    // batches of four nonzeros per lane, the next batch's columns and values loaded before this one's entries of x:
+    // the chain column -> x -> product is what bounds it (k = 3 cube, 20 M nonzeros: 82 -> 69 us, 240 MB)
+    constexpr int U = 4;
+    int c[U];
+    float2 v[U];
+    auto load = [&](int64_t e) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool on = e + 32 * u < e1;
+            c[u] = on ? __ldcs(cols + e + 32 * u) : 0;
+            v[u] = on ? __ldcs(vals + e + 32 * u) : make_float2(0.f, 0.f);
+        }
+    };
+    int64_t e = rowptr[row] + lane;
+    load(e);
+    while (e < e1) {
+        float2 xv[U], a[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            xv[u] = e + 32 * u < e1 ? __ldg(x + c[u]) : make_float2(0.f, 0.f);
+            a[u] = v[u];
+        }
+        e += 32 * U;
+        load(e);
+#pragma unroll
+        for (int u = 0; u < U; ++u) ff_fma(a[u].x, a[u].y, xv[u].x, xv[u].y, S, C);
     }
     ff_warp_sum(S, C);
     if (lane == 0) y[row] = ff_to_double(ff_norm(S, C));
