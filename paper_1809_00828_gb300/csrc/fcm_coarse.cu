@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "fcm_device.cuh"
+#include "fcm_reduce.cuh"
 
 namespace fcm {
 
@@ -96,7 +97,7 @@ void fcg_free(FcgState *F)
 
 namespace {
 
-constexpr int RT = 256;
+constexpr int RT = kReduceThreads;
 
 #define STOP_RETURN \
     if (stop && *stop) return
@@ -165,52 +166,6 @@ __global__ void prolong_add_kernel(const float *__restrict__ cells, const uint8_
         for (int a = 0; a < 3; ++a)
             if (mask[3 * node + a]) z[3 * node + a] += 0.125 * acc[a];
     }
-}
-
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Sum over the CTA; valid in thread 0.
-__device__ double block_sum(double v, double *sh)
-{
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    v = threadIdx.x < RT / 32 ? sh[threadIdx.x] : 0.0;
-    if (threadIdx.x < 32) v = warp_sum(v);
-    __syncthreads();
-    return v;
-}
-
-// K sums over the grid in a fixed order: every CTA publishes its partials, the last CTA
-// to arrive adds them up (thread 0 then holds the totals) and returns true.
-template <int K>
-__device__ bool grid_sums(double (&v)[K], double *partial, unsigned *counter)
-{
-    __shared__ double sh[RT / 32];
-    __shared__ bool last;
-#pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = block_sum(v[k], sh);
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) partial[K * blockIdx.x + k] = v[k];
-        __threadfence();
-        last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return false;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        double x = 0.0;
-        for (int i = threadIdx.x; i < (int)gridDim.x; i += RT) x += __ldcg(partial + K * i + k);
-        v[k] = block_sum(x, sh);
-    }
-    if (threadIdx.x == 0) *counter = 0u;
-    return true;
 }
 
 // sb_norm = ||S b||; resets the iteration state

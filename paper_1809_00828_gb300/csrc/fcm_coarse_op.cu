@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "fcm_device.cuh"
+#include "fcm_reduce.cuh"
 
 namespace fcm {
 
@@ -77,7 +78,7 @@ struct CoarseOp {
 
 namespace {
 
-constexpr int RT = 256;
+constexpr int RT = kReduceThreads;
 constexpr int kCenter = 62;               // offset index of (0, 0, 0) in the 5x5x5 stencil
 constexpr int kStored = 63;               // offsets kCenter..124 are stored; the others by symmetry
 constexpr int kTileCells = 32;            // cells per CTA of the K_H apply (one per lane)
@@ -176,50 +177,6 @@ __global__ void diag_inverse_kernel(const float *KH, float *Dinv, int64_t ncell)
         D[7] = (float)(-(a * l - b * k) * id);
         D[8] = (float)((a * f - b * e) * id);
     }
-}
-
-__device__ __forceinline__ double wsum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-__device__ double bsum(double v, double *sh)
-{
-    v = wsum(v);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    v = threadIdx.x < RT / 32 ? sh[threadIdx.x] : 0.0;
-    if (threadIdx.x < 32) v = wsum(v);
-    __syncthreads();
-    return v;
-}
-
-// Two sums over the grid in a fixed order; true in the last CTA, whose thread 0 then holds the totals.
-__device__ bool grid_sums2(double &x, double &y, double *partial, unsigned *counter)
-{
-    __shared__ double sh[RT / 32];
-    __shared__ bool last;
-    x = bsum(x, sh);
-    y = bsum(y, sh);
-    if (threadIdx.x == 0) {
-        partial[2 * blockIdx.x] = x;
-        partial[2 * blockIdx.x + 1] = y;
-        __threadfence();
-        last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return false;
-    double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += RT) {
-        a += __ldcg(partial + 2 * i);
-        b += __ldcg(partial + 2 * i + 1);
-    }
-    x = bsum(a, sh);
-    y = bsum(b, sh);
-    if (threadIdx.x == 0) *counter = 0u;
-    return true;
 }
 
 // y = K_H v over a tile of 32 cells per CTA (at most 64 registers, 4 offsets unrolled: more loads in
@@ -337,7 +294,7 @@ __global__ void __launch_bounds__(RT, 4) kh_kernel(const T *__restrict__ KH, con
         }
         return;
     }
-    double dot = 0.0, unused = 0.0;
+    double dot[1] = {0.0};
     if (w < 3) {
         // warp w finishes component w of the 32 cells
         float acc = 0.f;
@@ -350,14 +307,14 @@ __global__ void __launch_bounds__(RT, 4) kh_kernel(const T *__restrict__ KH, con
                 float v = x[w * ncell + c];
                 if (mode == 1) v = fmaf(beta, xb[w * ncell + c], v);
                 pout[w * ncell + c] = v;
-                dot = (double)v * acc;
+                dot[0] = (double)v * acc;
             }
         }
     }
     if (mode == 0) return;
-    if (!grid_sums2(dot, unused, partial, counter) || threadIdx.x) return;
-    sc[1] = dot;
-    sc[2] = (dot > 0.0 && isfinite(sc[0] / dot)) ? sc[0] / dot : 0.0;
+    if (!grid_sums(dot, partial, counter, 3) || threadIdx.x) return;
+    sc[1] = dot[0];
+    sc[2] = (dot[0] > 0.0 && isfinite(sc[0] / dot[0])) ? sc[0] / dot[0] : 0.0;
 }
 
 // line search t = f.y / y.q (0 when y.q <= 0), into sc[4]
@@ -365,13 +322,13 @@ __global__ void __launch_bounds__(RT) line_kernel(const float *f, const float *y
                                                    double *partial, unsigned *counter, double *sc, const int *stop)
 {
     STOP_RETURN;
-    double a = 0.0, b = 0.0;
+    double v[2] = {0.0, 0.0};
     for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) {
-        a += (double)f[i] * y[i];
-        b += (double)y[i] * q[i];
+        v[0] += (double)f[i] * y[i];
+        v[1] += (double)y[i] * q[i];
     }
-    if (!grid_sums2(a, b, partial, counter) || threadIdx.x) return;
-    sc[4] = (b > 0.0 && isfinite(a / b)) ? a / b : 0.0;
+    if (!grid_sums(v, partial, counter) || threadIdx.x) return;
+    sc[4] = (v[1] > 0.0 && isfinite(v[0] / v[1])) ? v[0] / v[1] : 0.0;
 }
 
 // Start of the coarse CG, one thread per cell:
@@ -383,7 +340,7 @@ __global__ void __launch_bounds__(RT) cstart_kernel(const float *f, float *y, fl
 {
     STOP_RETURN;
     const float t = start == 2 ? (float)sc[4] : 1.f;
-    double dot = 0.0, unused = 0.0;
+    double dot[1] = {0.0};
     for (int64_t c = blockIdx.x * (int64_t)RT + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * RT) {
         float rv[3];
         for (int a = 0; a < 3; ++a) {
@@ -402,13 +359,13 @@ __global__ void __launch_bounds__(RT) cstart_kernel(const float *f, float *y, fl
             for (int a = 0; a < 3; ++a) {
                 const float zv = D[3 * a] * rv[0] + D[3 * a + 1] * rv[1] + D[3 * a + 2] * rv[2];
                 z[a * ncell + c] = zv;
-                dot += (double)rv[a] * zv;
+                dot[0] += (double)rv[a] * zv;
             }
         }
     }
     if (!want_z) return;
-    if (!grid_sums2(dot, unused, partial, counter) || threadIdx.x) return;
-    sc[0] = dot;
+    if (!grid_sums(dot, partial, counter) || threadIdx.x) return;
+    sc[0] = dot[0];
 }
 
 // y += alpha p, r -= alpha q; unless last: z = Dinv r, rz' = r.z, beta = rz' / rz, rz = rz'
@@ -418,7 +375,7 @@ __global__ void __launch_bounds__(RT) cupd_kernel(float *y, float *r, float *z, 
 {
     STOP_RETURN;
     const float al = (float)sc[2];
-    double dot = 0.0, unused = 0.0;
+    double dot[1] = {0.0};
     for (int64_t c = blockIdx.x * (int64_t)RT + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * RT) {
         float rv[3];
         for (int a = 0; a < 3; ++a) {
@@ -432,14 +389,14 @@ __global__ void __launch_bounds__(RT) cupd_kernel(float *y, float *r, float *z, 
             for (int a = 0; a < 3; ++a) {
                 const float zv = D[3 * a] * rv[0] + D[3 * a + 1] * rv[1] + D[3 * a + 2] * rv[2];
                 z[a * ncell + c] = zv;
-                dot += (double)rv[a] * zv;
+                dot[0] += (double)rv[a] * zv;
             }
         }
     }
     if (last_step) return;
-    if (!grid_sums2(dot, unused, partial, counter) || threadIdx.x) return;
-    sc[3] = (sc[0] > 0.0 && isfinite(dot / sc[0])) ? dot / sc[0] : 0.0;
-    sc[0] = dot;
+    if (!grid_sums(dot, partial, counter) || threadIdx.x) return;
+    sc[3] = (sc[0] > 0.0 && isfinite(dot[0] / sc[0])) ? dot[0] / sc[0] : 0.0;
+    sc[0] = dot[0];
 }
 
 // ---- geometric multigrid on the cell grid (the V-cycle that may precondition the coarse CG) ----
@@ -599,10 +556,10 @@ __global__ void __launch_bounds__(RT) jacobi0_kernel(const float *__restrict__ f
 __global__ void __launch_bounds__(RT) sumsq_kernel(const float *u, int64_t n, double *partial, unsigned *counter,
                                                     double *out)
 {
-    double a = 0.0, unused = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) a += (double)u[i] * u[i];
-    if (!grid_sums2(a, unused, partial, counter) || threadIdx.x) return;
-    *out = a;
+    double a[1] = {0.0};
+    for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) a[0] += (double)u[i] * u[i];
+    if (!grid_sums(a, partial, counter) || threadIdx.x) return;
+    *out = a[0];
 }
 
 // u = s Dinv v (one thread per cell), for the power iteration
@@ -687,11 +644,11 @@ __global__ void __launch_bounds__(RT) rz_kernel(const float *r, const float *z, 
                                                  unsigned *counter, double *sc, const int *stop)
 {
     STOP_RETURN;
-    double a = 0.0, unused = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) a += (double)r[i] * z[i];
-    if (!grid_sums2(a, unused, partial, counter) || threadIdx.x) return;
-    if (!first) sc[3] = (sc[0] > 0.0 && isfinite(a / sc[0])) ? a / sc[0] : 0.0;
-    sc[0] = a;
+    double a[1] = {0.0};
+    for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) a[0] += (double)r[i] * z[i];
+    if (!grid_sums(a, partial, counter) || threadIdx.x) return;
+    if (!first) sc[3] = (sc[0] > 0.0 && isfinite(a[0] / sc[0])) ? a[0] / sc[0] : 0.0;
+    sc[0] = a[0];
 }
 
 // s_c = (tr K_cc / 3)^-1/2 from the centre block, and 1 / s_c (both 0 where the trace is 0)

@@ -11,57 +11,13 @@
 #include <cuda_runtime.h>
 
 #include "fcm_device.cuh"
+#include "fcm_reduce.cuh"
 
 namespace fcm {
 
 namespace {
 
-constexpr int RT = 256;
-
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Sum over the CTA; the result is valid in thread 0.
-__device__ __forceinline__ double block_sum(double v, double *sh)
-{
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    v = (threadIdx.x < RT / 32) ? sh[threadIdx.x] : 0.0;
-    if (warp == 0) v = warp_sum(v);
-    __syncthreads();
-    return v;
-}
-
-// Publishes the CTA partials and tells whether this CTA is the last one.
-__device__ __forceinline__ bool publish(double a, double b, double *partial, unsigned *counter, bool *last)
-{
-    if (threadIdx.x == 0) {
-        partial[2 * blockIdx.x] = a;
-        partial[2 * blockIdx.x + 1] = b;
-        __threadfence();
-        *last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    return *last;
-}
-
-// Fixed-order sum of the partials (run by the last CTA only).
-__device__ __forceinline__ void gather(const double *partial, double *sh, double &a, double &b)
-{
-    double x = 0.0, y = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += RT) {
-        x += __ldcg(partial + 2 * i);
-        y += __ldcg(partial + 2 * i + 1);
-    }
-    a = block_sum(x, sh);
-    b = block_sum(y, sh);
-}
+constexpr int RT = kReduceThreads;
 
 __global__ void __launch_bounds__(RT) init_kernel(double *x, double *r, const double *b, int64_t n)
 {
@@ -75,8 +31,6 @@ __global__ void __launch_bounds__(RT) init_kernel(double *x, double *r, const do
 __global__ void __launch_bounds__(RT) first_kernel(const double *r, const double *z, double *p, int64_t n,
                                                     double *partial, unsigned *counter, CgScalars *S)
 {
-    __shared__ double sh[RT / 32];
-    __shared__ bool last;
     double a = 0.0, b = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) {
         const double zi = z[i];
@@ -84,12 +38,11 @@ __global__ void __launch_bounds__(RT) first_kernel(const double *r, const double
         b = fma(zi, zi, b);
         p[i] = zi;
     }
-    a = block_sum(a, sh);
-    b = block_sum(b, sh);
-    if (!publish(a, b, partial, counter, &last)) return;
-    gather(partial, sh, a, b);
+    double v[2] = {a, b};
+    if (!grid_sums(v, partial, counter)) return;
     if (threadIdx.x == 0) {
-        *counter = 0u;
+        a = v[0];
+        b = v[1];
         S->rz = a;
         S->zz0 = b;
         S->zz = b;
@@ -112,16 +65,12 @@ __global__ void __launch_bounds__(RT) pq_kernel(const double *p, const double *q
                                                  unsigned *counter, CgScalars *S)
 {
     if (S->done) return;
-    __shared__ double sh[RT / 32];
-    __shared__ bool last;
     double a = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) a = fma(p[i], q[i], a);
-    a = block_sum(a, sh);
-    if (!publish(a, 0.0, partial, counter, &last)) return;
-    double b;
-    gather(partial, sh, a, b);
+    double v[1] = {a};
+    if (!grid_sums(v, partial, counter)) return;
     if (threadIdx.x == 0) {
-        *counter = 0u;
+        a = v[0];
         S->pq = a;
         const double alpha = S->rz / a;
         S->alpha = alpha;
@@ -149,20 +98,17 @@ __global__ void __launch_bounds__(RT) rz_kernel(const double *r, const double *z
                                                  unsigned *counter, CgScalars *S)
 {
     if (S->done) return;
-    __shared__ double sh[RT / 32];
-    __shared__ bool last;
     double a = 0.0, b = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) {
         const double zi = z[i];
         a = fma(r[i], zi, a);
         b = fma(zi, zi, b);
     }
-    a = block_sum(a, sh);
-    b = block_sum(b, sh);
-    if (!publish(a, b, partial, counter, &last)) return;
-    gather(partial, sh, a, b);
+    double v[2] = {a, b};
+    if (!grid_sums(v, partial, counter)) return;
     if (threadIdx.x == 0) {
-        *counter = 0u;
+        a = v[0];
+        b = v[1];
         S->zz = b;
         S->it += 1;
         const double rel = sqrt(b / S->zz0);
@@ -195,22 +141,17 @@ __global__ void __launch_bounds__(RT) p_kernel(double *p, const double *z, int64
 __global__ void __launch_bounds__(RT) resid_kernel(const double *kx, const double *b, int64_t n, double *partial,
                                                     unsigned *counter, double *out2)
 {
-    __shared__ double sh[RT / 32];
-    __shared__ bool last;
     double a = 0.0, c = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) {
         const double d = b[i] - kx[i];
         a = fma(d, d, a);
         c = fma(b[i], b[i], c);
     }
-    a = block_sum(a, sh);
-    c = block_sum(c, sh);
-    if (!publish(a, c, partial, counter, &last)) return;
-    gather(partial, sh, a, c);
+    double v[2] = {a, c};
+    if (!grid_sums(v, partial, counter)) return;
     if (threadIdx.x == 0) {
-        *counter = 0u;
-        out2[0] = a;
-        out2[1] = c;
+        out2[0] = v[0];
+        out2[1] = v[1];
     }
 }
 
