@@ -69,9 +69,9 @@ __global__ void __launch_bounds__(kThreads) mlhp_spmv_kernel(int n, const int64_
     if (row >= n) return;  // uniform across the warp
     float S = 0.f, C = 0.f;
     const int64_t e1 = rowptr[row + 1];
-    // batches of four nonzeros per lane, the next batch's columns and values loaded before this one's entries of x:
-    // the chain column -> x -> product is what bounds it (k = 3 cube, 20 M nonzeros: 82 -> 69 us, 240 MB)
-    constexpr int U = 4;
+    // batches of eight nonzeros per lane, the next batch's columns and values loaded before this one's entries of x:
+    // the chain column -> x -> product is what bounds it (k = 3 cube, 23.5 M nonzeros, 282 MB: 82 us one at a time, 69 with four, 62 with eight)
+    constexpr int U = 8;
     int c[U];
     float2 v[U];
     auto load = [&](int64_t e) {
