@@ -284,12 +284,14 @@ __global__ void conv_tiles_kernel(const __nv_bfloat16 *__restrict__ w, __nv_bflo
 // and one input channel of one plane of the tile, with their 27 taps (and the bias) in registers: eight voxels
 // along x cost 31 vector reads of shared memory and 448 multiply-adds (one output channel and four voxels a time
 // cost 19 reads for 112).  The tiles are dealt to enough CTAs to fill the GPU, each
-// writes its sums to `part`, and wgrad_sum_kernel adds them in a fixed order in FP64 (deterministic).  One CTA per
+// writes its sums to `part`, and wgrad_sum_kernel adds them in a fixed order in FP64 (deterministic).  Half of the
+// instructions of a first version went into the indices of the tiles' loads: a thread now keeps its point of the
+// tile and walks channels and planes, all 24 + 16 loads in flight.  One CTA per
 // (co, ci) pair with 27 unshared global reads per multiply-add row took 4.9 ms for the gradients of the
-// 16-to-64-channel network on four 32^3 cubes, one channel a thread 1.08 + 0.29 ms; this 0.90 + 0.12 ms.
+// 16-to-64-channel network on four 32^3 cubes, one channel a thread 1.08 + 0.29 ms; this 0.73 + 0.12 ms.
 constexpr int kWC = 8, kWO = 16, kWX = 8, kWY = 8, kWZ = 4, kWGo = kWX * kWY * kWZ + 4;
 constexpr int kWRow = 12, kWPlane = kWRow * (kWY + 2), kWCh = kWPlane * (kWZ + 2) + 4;  // 4 channels: distinct banks
-constexpr int kWTaps = 28;
+constexpr int kWTaps = 28, kHaloXY = (kWX + 2) * (kWY + 2);
 constexpr int kSumParts = 16;  // parts of the slabs that wgrad_sum_kernel adds side by side
 
 __global__ void __launch_bounds__(256, 2)
@@ -301,6 +303,9 @@ __global__ void __launch_bounds__(256, 2)
     const int co = tid & 7, ci = tid >> 3 & 7, zq = tid >> 6;  // output channels co, co + 8; plane zq of the tile
     const int tx = (nx + kWX - 1) / kWX, ty = (ny + kWY - 1) / kWY, tz = (nz + kWZ - 1) / kWZ;
     const int64_t tiles = (int64_t)B * tx * ty * tz;
+    const int64_t S = (int64_t)nx * ny * nz, S2 = (int64_t)(nx >> 1) * (ny >> 1) * (nz >> 1);
+    const int half = tid >> 7, pt = tid & 127, hx = pt % (kWX + 2), hy = pt / (kWX + 2);
+    static_assert(kHaloXY <= 128 && kWX * kWY * kWZ == 256 && kWZ + 2 == 6, "threads of the loads");
     float acc[2][kWTaps];
 #pragma unroll
     for (int t = 0; t < kWTaps; ++t) acc[0][t] = acc[1][t] = 0.f;
@@ -308,20 +313,40 @@ __global__ void __launch_bounds__(256, 2)
         const int b = (int)(tile / ((int64_t)tx * ty * tz)), q = (int)(tile % ((int64_t)tx * ty * tz));
         const int x0 = q % tx * kWX, y0 = q / tx % ty * kWY, z0 = q / (tx * ty) * kWZ;
         __syncthreads();
-#pragma unroll 10  // that many loads in flight
-        for (int e = tid; e < kWC * (kWZ + 2) * (kWY + 2) * (kWX + 2); e += 256) {
-            const int hx = e % (kWX + 2), hy = e / (kWX + 2) % (kWY + 2), hz = e / ((kWX + 2) * (kWY + 2)) % (kWZ + 2),
-                      c = e / ((kWX + 2) * (kWY + 2) * (kWZ + 2));
-            const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
-            const bool on = ci0 + c < cin && x >= 0 && y >= 0 && z >= 0 && x < nx && y < ny && z < nz;
-            si[c * kWCh + hz * kWPlane + hy * kWRow + hx] = on ? conv_load(in, b, ci0 + c, x, y, z, nx, ny, nz) : 0.f;
+        {  // the inputs with their halo: threads 128 h .. + 99 take a plane's points, the halves every other plane
+            const int x = x0 + hx - 1, y = y0 + hy - 1;
+            const bool inxy = pt < kHaloXY && x >= 0 && y >= 0 && x < nx && y < ny;
+            float v[3][kWC];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const int z = z0 + 2 * i + half - 1;
+                const bool on = inxy && z >= 0 && z < nz;
+                const float *pf = in.full + (((int64_t)b * in.c1 + ci0 - in.c0) * nz + z) * ny * nx + (int64_t)y * nx + x;
+                const float *ph = in.half + (((int64_t)b * in.c0 + ci0) * (nz >> 1) + (z >> 1)) * (ny >> 1) * (nx >> 1) +
+                                  (int64_t)(y >> 1) * (nx >> 1) + (x >> 1);
+#pragma unroll
+                for (int c = 0; c < kWC; ++c)
+                    v[i][c] = on && ci0 + c < cin ? __ldg(ci0 + c < in.c0 ? ph + c * S2 : pf + c * S) : 0.f;
+            }
+            if (pt < kHaloXY)
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+#pragma unroll
+                    for (int c = 0; c < kWC; ++c) si[c * kWCh + (2 * i + half) * kWPlane + hy * kWRow + hx] = v[i][c];
         }
-#pragma unroll 8
-        for (int e = tid; e < kWO * kWX * kWY * kWZ; e += 256) {
-            const int v = e % (kWX * kWY * kWZ), c = e / (kWX * kWY * kWZ);
-            const int x = x0 + v % kWX, y = y0 + v / kWX % kWY, z = z0 + v / (kWX * kWY);
-            const bool on = co0 + c < cout && x < nx && y < ny && z < nz;
-            sg[c][v] = on ? conv_load(go, b, co0 + c, x, y, z, nx, ny, nz) : 0.f;
+        {  // the gradients: a voxel per thread
+            const int x = x0 + tid % kWX, y = y0 + tid / kWX % kWY, z = z0 + tid / (kWX * kWY);
+            const bool on = x < nx && y < ny && z < nz;
+            const int64_t at = (((int64_t)b * cout + co0) * nz + z) * ny * nx + (int64_t)y * nx + x;
+            float v[kWO];
+#pragma unroll
+            for (int c = 0; c < kWO; ++c) v[c] = on && co0 + c < cout ? __ldg(go.full + at + c * S) : 0.f;
+            if (go.gate)
+#pragma unroll
+                for (int c = 0; c < kWO; ++c)
+                    if (!(on && co0 + c < cout && __ldg(go.gate + at + c * S) > 0.f)) v[c] = 0.f;
+#pragma unroll
+            for (int c = 0; c < kWO; ++c) sg[c][tid] = v[c];
         }
         __syncthreads();
 #pragma unroll 1
