@@ -74,7 +74,7 @@ COARSE_DEFAULTS = {"porous40_32_p3": ("jacobi", 20, "fp32"), "porous40_32_p2": (
 def _schwarz_traffic(workload_name, precision):
     """DRAM bytes of one S apply from the committed ncu capture, or None.
 
-    The capture (dram__bytes_read.sum + dram__bytes_write.sum over the 8 colour launches of one S
+    The capture (dram__bytes_read.sum + dram__bytes_write.sum over the launches of one S
     apply) holds for the kernel source it was taken with: the profile records the SHA-256 of
     fcm_schwarz.cu, and any other source gives None.
     """
@@ -348,8 +348,8 @@ def _launches_per_solve(args, info, its, flex_its, net, mg_levels=0):
 
 def _unet_launches(net):
     L = net.desc[3]
-    # per level: pool (l > 0), 2 x (conv, relu); per decoder level: up, copy, 2 x (conv, relu); output conv
-    return (L - 1) + 4 * L + 6 * (L - 1) + 1
+    # per level: pool (l > 0), 2 convolutions; per decoder level: 2; output convolution
+    return (L - 1) + 2 * L + 2 * (L - 1) + 1
 
 
 def max_over_ranks(value, dist, device):
@@ -506,8 +506,9 @@ def run_fcm(args, rank, world, local_rank):
     achieved_gbs = s_bytes / t_s / 1e9
     shared = (f"tc_gemm_kernel<{w.p}> (tcgen05, shared factors)" if args.precision != "fp64" and w.p in (2, 3)
               else f"schwarz_gemm_kernel<{w.p}> (shared factors)")
-    kernel = (f"S apply, {info['s_apply_launches']} launches: {shared} + "
-              f"{'schwarz_rows_kernel' if w.p == 3 else 'schwarz_cols_kernel'}<{w.p}> (streamed factors) + "
+    streamed = ("schwarz_rows_kernel" if w.p == 3 else
+                "schwarz_fold_kernel" if w.p <= 2 and args.precision != "fp64" else "schwarz_cols_kernel")
+    kernel = (f"S apply, {info['s_apply_launches']} launches: {shared} + {streamed}<{w.p}> (streamed factors) + "
               f"schwarz_sum_kernel<{w.p}>, shared-factor products "
               f"{'beside' if info['schwarz_concurrent'] else 'before'} the streamed ones (the shape the build's "
               f"autotuner kept)")

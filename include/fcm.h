@@ -289,7 +289,9 @@ typedef struct {
 fcm_status fcm_unet_create(const fcm_unet_desc *desc, void *cuda_stream, fcm_unet **out);
 /* Number of parameters (all weights then all biases, layer by layer). */
 fcm_status fcm_unet_params(const fcm_unet *net, int64_t *count);
-/* Copy the FP32 master parameters (and, if g_host != NULL, their gradients) to host memory. */
+/* Copy the FP32 master parameters (and, if g_host != NULL, their gradients) to host memory.
+ * FCM_ETIMEOUT: a convolution since the last call gave up its bounded wait for the tensor core, so an
+ * output or gradient since then is not valid (the parameters are copied all the same). */
 fcm_status fcm_unet_get(fcm_unet *net, float *w_host, float *g_host);
 /* Replace the FP32 master parameters from host memory (BF16 copies are refreshed). */
 fcm_status fcm_unet_set(fcm_unet *net, const float *w_host);
