@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "fcm_device.cuh"
+#include "fcm_ff.cuh"
 #include "fcm_tma.cuh"
 
 namespace fcm {
@@ -284,19 +285,26 @@ __global__ void conv_tiles_kernel(const __nv_bfloat16 *__restrict__ w, __nv_bflo
 // and one input channel of one plane of the tile, with their 27 taps (and the bias) in registers: eight voxels
 // along x cost 31 vector reads of shared memory and 448 multiply-adds (one output channel and four voxels a time
 // cost 19 reads for 112).  The tiles are dealt to enough CTAs to fill the GPU, each
-// writes its sums to `part`, and wgrad_sum_kernel adds them in a fixed order in FP64 (deterministic).  Half of the
+// writes its sums to `part`, and wgrad_sum_kernel adds them in a fixed order in FP64 (deterministic).  The more
+// channels a layer has, the fewer CTAs share a channel pair's voxels (with 256 x 256 channels one), so every `fold`
+// tiles the registers' FP32 sums are added to float pairs in shared memory: no chain of FP32 additions is longer
+// than 64 or a 256th of the voxels (wgrad_fold), whatever the layer.  With chains over all of a CTA's voxels the gradients
+// of a 256 -> 256 layer on 32^3 voxels were 9.4e-7 off (2-norm), now 1.2e-7, and those of 192 -> 64 on 48^3 3.7e-6,
+// now 0.8e-6; the folds take 0.6 % of a training step.  Half of the
 // instructions of a first version went into the indices of the tiles' loads: a thread now keeps its point of the
 // tile and walks channels and planes, all 24 + 16 loads in flight.  One CTA per
 // (co, ci) pair with 27 unshared global reads per multiply-add row took 4.9 ms for the gradients of the
 // 16-to-64-channel network on four 32^3 cubes, one channel a thread 1.08 + 0.29 ms; this 0.73 + 0.12 ms.
 constexpr int kWC = 8, kWO = 16, kWX = 8, kWY = 8, kWZ = 4, kWGo = kWX * kWY * kWZ + 4;
 constexpr int kWRow = 12, kWPlane = kWRow * (kWY + 2), kWCh = kWPlane * (kWZ + 2) + 4;  // 4 channels: distinct banks
-constexpr int kWTaps = 28, kHaloXY = (kWX + 2) * (kWY + 2);
+constexpr int kWTaps = 28, kWRun = 64 * 2 * kWTaps * 8 /* bytes of the running sums */, kHaloXY = (kWX + 2) * (kWY + 2);
 constexpr int kSumParts = 16;  // parts of the slabs that wgrad_sum_kernel adds side by side
 
 __global__ void __launch_bounds__(256, 2)
-    conv3_wgrad_kernel(ConvSrc in, ConvSrc go, int cin, int cout, int B, int nx, int ny, int nz, float *__restrict__ part)
+    conv3_wgrad_kernel(ConvSrc in, ConvSrc go, int cin, int cout, int B, int nx, int ny, int nz, int fold,
+                       float *__restrict__ part)
 {
+    extern __shared__ float2 run[];  // running sums, [2 x 28][64 threads] (where a CTA folds more than once)
     __shared__ __align__(16) float si[kWC * kWCh];
     __shared__ __align__(16) float sg[kWO][kWGo];
     const int ci0 = blockIdx.x * kWC, co0 = blockIdx.y * kWO, tid = threadIdx.x;
@@ -309,6 +317,10 @@ __global__ void __launch_bounds__(256, 2)
     float acc[2][kWTaps];
 #pragma unroll
     for (int t = 0; t < kWTaps; ++t) acc[0][t] = acc[1][t] = 0.f;
+    float *red = si;  // 64 x 2 x 28 floats
+    static_assert(64 * 2 * kWTaps <= kWC * kWCh, "reduction buffer");
+    int held = 0;  // tiles in acc
+    bool first = true;
     for (int64_t tile = blockIdx.z; tile < tiles; tile += gridDim.z) {
         const int b = (int)(tile / ((int64_t)tx * ty * tz)), q = (int)(tile % ((int64_t)tx * ty * tz));
         const int x0 = q % tx * kWX, y0 = q / tx % ty * kWY, z0 = q / (tx * ty) * kWZ;
@@ -374,21 +386,36 @@ __global__ void __launch_bounds__(256, 2)
                         for (int o = 0; o < 2; ++o) acc[o][3 * d + dx] = fmaf(g[o][k], v[k + dx], acc[o][3 * d + dx]);
             }
         }
-    }
-    // the four planes, then this CTA's sums: part[z][co][ci][tap]
-    float *red = si;  // 64 x 2 x 28 floats
-    static_assert(64 * 2 * kWTaps <= kWC * kWCh, "reduction buffer");
+        const bool last = tile + gridDim.z >= tiles;
+        if (++held < fold && !last) continue;
+        held = 0;
+        // the four planes, then the running sums
 #pragma unroll 1
-    for (int w = 1; w < kWZ; ++w) {
-        __syncthreads();
-        if (zq == w)
+        for (int w = 1; w < kWZ; ++w) {
+            __syncthreads();
+            if (zq == w)
 #pragma unroll
-            for (int t = 0; t < 2 * kWTaps; ++t) red[t * 64 + (tid & 63)] = acc[t / kWTaps][t % kWTaps];
-        __syncthreads();
-        if (zq == 0)
+                for (int t = 0; t < 2 * kWTaps; ++t) red[t * 64 + (tid & 63)] = acc[t / kWTaps][t % kWTaps];
+            __syncthreads();
+            if (zq == 0)
 #pragma unroll
-            for (int t = 0; t < 2 * kWTaps; ++t) acc[t / kWTaps][t % kWTaps] += red[t * 64 + tid];
+                for (int t = 0; t < 2 * kWTaps; ++t) acc[t / kWTaps][t % kWTaps] += red[t * 64 + tid];
+        }
+        if (zq == 0 && !(first && last))
+#pragma unroll
+            for (int t = 0; t < 2 * kWTaps; ++t) {
+                float &a = acc[t / kWTaps][t % kWTaps];
+                float2 r = first ? make_float2(0.f, 0.f) : run[t * 64 + tid];
+                ff_add(r.x, r.y, a, 0.f);
+                if (!last) run[t * 64 + tid] = r;
+                else a = r.y == r.y ? r.x + r.y : r.x;  // the errors of an infinite sum are NaN
+            }
+        first = false;
+        if (!last)
+#pragma unroll
+            for (int t = 0; t < kWTaps; ++t) acc[0][t] = acc[1][t] = 0.f;
     }
+    // this CTA's sums: part[z][co][ci][tap]
     if (zq == 0) {
 #pragma unroll
         for (int o = 0; o < 2; ++o) {
@@ -617,6 +644,10 @@ int wgrad_slabs(int cin, int cout, int64_t tiles)
     return (int)std::max<int64_t>(1, std::min<int64_t>({tiles, 304 / ch, (int64_t)65535}));
 }
 
+// Tiles (64 voxels per thread) whose products a weight gradient adds in one chain of FP32 additions: a 256th of the
+// voxels of a channel pair, at least one tile
+int wgrad_fold(int64_t voxels) { return (int)std::max<int64_t>(1, voxels / (256 * kWX * kWY)); }
+
 // out = [relu](bias + conv(src)) at level l with the tiles of a convolution cin -> cout
 void conv_launch(fcm_unet *N, const ConvSrc &src, int64_t tiles, const float *bias, float *out, int cin, int cout, int l,
                  bool relu)
@@ -653,7 +684,9 @@ void conv_bwd(fcm_unet *N, int layer, const ConvSrc &in, const float *gout, cons
     const ConvSrc go{nullptr, gout, gate, 0, c.cout};
     const int64_t tiles = (int64_t)N->B * ((nx + kWX - 1) / kWX) * ((ny + kWY - 1) / kWY) * ((nz + kWZ - 1) / kWZ);
     const int cit = (c.cin + kWC - 1) / kWC, cot = (c.cout + kWO - 1) / kWO, ns = wgrad_slabs(c.cin, c.cout, tiles);
-    conv3_wgrad_kernel<<<dim3(cit, cot, ns), 256, 0, N->stream>>>(in, go, c.cin, c.cout, N->B, nx, ny, nz, N->part);
+    const int fold = wgrad_fold((int64_t)N->B * N->S[l]);
+    conv3_wgrad_kernel<<<dim3(cit, cot, ns), 256, (tiles + ns - 1) / ns > fold ? kWRun : 0, N->stream>>>(
+        in, go, c.cin, c.cout, N->B, nx, ny, nz, fold, N->part);
     const int np = std::max(1, std::min(ns / 8, kSumParts));
     wgrad_sum_kernel<<<blocks_for((int64_t)c.cin * c.cout * kWTaps * 8), dim3(32, np), 0, N->stream>>>(
         N->part, ns, c.cin, c.cout, cit * kWC, cot * kWO, N->g + c.woff, N->g + c.boff);
@@ -783,6 +816,8 @@ fcm_status fcm_unet_create(const fcm_unet_desc *d, void *cuda_stream, fcm_unet *
     if ((e = cudaMalloc((void **)&N->part, sizeof(float) * npart)) != cudaSuccess) return fail(e);
     if ((e = cudaMalloc((void **)&N->err, sizeof(int))) != cudaSuccess) return fail(e);
     if ((e = cudaMemsetAsync(N->err, 0, sizeof(int), N->stream)) != cudaSuccess) return fail(e);
+    if ((e = cudaFuncSetAttribute(conv3_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWRun)) != cudaSuccess)
+        return fail(e);
     if ((e = cudaFuncSetAttribute(conv3_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   conv_smem(1, kCoMax))) != cudaSuccess ||
         (e = cudaFuncSetAttribute(conv3_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, conv_smem(2, 32))) !=
