@@ -261,8 +261,9 @@ fcm_status fcm_apply_S_many(fcm_ctx *ctx, const double *r_dev, int nrhs, double 
  * the S apply (factors) or of the double-float K apply (element matrices, p <= 2)
  * waits for a bulk copy into shared memory (default 2^21).  A wait that runs
  * out lets the copies in flight land, marks the apply
- * as failed and returns; the solves then stop with FCM_ETIMEOUT (and
- * fcm_info.device_error reports it after fcm_apply_S).  tries = 0 gives up at
+ * as failed and returns; the solves then return FCM_ETIMEOUT, also when only the K
+ * apply of the true residual failed (fcm_last_error names the apply), and
+ * fcm_info.device_error reports it after fcm_apply_S or fcm_apply_K.  tries = 0 gives up at
  * the first poll (for tests); tries < 0 restores the default.  Captured solver
  * graphs are dropped (captured again by the next solve). */
 fcm_status fcm_set_wait_limit(fcm_ctx *ctx, int tries);

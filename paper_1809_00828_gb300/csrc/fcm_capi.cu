@@ -138,16 +138,11 @@ fcm_status solve_one(fcm_ctx *C, const double *rhs, double tol, int maxit, doubl
         fcm_status s = build_graph(C);
         if (s != FCM_OK) return s;
     }
-    bool timed_out = false;
     for (;;) {
         API_CUDA(C, cudaMemcpyAsync(&h, C->d_s, sizeof h, cudaMemcpyDeviceToHost, st));
         API_CUDA(C, cudaMemcpyAsync(C->h_err, C->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
         API_CUDA(C, cudaStreamSynchronize(st));
-        if (*C->h_err) {
-            timed_out = true;  // a Schwarz apply gave up waiting for a factor copy: its z is wrong
-            break;
-        }
-        if (h.done) break;
+        if (*C->h_err || h.done) break;  // an apply that gave up its wait: the iterate is wrong
         API_CUDA(C, cudaGraphLaunch(C->graph, st));
     }
     API_CUDA(C, cudaEventRecord(C->ev_t1, st));
@@ -156,18 +151,15 @@ fcm_status solve_one(fcm_ctx *C, const double *rhs, double tol, int maxit, doubl
     apply_K_dev(C, C->d_x, C->d_q, nullptr);
     fcm::cg_residual_norms(w, C->d_q, C->d_b, C->d_out2, st);
     API_CUDA(C, cudaMemcpyAsync(bb, C->d_out2, sizeof bb, cudaMemcpyDeviceToHost, st));
+    API_CUDA(C, cudaMemcpyAsync(C->h_err, C->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));  // of that K apply too
     API_CUDA(C, cudaStreamSynchronize(st));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, C->ev_t0, C->ev_t1);
     info.iterations = h.it;
     info.relres = h.relres;
     info.true_relres = bb[1] > 0.0 ? std::sqrt(bb[0] / bb[1]) : 0.0;
-    info.status = timed_out ? FCM_ETIMEOUT : h.status;
+    info.status = *C->h_err ? fcm::ctx_timeout(C, "fcm_pcg_solve") : h.status;
     info.seconds = ms * 1e-3;
-    if (timed_out) {
-        API_CUDA(C, cudaMemsetAsync(C->d_err, 0, sizeof(int), st));
-        C->err = "a Schwarz apply gave up waiting for a factor copy (bounded mbarrier wait); the iterate is not valid";
-    }
     return (fcm_status)info.status;
 }
 
@@ -210,6 +202,15 @@ void ctx_apply_K(fcm_ctx *C, const double *x, double *y) { apply_K_dev(C, x, y, 
 void ctx_apply_S(fcm_ctx *C, const double *r, double *z) { apply_S_dev(C, r, z, nullptr); }
 void ctx_apply_K_flag(fcm_ctx *C, const double *x, double *y, const int *stop) { apply_K_dev(C, x, y, stop); }
 void ctx_apply_S_flag(fcm_ctx *C, const double *r, double *z, const int *stop) { apply_S_dev(C, r, z, stop); }
+fcm_status ctx_timeout(fcm_ctx *C, const char *call)
+{
+    C->err = std::string(call) + (*C->h_err == kErrElement ? ": a K apply gave up waiting for an element matrix"
+                                                           : ": a Schwarz apply gave up waiting for a factor") +
+             " copy (bounded mbarrier wait); the result is not valid";
+    API_CUDA(C, cudaMemsetAsync(C->d_err, 0, sizeof(int), C->stream));
+    return FCM_ETIMEOUT;
+}
+
 fcm_status ctx_solve_one(fcm_ctx *C, const double *rhs, double tol, int maxit, double *u, fcm_solve_info &info)
 {
     return solve_one(C, rhs, tol, maxit, u, info);
@@ -433,7 +434,7 @@ fcm_status fcm_info(const fcm_ctx *C, fcm_info_t *out)
         int e = 0;
         if (cudaMemcpyAsync(&e, C->d_err, sizeof(int), cudaMemcpyDeviceToHost, C->stream) == cudaSuccess &&
             cudaStreamSynchronize(C->stream) == cudaSuccess)
-            out->device_error = e;
+            out->device_error = e != 0;
     }
     return FCM_OK;
 }
@@ -567,12 +568,7 @@ static fcm_status solve_multi(fcm_ctx *C, const double *rhs, int nr, double tol,
             API_CUDA(C, cudaMemcpyAsync(C->h_ms, C->d_ms, sizeof(CgScalars) * nr, cudaMemcpyDeviceToHost, st));
             API_CUDA(C, cudaMemcpyAsync(C->h_err, C->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
             API_CUDA(C, cudaStreamSynchronize(st));
-            if (*C->h_err) {
-                API_CUDA(C, cudaMemsetAsync(C->d_err, 0, sizeof(int), st));
-                C->err = "a Schwarz apply gave up waiting for a factor copy (bounded mbarrier wait); the iterates are not valid";
-                agg.status = FCM_ETIMEOUT;
-                return FCM_ETIMEOUT;
-            }
+            if (*C->h_err) return fcm::ctx_timeout(C, "fcm_pcg_solve");
             bool all = true;
             for (int k = 0; k < nr; ++k) all = all && C->h_ms[k].done;
             if (all) break;
@@ -590,7 +586,9 @@ static fcm_status solve_multi(fcm_ctx *C, const double *rhs, int nr, double tol,
         apply_K_dev(C, w[k].x, C->d_q, nullptr);
         fcm::cg_residual_norms(w[k], C->d_q, w[k].b, C->d_out2, st);
         API_CUDA(C, cudaMemcpyAsync(bb, C->d_out2, sizeof bb, cudaMemcpyDeviceToHost, st));
+        API_CUDA(C, cudaMemcpyAsync(C->h_err, C->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));  // of that K apply
         API_CUDA(C, cudaStreamSynchronize(st));
+        if (*C->h_err) return fcm::ctx_timeout(C, "fcm_pcg_solve");
         const CgScalars &h = C->h_ms[k];
         agg.iterations = std::max(agg.iterations, h.it);
         agg.relres = std::max(agg.relres, h.relres);

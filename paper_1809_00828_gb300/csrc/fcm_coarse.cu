@@ -637,19 +637,17 @@ fcm_status fcm_fpcg_solve(fcm_ctx *C, fcm_unet *net, double gamma, int coarse_it
     fk_newp_kernel<<<C->red_blocks, RT, 0, st>>>(C->d_p, zS, F->ring, n, F->d);
     CO_CUDA(C, cudaGetLastError());
     if ((s = fcg_graph(C, net, gamma, coarse_iters)) != FCM_OK) return s;
+    const auto timed_out = [&] {  // an apply gave up its wait (h_err): the iterate, or its residual, is not valid
+        C->last.status = ctx_timeout(C, "fcm_fpcg_solve");
+        cudaEventRecord(C->ev_out, st);
+        cudaStreamWaitEvent(C->ustream, C->ev_out, 0);
+        return (fcm_status)C->last.status;
+    };
     for (;;) {
         CO_CUDA(C, cudaMemcpyAsync(&h, F->d, sizeof h, cudaMemcpyDeviceToHost, st));
         CO_CUDA(C, cudaMemcpyAsync(C->h_err, C->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
         CO_CUDA(C, cudaStreamSynchronize(st));
-        if (*C->h_err) {
-            // a Schwarz apply gave up waiting for a factor copy: the iterate is not valid
-            CO_CUDA(C, cudaMemsetAsync(C->d_err, 0, sizeof(int), st));
-            C->err = "fcm_fpcg_solve: a Schwarz apply gave up waiting for a factor copy (bounded mbarrier wait)";
-            C->last.status = FCM_ETIMEOUT;
-            cudaEventRecord(C->ev_out, st);
-            cudaStreamWaitEvent(C->ustream, C->ev_out, 0);
-            return FCM_ETIMEOUT;
-        }
+        if (*C->h_err) return timed_out();
         if (h.stop) break;
         CO_CUDA(C, cudaGraphLaunch(F->graph, st));
     }
@@ -688,7 +686,9 @@ fcm_status fcm_fpcg_solve(fcm_ctx *C, fcm_unet *net, double gamma, int coarse_it
     if ((s = dot2(C, b, b, nullptr, nullptr, h2)) != FCM_OK) return s;
     const double bb = h2[0];
     sub_kernel<<<nblk(n), 256, 0, st>>>(F->c, b, q, n);
+    CO_CUDA(C, cudaMemcpyAsync(C->h_err, C->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));  // of that K apply
     if ((s = dot2(C, F->c, F->c, nullptr, nullptr, h2)) != FCM_OK) return s;
+    if (*C->h_err) return timed_out();
     float ms = 0.f;
     cudaEventElapsedTime(&ms, C->ev_f0, C->ev_f1);
     C->last.iterations = total;

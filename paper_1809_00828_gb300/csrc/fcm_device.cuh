@@ -66,7 +66,7 @@ struct KCells {
     const int *uncut;           // cell ids
     const CutCell *cut;         // element 0 (the reference matrix) for uncut cells taken along (k_dense_uncut)
     int n_uncut, n_cut;
-    int *err;                   // device flag, set to 1 by a bulk-copy wait that ran out
+    int *err;                   // device flag, set to kErrElement by a bulk-copy wait that ran out
     int wait_tries;             // polls of a bulk-copy wait before it gives up
     const int32_t *cell_elem;   // per cell, negative where inactive
     const double *modal;        // weight tables of the modal form (make_modal_tables; p <= 3)
@@ -186,6 +186,8 @@ cudaError_t schwarz_fold_factor(const double *F, int n, int prec, float *out, cu
 cudaError_t schwarz_prepare(int p);
 // polls of a bulk-copy wait before it gives up (default)
 constexpr int kWaitTries = 1 << 21;
+// values of the error flag: what gave up its wait
+constexpr int kErrFactor = 1, kErrElement = 2;
 void launch_mask_copy(const double *in, double *out, const uint8_t *mask, int64_t n, cudaStream_t s);
 // fcm_noalloc.cu: device address of the static scratch of fcm_apply_S_noalloc on the current device
 cudaError_t noalloc_scratch_address(double **out);
@@ -210,6 +212,8 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o);
 
 // fcm_capi.cu: operators and the plain PCG on a context's own work stream
 void ctx_apply_K(fcm_ctx *C, const double *x, double *y);
+// FCM_ETIMEOUT of `call` after a nonzero d_err was read into h_err: clears d_err, names what gave up in C->err
+fcm_status ctx_timeout(fcm_ctx *C, const char *call);
 void ctx_apply_S(fcm_ctx *C, const double *r, double *z);
 // the same, skipped on the device while *stop != 0 (stop may be null)
 void ctx_apply_K_flag(fcm_ctx *C, const double *x, double *y, const int *stop);
@@ -284,7 +288,7 @@ struct fcm_ctx {
     int64_t n_ff_factors = 0;        // factors stored as double-float pairs
     int64_t n_gemm_blocks = 0;       // blocks applied by the shared-factor GEMM
     double *d_jac = nullptr;         // diagonal part of S (element blocks), lattice; null if none
-    int *d_err = nullptr;            // set by a CTA (Schwarz or K apply) whose bulk-copy wait ran out
+    int *d_err = nullptr;            // set (kErr*) by a CTA (Schwarz or K apply) whose bulk-copy wait ran out
     double *noalloc_scratch = nullptr;  // device address of fcm_apply_S_noalloc's static scratch
     std::string noalloc_err;            // why it is null (problem too large, or the lookup failed)
     int device = 0;                     // CUDA device current at fcm_setup

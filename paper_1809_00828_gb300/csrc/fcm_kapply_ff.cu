@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
     }
     __syncthreads();
     if (!mbar_wait(&bar, 0, wait_tries)) {
-        atomicExch(err, 1);
+        atomicExch(err, kErrElement);
         mbar_wait(&bar, 0, kDrainTries);
         return;
     }

@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(fold_threads(P))
     }
     __syncthreads();
     if (!mbar_wait(&bar, 0, wait_tries)) {
-        atomicExch(err, 1);
+        atomicExch(err, kErrFactor);
         mbar_wait(&bar, 0, kDrainTries);
         return;
     }
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(gemm_threads(P))
                 if (!ok) {
                     // flag the apply as failed; the copies still in flight land before the CTA leaves
                     if (tid == 0) {
-                        atomicExch(err, 1);
+                        atomicExch(err, kErrFactor);
                         mbar_wait(&bar[s], (q >> 1) & 1, kDrainTries);
                         if (q + 1 < Q) mbar_wait(&bar[s ^ 1], ((q + 1) >> 1) & 1, kDrainTries);
                     }
@@ -1035,7 +1035,7 @@ __global__ void __launch_bounds__(TcCfg<P>::THREADS, TcCfg<P>::CTAS_PER_SM)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     failed = __syncthreads_or(failed || !ok || *reinterpret_cast<volatile int *>(flag));
     if (failed) {
-        if (threadIdx.x == 0) atomicExch(err, 1);
+        if (threadIdx.x == 0) atomicExch(err, kErrFactor);
     } else if (warp >= 1) {
         // warp w reads TMEM lanes 32 (w % 4) .. + 31 (columns m) and half (w - 1) / 4 of the rows, 16 at
         // a time, and writes them through a 32 x 17 transpose buffer: each store covers 16 rows of a block
