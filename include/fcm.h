@@ -323,7 +323,8 @@ fcm_status fcm_coarse_prolong(fcm_ctx *ctx, const float *cells_dev, double s, do
  * K_H is assembled on the first call by probing K with 375 coloured cell
  * vectors (each cell couples with the cells of its 5x5x5 neighbourhood) and
  * is kept in FP32 on the context (n_cells * 125 * 9 floats).  Returns
- * FCM_ENOMEM if it does not fit. */
+ * FCM_ENOMEM if it does not fit, FCM_ETIMEOUT (and keeps nothing) if one of those K
+ * applies gave up its bounded wait (fcm_set_wait_limit). */
 fcm_status fcm_coarse_apply(fcm_ctx *ctx, const float *x_cells_dev, float *y_cells_dev);
 
 /* Flexible PCG with a coarse correction: z = S r + P y, S the Additive-Schwarz

@@ -202,11 +202,16 @@ void ctx_apply_K(fcm_ctx *C, const double *x, double *y) { apply_K_dev(C, x, y, 
 void ctx_apply_S(fcm_ctx *C, const double *r, double *z) { apply_S_dev(C, r, z, nullptr); }
 void ctx_apply_K_flag(fcm_ctx *C, const double *x, double *y, const int *stop) { apply_K_dev(C, x, y, stop); }
 void ctx_apply_S_flag(fcm_ctx *C, const double *r, double *z, const int *stop) { apply_S_dev(C, r, z, stop); }
+std::string timeout_text(const char *call, int flag)
+{
+    return std::string(call) + (flag == kErrElement ? ": a K apply gave up waiting for an element matrix"
+                                                    : ": a Schwarz apply gave up waiting for a factor") +
+           " copy (bounded mbarrier wait); the result is not valid";
+}
+
 fcm_status ctx_timeout(fcm_ctx *C, const char *call)
 {
-    C->err = std::string(call) + (*C->h_err == kErrElement ? ": a K apply gave up waiting for an element matrix"
-                                                           : ": a Schwarz apply gave up waiting for a factor") +
-             " copy (bounded mbarrier wait); the result is not valid";
+    C->err = timeout_text(call, *C->h_err);
     API_CUDA(C, cudaMemsetAsync(C->d_err, 0, sizeof(int), C->stream));
     return FCM_ETIMEOUT;
 }

@@ -769,8 +769,11 @@ fcm_status coarse_ensure(fcm_ctx *C)
     cudaMemsetAsync(op->counter, 0, sizeof(unsigned), st);
     cudaMemsetAsync(op->sc, 0, sizeof(double) * 8, st);
     cudaMemsetAsync(op->KH, 0, sizeof(float) * kh_words, st);
-    double *ecell = nullptr;
-    if ((e = cudaMalloc(&ecell, sizeof(double) * n3)) != cudaSuccess) return fail(e);
+    double *ecell = nullptr;  // and the error flag of these K applies (d_err may hold that of an earlier apply)
+    if ((e = cudaMalloc(&ecell, sizeof(double) * (n3 + 1))) != cudaSuccess) return fail(e);
+    int *const err = C->kc.err;
+    C->kc.err = reinterpret_cast<int *>(ecell + n3);
+    cudaMemsetAsync(C->kc.err, 0, sizeof(int), st);
     // lattice scratch: the context's d_t (probe) and d_q (K times probe)
     for (int oz = 0; oz < 5; ++oz)
         for (int oy = 0; oy < 5; ++oy)
@@ -784,6 +787,8 @@ fcm_status coarse_ensure(fcm_ctx *C)
                 }
     diag_inverse_kernel<<<nb(ncell), 256, 0, st>>>(op->KH, op->Dinv, ncell);
     cudaEventRecord(t1, st);
+    cudaMemcpyAsync(C->h_err, C->kc.err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    C->kc.err = err;
     e = cudaStreamSynchronize(st);
     float ms = 0.f;
     cudaEventElapsedTime(&ms, t0, t1);
@@ -792,6 +797,11 @@ fcm_status coarse_ensure(fcm_ctx *C)
     cudaEventDestroy(t1);
     cudaFree(ecell);
     if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return fail(e);
+    if (*C->h_err) {  // K_H would be wrong: not kept, the next call assembles it again
+        coarse_free(op);
+        C->err = timeout_text("coarse operator", *C->h_err);
+        return FCM_ETIMEOUT;
+    }
     C->coarse = op;
     return coarse_ensure(C);  // the FP16 copy and the hierarchy, where asked for
 }

@@ -214,6 +214,8 @@ std::string build_preconditioner(fcm_ctx *C, const fcm_precond_opts &o);
 void ctx_apply_K(fcm_ctx *C, const double *x, double *y);
 // FCM_ETIMEOUT of `call` after a nonzero d_err was read into h_err: clears d_err, names what gave up in C->err
 fcm_status ctx_timeout(fcm_ctx *C, const char *call);
+// its message for a value of the error flag
+std::string timeout_text(const char *call, int flag);
 void ctx_apply_S(fcm_ctx *C, const double *r, double *z);
 // the same, skipped on the device while *stop != 0 (stop may be null)
 void ctx_apply_K_flag(fcm_ctx *C, const double *x, double *y, const int *stop);

@@ -1,5 +1,5 @@
 """Bounded waits of the double-float K apply (element matrices copied in bulk, p <= 2) outside the iterations: the true
-residual at the end of each solve.
+residual at the end of each solve, and the assembly of the coarse operator by probing K.
 
 A wait limit of 0 makes every K apply give up (the copies land, the kernels return), and a preconditioner without
 blocks (pure Jacobi) waits for nothing.  With b = 0 the solves stop before their first iteration, so the only K
@@ -42,3 +42,19 @@ def test_a_true_residual_that_timed_out_is_reported(kind):
     assert solve(zero)[3] == fcm.FCM_OK
     assert s.get_info()["device_error"] == 0
     s.close()
+
+
+def test_a_coarse_operator_from_timed_out_products_is_not_kept():
+    from paper_1809_00828_gb300 import fcm
+    s = _solver()
+    x = torch.from_numpy(I.random_vector(3, 3 * 8 ** 3)).float().cuda()
+    s.set_wait_limit(0)
+    with pytest.raises(fcm.FcmError) as e:
+        s.coarse_apply(x)
+    assert e.value.status == fcm.FCM_ETIMEOUT
+    s.set_wait_limit(-1)
+    y = s.coarse_apply(x)
+    fresh = _solver()
+    assert torch.equal(y, fresh.coarse_apply(x))
+    for q in (s, fresh):
+        q.close()
