@@ -40,3 +40,23 @@ def test_entries_that_are_not_free_are_ignored(p, n, precision, k):
         h = gx.clone()
         assert torch.equal(s.apply_S(h, out=h), z)
     s.close()
+
+
+@pytest.mark.parametrize("p,n", [(2, (7, 5, 6)), (3, (5, 4, 6))])
+@pytest.mark.parametrize("blocks", ["vertex", "element"])
+@pytest.mark.parametrize("bc", [0, 1])  # one clamped face; three faces with a fixed component each
+def test_shared_factors_ignore_entries_that_are_not_free(p, n, blocks, bc):
+    """The shared factors' tensor-core product on blocks at fixed faces: NaN in the entries that are not free gives
+    the bits that zeros give."""
+    from paper_1809_00828_gb300 import fcm
+    w = I.Workload("shared", n, p, 1.0, I.uncut(), 1e-9, bc=bc)
+    s = fcm.Solver(w)
+    s.precond_build(precision="mixed", blocks=blocks, launch="concurrent")
+    assert s.info["n_cells_cut"] == 0 and s.info["n_gemm_blocks"] > 0 and s.info["n_blocks_fp32"] > 0
+    free = O.Problem.from_workload(w).free_lat
+    x = np.zeros(s.n)
+    x[free] = I.random_vector(11, len(free))
+    z = s.apply_S(torch.from_numpy(x).cuda())
+    x[np.setdiff1d(np.arange(s.n), free)] = np.nan
+    assert float(z.abs().max()) > 0 and torch.equal(s.apply_S(torch.from_numpy(x).cuda()), z)
+    s.close()
