@@ -425,9 +425,8 @@ fcm_status fcm_info(const fcm_ctx *C, fcm_info_t *out)
     {
         const fcm::SchwarzPlan &pl = C->plan;
         const bool tc = pl.n_tc_tiles > 0;
-        const int own = (fcm::schwarz_uses_rows_kernel(C->p) ? pl.n_row_items : pl.n_col_items) > 0;
         out->s_apply_launches = C->have_precond ? (tc ? 1 : 0) + ((tc ? pl.n_tiles32_plain : pl.n_tiles32) > 0) +
-                                                      (pl.n_tiles64 > 0) + (pl.n_fold32 > 0) + (pl.n_fold_ff > 0) + own + 1
+                                                      (pl.n_tiles64 > 0) + fcm::schwarz_own_launches(C->p, pl) + 1
                                                 : 0;
         const int k = (C->kc.n_uncut > 0) + (C->kc.n_cut > 0) + 1;  // uncut cells, cut cells, sum
         out->k_apply_launches = k;

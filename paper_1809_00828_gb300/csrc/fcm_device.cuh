@@ -177,6 +177,8 @@ bool schwarz_tc_supported(int p);
 int64_t schwarz_tc_factor_floats(int p, int n);
 cudaError_t schwarz_tc_factor(int p, const double *F, int n, float *ft, cudaStream_t s);
 int schwarz_rows_threads();
+// launches of one right-hand side's own blocks
+int schwarz_own_launches(int p, const SchwarzPlan &pl);
 // whether own FP32 and double-float factors are stored folded; floats of one (prec 1 or 2), and the kernel
 // that folds an FP64 factor (rows padded to factor_ld<double>(n))
 bool schwarz_folds(int p);

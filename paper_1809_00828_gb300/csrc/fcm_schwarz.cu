@@ -388,15 +388,12 @@ __device__ __forceinline__ void cols_ff(const double *__restrict__ r, const uint
 }
 
 template <int P, int NR>
-__global__ void __launch_bounds__(cols_threads(P))
-    schwarz_cols_kernel(const double *__restrict__ r, int64_t nlat, int nr, const double *__restrict__ f64,
-                        const float *__restrict__ f32, const PatchRec *__restrict__ slots,
-                        const int2 *__restrict__ items, Grid3 g, int rule, double *__restrict__ zb, int zs,
-                        int64_t zsize, int pairs, const uint8_t *__restrict__ xmask, const int *__restrict__ done)
+__device__ __forceinline__ void cols_item(const double *__restrict__ r, int64_t nlat, int nr,
+                                          const double *__restrict__ f64, const float *__restrict__ f32,
+                                          const PatchRec *__restrict__ slots, int2 it, const Grid3 &g, int rule,
+                                          double *__restrict__ zb, int zs, int64_t zsize, int pairs,
+                                          const uint8_t *__restrict__ xmask, unsigned char *smem)
 {
-    extern __shared__ __align__(1024) unsigned char smem[];
-    if (done && *done) return;
-    const int2 it = items[blockIdx.x];
     const PatchRec pr = slots[it.x];
     const SBox b = sbox(rule, P, g, pr.v);
     double *zout = zb + (size_t)it.x * zs;
@@ -407,6 +404,18 @@ __global__ void __launch_bounds__(cols_threads(P))
     else cols_plain<P, NR, double>(r, xm, nlat, nr, f64 + pr.off, b, g, it.y, zout, zsize, pairs, smem);
 }
 
+template <int P, int NR>
+__global__ void __launch_bounds__(cols_threads(P))
+    schwarz_cols_kernel(const double *__restrict__ r, int64_t nlat, int nr, const double *__restrict__ f64,
+                        const float *__restrict__ f32, const PatchRec *__restrict__ slots,
+                        const int2 *__restrict__ items, Grid3 g, int rule, double *__restrict__ zb, int zs,
+                        int64_t zsize, int pairs, const uint8_t *__restrict__ xmask, const int *__restrict__ done)
+{
+    extern __shared__ __align__(1024) unsigned char smem[];
+    if (done && *done) return;
+    cols_item<P, NR>(r, nlat, nr, f64, f32, slots, items[blockIdx.x], g, rule, zb, zs, zsize, pairs, xmask, smem);
+}
+
 // ---- phase 1b': own FP32 and double-float factors of small blocks (p <= 2), folded (fcm_sym.cuh)
 //
 // Half of a symmetric factor's bytes, which bound the apply: a CTA per block, a thread per row, the columns in
@@ -415,23 +424,26 @@ __global__ void __launch_bounds__(cols_threads(P))
 
 __host__ __device__ constexpr int fold_threads(int P) { return rnd32(sbox_max(P)); }
 
+// entries of shared memory of a block: the folded factor and the residuals
+__host__ __device__ constexpr int fold_smem(int P, int NR)
+{
+    return fold_entries(sbox_max(P)) + (sbox_max(P) + 3) / 4 * 4 * NR;
+}
+
 template <int P, int NR, class T>
-__global__ void __launch_bounds__(fold_threads(P))
-    schwarz_fold_kernel(const double *__restrict__ r, int64_t nlat, int nr, const float *__restrict__ f32,
-                        const FoldItem *__restrict__ items, Grid3 g, double *__restrict__ zb, int zs, int64_t zsize,
-                        int pairs, const uint8_t *__restrict__ xmask, int *err, int wait_tries,
-                        const int *__restrict__ done)
+__device__ __forceinline__ void fold_block(const double *__restrict__ r, int64_t nlat, int nr,
+                                           const float *__restrict__ f32, const FoldItem &it, const Grid3 &g,
+                                           double *__restrict__ zb, int zs, int64_t zsize, int pairs,
+                                           const uint8_t *__restrict__ xmask, int *err, int wait_tries, T *m,
+                                           uint64_t *bar)
 {
     constexpr int NM = sbox_max(P);
-    if (done && *done) return;
-    __shared__ __align__(16) T m[fold_entries(NM)], xs[(NM + 3) / 4 * 4 * NR];
-    __shared__ uint64_t bar;
-    const FoldItem it = items[blockIdx.x];
+    T *xs = m + fold_entries(NM);
     const int n = 3 * it.d[0] * it.d[1] * it.d[2], bytes = fold_entries(n) * (int)sizeof(T);
     if (threadIdx.x == 0) {
-        mbar_init(&bar);
-        mbar_expect(&bar, bytes);
-        bulk_g2s(m, f32 + it.off, bytes, &bar);
+        mbar_init(bar);
+        mbar_expect(bar, bytes);
+        bulk_g2s(m, f32 + it.off, bytes, bar);
     }
     for (int t = threadIdx.x; t < n; t += blockDim.x) {
         const int l = t / 3;
@@ -456,9 +468,9 @@ __global__ void __launch_bounds__(fold_threads(P))
         }
     }
     __syncthreads();
-    if (!mbar_wait(&bar, 0, wait_tries)) {
+    if (!mbar_wait(bar, 0, wait_tries)) {
         atomicExch(err, kErrFactor);
-        mbar_wait(&bar, 0, kDrainTries);
+        mbar_wait(bar, 0, kDrainTries);
         return;
     }
     const int t0 = threadIdx.x & ~31;
@@ -484,6 +496,44 @@ __global__ void __launch_bounds__(fold_threads(P))
         for (int k = 0; k < NR; ++k)
             if (k < nr && row < n) put_ff(zout + k * zsize, row, S[k], C[k], pairs);
     }
+}
+
+template <int P, int NR, class T>
+__global__ void __launch_bounds__(fold_threads(P))
+    schwarz_fold_kernel(const double *__restrict__ r, int64_t nlat, int nr, const float *__restrict__ f32,
+                        const FoldItem *__restrict__ items, Grid3 g, double *__restrict__ zb, int zs, int64_t zsize,
+                        int pairs, const uint8_t *__restrict__ xmask, int *err, int wait_tries,
+                        const int *__restrict__ done)
+{
+    if (done && *done) return;
+    __shared__ __align__(16) T m[fold_smem(P, NR)];
+    __shared__ uint64_t bar;
+    fold_block<P, NR, T>(r, nlat, nr, f32, items[blockIdx.x], g, zb, zs, zsize, pairs, xmask, err, wait_tries, m, &bar);
+}
+
+// All own blocks in one launch, for a grid of few of them: n32 + n_ff folded ones, then those that stream their rows.
+template <int P, int NR>
+__global__ void __launch_bounds__(fold_threads(P))
+    schwarz_own_kernel(const double *__restrict__ r, int64_t nlat, int nr, const double *__restrict__ f64,
+                       const float *__restrict__ f32, const FoldItem *__restrict__ fold, int n32, int n_ff,
+                       const PatchRec *__restrict__ slots, const int2 *__restrict__ items, Grid3 g, int rule,
+                       double *__restrict__ zb, int zs, int64_t zsize, int pairs, const uint8_t *__restrict__ xmask,
+                       int *err, int wait_tries, const int *__restrict__ done)
+{
+    static_assert(fold_threads(P) == cols_threads(P), "one block shape");
+    if (done && *done) return;
+    __shared__ __align__(16) float2 m[fold_smem(P, NR)];
+    __shared__ uint64_t bar;
+    static_assert(sizeof(m) >= factor_ld<double>(sbox_max(P)) * NR * 8, "residuals of a streamed block");
+    const int b = blockIdx.x;
+    if (b < n32)
+        fold_block<P, NR, float>(r, nlat, nr, f32, fold[b], g, zb, zs, zsize, pairs, xmask, err, wait_tries,
+                                 reinterpret_cast<float *>(m), &bar);
+    else if (b < n32 + n_ff)
+        fold_block<P, NR, float2>(r, nlat, nr, f32, fold[b], g, zb, zs, zsize, pairs, xmask, err, wait_tries, m, &bar);
+    else
+        cols_item<P, NR>(r, nlat, nr, f64, f32, slots, items[b - n32 - n_ff], g, rule, zb, zs, zsize, pairs, xmask,
+                         reinterpret_cast<unsigned char *>(m));
 }
 
 // folded copy of an FP64 factor (rows padded to factor_ld<double>): FP32, or float pairs
@@ -1112,6 +1162,15 @@ void cols_launch(const double *r, int64_t nlat, int nr, const double *f64, const
 }
 
 template <int P, int NR>
+void own_launch(const double *r, int64_t nlat, int nr, const double *f64, const float *f32, const SchwarzPlan &pl,
+                double *zb, int64_t zsize, const uint8_t *xm, const int *done, cudaStream_t s)
+{
+    schwarz_own_kernel<P, NR><<<pl.n_fold32 + pl.n_fold_ff + pl.n_col_items, fold_threads(P), 0, s>>>(
+        r, nlat, nr, f64, f32, pl.fold_items, pl.n_fold32, pl.n_fold_ff, pl.slots, pl.col_items, pl.g, pl.rule, zb, pl.zs,
+        zsize, pl.pairs, xm, pl.err, pl.wait_tries, done);
+}
+
+template <int P, int NR>
 void fold_launch(const double *r, int64_t nlat, int nr, const float *f32, const SchwarzPlan &pl, double *zb,
                  int64_t zsize, const uint8_t *xm, const int *done, cudaStream_t s)
 {
@@ -1122,6 +1181,20 @@ void fold_launch(const double *r, int64_t nlat, int nr, const float *f32, const 
         schwarz_fold_kernel<P, NR, float2><<<pl.n_fold_ff, fold_threads(P), 0, s>>>(
             r, nlat, nr, f32, pl.fold_items + pl.n_fold32, pl.g, zb, pl.zs, zsize, pl.pairs, xm, pl.err, pl.wait_tries,
             done);
+}
+
+// Whether one launch takes the own blocks of all kinds.  Kinds launched one after the other cost a small grid a
+// launch's latency each; many blocks fill the GPU with one kind, whose registers and shared memory fit it (80^3
+// p = 2: 246 + 211 us apart, 740 in one).  Measured apart / in one launch, us: element blocks, p = 2, 121 blocks
+// 23.9 / 21.9, 822 blocks 28.5 / 24.0, 1,880 blocks 29.9 / 28.0; p = 1, 192 blocks 20.6 / 17.1, 3,344 blocks 22.6 /
+// 19.4.  Beside shared-factor products the line is lower: vertex patches, p = 2, six right-hand sides, 521 blocks
+// 236 / 236, 1,104 blocks 248 / 316.
+bool own_together(int p, const SchwarzPlan &pl)
+{
+    const int fold = pl.n_fold32 + pl.n_fold_ff;
+    const bool beside = pl.n_tiles32 + pl.n_tiles64 + pl.n_tc_tiles > 0;
+    return (pl.n_fold32 > 0) + (pl.n_fold_ff > 0) + (pl.n_col_items > 0) > 1 && fold > 0 &&
+           fold + pl.n_col_items <= 152 * (beside ? 4 : p == 1 ? 24 : 12);
 }
 
 template <int P>
@@ -1141,9 +1214,13 @@ void apply_p(const double *r, double *z, int64_t nlat, int nr, const double *f64
     } else if (gemm) {
         gemm_launch<P>(r, nlat, nr, f64, f32, pl, zb, zsize, xm, done, s);
     }
+    const bool together = own_together(P, pl);
     if constexpr (P <= 2)
-        with_columns(nr, [&](auto c) { fold_launch<P, decltype(c)::value>(r, nlat, nr, f32, pl, zb, zsize, xm, done, s); });
-    if (own) {
+        with_columns(nr, [&](auto c) {
+            if (together) own_launch<P, decltype(c)::value>(r, nlat, nr, f64, f32, pl, zb, zsize, xm, done, s);
+            else fold_launch<P, decltype(c)::value>(r, nlat, nr, f32, pl, zb, zsize, xm, done, s);
+        });
+    if (own && !together) {
         if (P == 3 && nr == 1) {
             if constexpr (P == 3)
                 schwarz_rows_kernel<P><<<pl.n_row_items, kRowsThreads, 0, s>>>(
@@ -1241,6 +1318,12 @@ cudaError_t schwarz_fold_factor(const double *F, int n, int prec, float *out, cu
     if (prec == 2) fold_factor_kernel<float2><<<grid, 256, 0, s>>>(F, reinterpret_cast<float2 *>(out), n);
     else fold_factor_kernel<float><<<grid, 256, 0, s>>>(F, out, n);
     return cudaGetLastError();
+}
+
+int schwarz_own_launches(int p, const SchwarzPlan &pl)
+{
+    if (own_together(p, pl)) return 1;
+    return (pl.n_fold32 > 0) + (pl.n_fold_ff > 0) + ((schwarz_uses_rows_kernel(p) ? pl.n_row_items : pl.n_col_items) > 0);
 }
 
 int schwarz_rows_threads() { return kRowsThreads; }

@@ -69,3 +69,26 @@ def test_wait_limit_of_the_streamed_factors_and_matrices():
     assert its == its_ref and torch.equal(u, u_ref) and torch.equal(s.apply_K(b), y_ref)
     assert s.get_info()["device_error"] == 0
     s.close()
+
+
+@pytest.mark.parametrize("p,n", [(1, (5, 4, 6)), (2, (3, 4, 3))])
+@pytest.mark.parametrize("precision", ["mixed", "mixed_fp64"])
+def test_own_blocks_of_several_kinds_in_one_launch(p, n, precision):
+    """A small grid's folded FP32 blocks and its double-float or FP64 ones share a launch (then one for the sum)."""
+    from paper_1809_00828_gb300 import fcm
+    w = I.Workload("s_own", n, p, 1e-6, I.random_sphere_voids(9, 3, 0.15, 0.3, octree_depth=2), 1e-9, hi=(1.0, 1.2, 0.9))
+    P = O.Problem.from_workload(w)
+    P.precond_build(3, 1e-13, 0.9)
+    conds = sorted(P.block(b)[2][0] for b in range(P.nblocks()))
+    s = fcm.Solver(w)
+    s.precond_build(precision=precision, cond_fp64=conds[len(conds) // 2], blocks="element", eta_bar=0.9)
+    kinds = s.info["n_blocks_fp32"], s.info["n_factors"] - s.info["n_blocks_fp32"]
+    assert min(kinds) > 0 and s.info["n_gemm_blocks"] == 0 and s.info["s_apply_launches"] == 2
+    for nr in (1, 3, 8):
+        X = np.stack([I.random_vector(90 + k, s.n) for k in range(nr)])
+        Z = s.apply_S(torch.from_numpy(X.reshape(-1)).cuda()).cpu().numpy().reshape(nr, -1)
+        for x, z in zip(X, Z):
+            ref = P.apply_S(x[P.free_lat])
+            bound = dof_bound(P, x[P.free_lat], u_factor=2.0 ** -20) + 1e-14 * np.abs(ref).max()
+            assert np.all(np.abs(z[P.free_lat] - ref) <= bound), nr
+    s.close()
