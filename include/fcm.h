@@ -291,9 +291,17 @@ fcm_status fcm_unet_create(const fcm_unet_desc *desc, void *cuda_stream, fcm_une
 /* Number of parameters (all weights then all biases, layer by layer). */
 fcm_status fcm_unet_params(const fcm_unet *net, int64_t *count);
 /* Copy the FP32 master parameters (and, if g_host != NULL, their gradients) to host memory.
- * FCM_ETIMEOUT: a convolution since the last call gave up its bounded wait for the tensor core, so an
- * output or gradient since then is not valid (the parameters are copied all the same). */
+ * FCM_ETIMEOUT as fcm_unet_status (the parameters are copied all the same). */
 fcm_status fcm_unet_get(fcm_unet *net, float *w_host, float *g_host);
+/* Waits for the network's stream.  FCM_ETIMEOUT: a convolution gave up its bounded wait for the tensor core,
+ * so an output or gradient since the last report is not valid.  The report is given once, by whichever comes
+ * first: this call, fcm_unet_get, or (without waiting, for a convolution that has given up by then, and doing
+ * nothing else) fcm_unet_forward, fcm_unet_backward or fcm_unet_adam.  An Adam step queued after such a
+ * convolution and before its report leaves the parameters as they are.  Inside fcm_fpcg_solve the solve
+ * itself returns FCM_ETIMEOUT. */
+fcm_status fcm_unet_status(fcm_unet *net);
+/* Polls of that wait (as fcm_set_wait_limit: default 2^21, 0 gives up at once, < 0 restores the default). */
+fcm_status fcm_unet_set_wait_limit(fcm_unet *net, int tries);
 /* Replace the FP32 master parameters from host memory (BF16 copies are refreshed). */
 fcm_status fcm_unet_set(fcm_unet *net, const float *w_host);
 /* out_dev[batch][out_ch][nz][ny][nx] = U-Net(in_dev[batch][in_ch][nz][ny][nx]); keeps the activations

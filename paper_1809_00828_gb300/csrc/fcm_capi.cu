@@ -204,9 +204,11 @@ void ctx_apply_K_flag(fcm_ctx *C, const double *x, double *y, const int *stop) {
 void ctx_apply_S_flag(fcm_ctx *C, const double *r, double *z, const int *stop) { apply_S_dev(C, r, z, stop); }
 std::string timeout_text(const char *call, int flag)
 {
-    return std::string(call) + (flag == kErrElement ? ": a K apply gave up waiting for an element matrix"
-                                                    : ": a Schwarz apply gave up waiting for a factor") +
-           " copy (bounded mbarrier wait); the result is not valid";
+    return std::string(call) +
+           (flag == kErrConv      ? ": a convolution gave up waiting for the tensor core"
+            : flag == kErrElement ? ": a K apply gave up waiting for an element matrix copy"
+                                  : ": a Schwarz apply gave up waiting for a factor copy") +
+           " (bounded mbarrier wait); the result is not valid";
 }
 
 fcm_status ctx_timeout(fcm_ctx *C, const char *call)

@@ -602,15 +602,15 @@ fcm_status fcm_fpcg_solve(fcm_ctx *C, fcm_unet *net, double gamma, int coarse_it
     FcgState *F = C->fcg;
     cudaStream_t st = C->stream;
     const int64_t n = C->nlat;
-    // the network runs on the solver's stream for the duration of the solve
+    // the network runs on the solver's stream for the duration of the solve, and reports to its error flag
     struct Restore {
         fcm_unet *n;
         cudaStream_t s;
         ~Restore()
         {
-            if (n) unet_set_stream(n, s);
+            if (n) unet_bind(n, s, nullptr);
         }
-    } restore{net, net ? unet_set_stream(net, st) : nullptr};
+    } restore{net, net ? unet_bind(net, st, C->d_err) : nullptr};
 
     double *x = C->d_x, *r = C->d_r, *zS = C->d_z, *q = C->d_q, *b = C->d_b;
     CO_CUDA(C, cudaMemsetAsync(C->d_err, 0, sizeof(int), st));  // earlier fcm_apply_S failures are not this solve's

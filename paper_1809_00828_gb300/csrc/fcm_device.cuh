@@ -189,7 +189,7 @@ cudaError_t schwarz_prepare(int p);
 // polls of a bulk-copy wait before it gives up (default)
 constexpr int kWaitTries = 1 << 21;
 // values of the error flag: what gave up its wait
-constexpr int kErrFactor = 1, kErrElement = 2;
+constexpr int kErrFactor = 1, kErrElement = 2, kErrConv = 3;
 void launch_mask_copy(const double *in, double *out, const uint8_t *mask, int64_t n, cudaStream_t s);
 // fcm_noalloc.cu: device address of the static scratch of fcm_apply_S_noalloc on the current device
 cudaError_t noalloc_scratch_address(double **out);
@@ -225,7 +225,7 @@ void ctx_apply_S_flag(fcm_ctx *C, const double *r, double *z, const int *stop);
 fcm_status ctx_solve_one(fcm_ctx *C, const double *rhs, double tol, int maxit, double *u, fcm_solve_info &info);
 
 // fcm_unet.cu: redirect a network's launches to stream s; returns the previous stream
-cudaStream_t unet_set_stream(fcm_unet *N, cudaStream_t s);
+cudaStream_t unet_bind(fcm_unet *N, cudaStream_t s, int *err);
 // identity of a network and of its current activation buffers (changes when they are reallocated)
 void unet_identity(const fcm_unet *N, uint64_t *serial, uint64_t *gen);
 

@@ -108,15 +108,23 @@ __device__ __forceinline__ void split3(float x, uint32_t &hi, uint32_t &mid, uin
     }
 }
 
+// A convolution's wait for the tensor core: polls before it gives up, and the flags it then sets: `err` (device) to
+// `code`, `seen` (pinned host memory, may be null) to 1.
+struct ConvWait {
+    int *err, *seen;
+    int code, tries;
+};
+
 template <int ZT>
 __global__ void __launch_bounds__(kConvThreads, 2)
     conv3_tc_kernel(ConvSrc src, const uint4 *__restrict__ w, const float *__restrict__ bias, float *__restrict__ out,
-                    int cin, int cout, int nx, int ny, int nz, int relu, int *err)
+                    int cin, int cout, int nx, int ny, int nz, int relu, ConvWait wait)
 {
     constexpr int HV = conv_hv(ZT);
     extern __shared__ __align__(1024) unsigned char csm[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(csm);
     uint32_t *slot = reinterpret_cast<uint32_t *>(csm + 8);
+    volatile int *gave_up = reinterpret_cast<int *>(csm + 12);  // the 16 channels at which a wait ran out, else nch
     unsigned char *A = csm + 1024, *W = A + conv_a_bytes(ZT);
     const int nb = conv_nb(cout), nch = up16(cin) / 16;
     const int tx = (nx + kTX - 1) / kTX, ty = (ny + kTY - 1) / kTY;
@@ -124,7 +132,10 @@ __global__ void __launch_bounds__(kConvThreads, 2)
     const int b = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t S = (int64_t)nx * ny * nz, S2 = (int64_t)(nx >> 1) * (ny >> 1) * (nz >> 1);
     const uint32_t cols = 4 * ZT * nb <= 64 ? 64 : 4 * ZT * nb <= 128 ? 128 : 256;
-    if (tid == 0) mbar_init(bar);
+    if (tid == 0) {
+        mbar_init(bar);
+        *gave_up = nch;
+    }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols)
                      : "memory");
@@ -184,6 +195,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
         // the tensor core reads shared memory through the async proxy
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
+        if (*gave_up < ch) break;  // the same for all threads: what they write below is at least ch
         if (warp == 0 && tc_elect()) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // FP32 accumulator, BF16 A and B, both K-major, M = 128, N = nb .. 3 nb
@@ -209,9 +221,11 @@ __global__ void __launch_bounds__(kConvThreads, 2)
             tc_commit(bar);
         }
         __syncwarp();
-        if (!mbar_wait(bar, ch & 1, kWaitTries)) {
-            atomicExch(err, 1);  // the products still in flight land before shared memory is written again
-            mbar_wait(bar, ch & 1, kDrainTries);
+        if (!mbar_wait(bar, ch & 1, wait.tries)) {
+            *gave_up = ch;
+            atomicExch(wait.err, wait.code);
+            if (wait.seen) *reinterpret_cast<volatile int *>(wait.seen) = 1;
+            mbar_wait(bar, ch & 1, kDrainTries);  // the products still in flight land before the CTA leaves
         }
         __syncwarp();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -520,10 +534,11 @@ __global__ void to_bf16_kernel(const float *a, __nv_bfloat16 *b, int64_t n)
         b[i] = __float2bfloat16_rn(a[i]);
 }
 
-// Adam (Kingma & Ba, 2015) with bias correction.
+// Adam (Kingma & Ba, 2015) with bias correction; nothing if a convolution gave up its wait (*err): g is not valid.
 __global__ void adam_kernel(float *w, const float *g, float *m, float *v, int64_t n, float lr, float b1, float b2,
-                            float eps, float c1, float c2)
+                            float eps, float c1, float c2, const int *err)
 {
+    if (*err) return;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -560,7 +575,9 @@ struct fcm_unet {
     __nv_bfloat16 *tiles = nullptr;  // weight tiles of every layer (conv_tiles_kernel), made with w16
     float *part = nullptr;           // partial sums of a weight gradient
     float *host = nullptr;           // pinned copy of parameters and gradients for fcm_unet_get (made on first use)
-    int *err = nullptr;              // set by a convolution whose wait for the tensor core ran out
+    int *err = nullptr;              // set by a convolution whose wait for the tensor core ran out, until reported
+    int *seen = nullptr;             // the same in pinned host memory
+    ConvWait wait = {};              // what the convolutions get: these flags, or those of the solve they run in
     // activations for the current shape
     int B = 0, n[3] = {0, 0, 0};
     std::vector<float *> act;  // owned buffers
@@ -666,7 +683,7 @@ void conv_launch(fcm_unet *N, const ConvSrc &src, int64_t tiles, const float *bi
         if (cost(k) < cost(zt)) zt = k;
     const auto kernel = zt == 3 ? conv3_tc_kernel<3> : zt == 2 ? conv3_tc_kernel<2> : conv3_tc_kernel<1>;
     const dim3 grid((unsigned)(txy * ((nz + zt - 1) / zt)), conv_blocks(cout), N->B);
-    kernel<<<grid, kConvThreads, conv_smem(zt, nb), N->stream>>>(src, w, bias, out, cin, cout, nx, ny, nz, relu, N->err);
+    kernel<<<grid, kConvThreads, conv_smem(zt, nb), N->stream>>>(src, w, bias, out, cin, cout, nx, ny, nz, relu, N->wait);
 }
 
 void conv_fwd(fcm_unet *N, int layer, const ConvSrc &src, float *out, int l, bool relu)
@@ -729,10 +746,13 @@ void unet_identity(const fcm_unet *N, uint64_t *serial, uint64_t *gen)
     *gen = N ? N->act_gen : 0;
 }
 
-cudaStream_t unet_set_stream(fcm_unet *N, cudaStream_t s)
+cudaStream_t unet_bind(fcm_unet *N, cudaStream_t s, int *err)
 {
     cudaStream_t old = N->stream;
     N->stream = s;
+    N->wait.err = err ? err : N->err;
+    N->wait.seen = err ? nullptr : N->seen;
+    N->wait.code = kErrConv;
     return old;
 }
 }  // namespace fcm
@@ -745,6 +765,22 @@ cudaStream_t unet_set_stream(fcm_unet *N, cudaStream_t s)
             return e_ == cudaErrorMemoryAllocation ? FCM_ENOMEM : FCM_ECUDA;                  \
         }                                                                                     \
     } while (0)
+
+namespace {
+
+// FCM_ETIMEOUT, once, if a convolution is known to have given up its wait: takes both flags back (the device's in
+// stream order, so that an Adam step queued behind the convolution still sees it)
+fcm_status unet_report(fcm_unet *N)
+{
+    volatile int *seen = N->seen;
+    if (N->wait.seen != N->seen || !*seen) return FCM_OK;
+    *seen = 0;
+    UN_CUDA(cudaMemsetAsync(N->err, 0, sizeof(int), N->stream));
+    fcm_unet_last_error() = timeout_text("U-Net", kErrConv);
+    return FCM_ETIMEOUT;
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -816,6 +852,10 @@ fcm_status fcm_unet_create(const fcm_unet_desc *d, void *cuda_stream, fcm_unet *
     if ((e = cudaMalloc((void **)&N->part, sizeof(float) * npart)) != cudaSuccess) return fail(e);
     if ((e = cudaMalloc((void **)&N->err, sizeof(int))) != cudaSuccess) return fail(e);
     if ((e = cudaMemsetAsync(N->err, 0, sizeof(int), N->stream)) != cudaSuccess) return fail(e);
+    if ((e = cudaMallocHost((void **)&N->seen, sizeof(int))) != cudaSuccess) return fail(e);
+    *N->seen = 0;
+    N->wait.tries = kWaitTries;
+    unet_bind(N, N->stream, nullptr);
     if ((e = cudaFuncSetAttribute(conv3_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWRun)) != cudaSuccess)
         return fail(e);
     if ((e = cudaFuncSetAttribute(conv3_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -845,19 +885,27 @@ fcm_status fcm_unet_get(fcm_unet *N, float *w_host, float *g_host)
     if (!N || !w_host) return FCM_EINVAL;
     // through pinned memory: a copy to the caller's pageable buffers runs at 3.4 GB/s (2 MB each, 1.2 ms)
     const size_t bytes = sizeof(float) * N->nparam;
-    if (!N->host) UN_CUDA(cudaMallocHost((void **)&N->host, 2 * bytes + sizeof(int)));
-    int &err = *reinterpret_cast<int *>(N->host + 2 * N->nparam);
+    if (!N->host) UN_CUDA(cudaMallocHost((void **)&N->host, 2 * bytes));
     UN_CUDA(cudaMemcpyAsync(N->host, N->w, bytes, cudaMemcpyDeviceToHost, N->stream));
     if (g_host) UN_CUDA(cudaMemcpyAsync(N->host + N->nparam, N->g, bytes, cudaMemcpyDeviceToHost, N->stream));
-    UN_CUDA(cudaMemcpyAsync(&err, N->err, sizeof(int), cudaMemcpyDeviceToHost, N->stream));
     UN_CUDA(cudaStreamSynchronize(N->stream));
     std::memcpy(w_host, N->host, bytes);
     if (g_host) std::memcpy(g_host, N->host + N->nparam, bytes);
-    if (err) {
-        UN_CUDA(cudaMemsetAsync(N->err, 0, sizeof(int), N->stream));
-        fcm_unet_last_error() = "a convolution gave up waiting for the tensor core (bounded wait); its output is not valid";
-        return FCM_ETIMEOUT;
-    }
+    return unet_report(N);
+}
+
+fcm_status fcm_unet_status(fcm_unet *N)
+{
+    if (!N) return FCM_EINVAL;
+    UN_CUDA(cudaStreamSynchronize(N->stream));
+    return unet_report(N);
+}
+
+fcm_status fcm_unet_set_wait_limit(fcm_unet *N, int tries)
+{
+    if (!N) return FCM_EINVAL;
+    N->wait.tries = tries < 0 ? kWaitTries : tries;
+    ++N->act_gen;  // graphs that captured launches with another limit are captured again
     return FCM_OK;
 }
 
@@ -878,6 +926,8 @@ fcm_status fcm_unet_forward(fcm_unet *N, const float *in, int B, int nx, int ny,
         fcm_unet_last_error() = "fcm_unet_forward: spatial sizes must be positive multiples of 2^(levels-1)";
         return FCM_EINVAL;
     }
+    const fcm_status s = unet_report(N);
+    if (s != FCM_OK) return s;
     UN_CUDA(ensure_shape(N, B, nx, ny, nz));
     const int L = N->levels;
     N->input = in;
@@ -906,6 +956,8 @@ fcm_status fcm_unet_backward(fcm_unet *N, const float *gout, float *gin)
         fcm_unet_last_error() = "fcm_unet_backward: call fcm_unet_forward first";
         return N ? FCM_ESTATE : FCM_EINVAL;
     }
+    const fcm_status s = unet_report(N);
+    if (s != FCM_OK) return s;
     const int L = N->levels, B = N->B;
     float *gtop = (L >= 2) ? N->gdB[0] : N->geB[0];
     const float *top = (L >= 2) ? N->dB[0] : N->eB[0];
@@ -947,8 +999,10 @@ fcm_status fcm_unet_zero_grad(fcm_unet *N)
 fcm_status fcm_unet_adam(fcm_unet *N, float lr, float b1, float b2, float eps, int step)
 {
     if (!N || step < 1) return FCM_EINVAL;
+    const fcm_status s = unet_report(N);
+    if (s != FCM_OK) return s;
     const float c1 = 1.f - std::pow(b1, (float)step), c2 = 1.f - std::pow(b2, (float)step);
-    adam_kernel<<<blocks_for(N->nparam), 256, 0, N->stream>>>(N->w, N->g, N->m, N->v, N->nparam, lr, b1, b2, eps, c1, c2);
+    adam_kernel<<<blocks_for(N->nparam), 256, 0, N->stream>>>(N->w, N->g, N->m, N->v, N->nparam, lr, b1, b2, eps, c1, c2, N->err);
     refresh_weights(N);
     UN_CUDA(cudaGetLastError());
     return FCM_OK;
@@ -963,6 +1017,7 @@ void fcm_unet_destroy(fcm_unet *N)
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (N->host) cudaFreeHost(N->host);
+    if (N->seen) cudaFreeHost(N->seen);
     delete N;
 }
 

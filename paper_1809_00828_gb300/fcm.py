@@ -24,8 +24,8 @@ EXPORTED = ("fcm_setup", "fcm_info", "fcm_rhs", "fcm_precond_build", "fcm_pcg_so
             "fcm_last_solve", "fcm_apply_K", "fcm_apply_S", "fcm_apply_S_noalloc", "fcm_apply_S_many",
             "fcm_set_wait_limit", "fcm_set_k_precision", "fcm_last_error", "fcm_destroy",
             "fcm_unet_create", "fcm_unet_params", "fcm_unet_get", "fcm_unet_set", "fcm_unet_forward",
-            "fcm_unet_backward", "fcm_unet_zero_grad", "fcm_unet_adam", "fcm_unet_destroy", "fcm_coarse_restrict",
-            "fcm_coarse_prolong", "fcm_coarse_apply", "fcm_fpcg_solve", "fcm_fpcg_solve_host",
+            "fcm_unet_backward", "fcm_unet_zero_grad", "fcm_unet_adam", "fcm_unet_destroy", "fcm_unet_status",
+            "fcm_unet_set_wait_limit", "fcm_coarse_restrict", "fcm_coarse_prolong", "fcm_coarse_apply", "fcm_fpcg_solve", "fcm_fpcg_solve_host",
             "fcm_fpcg_set_stall_window", "fcm_coarse_set_preconditioner", "fcm_coarse_set_storage", "fcm_coarse_levels",
             "fcm_coarse_vcycle",
             "fcm_mlhp_create", "fcm_mlhp_get_info", "fcm_mlhp_leaf", "fcm_mlhp_function",
@@ -371,6 +371,8 @@ def _bind_unet(L):
     L.fcm_unet_backward.argtypes = [P, P, P]
     L.fcm_unet_zero_grad.argtypes = [P]
     L.fcm_unet_adam.argtypes = [P, ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_int]
+    L.fcm_unet_status.argtypes = [P]
+    L.fcm_unet_set_wait_limit.argtypes = [P, ctypes.c_int]
     L.fcm_unet_destroy.argtypes = [P]
     L.fcm_unet_destroy.restype = None
     L.fcm_coarse_restrict.argtypes = [P, P, ctypes.c_float, ctypes.c_int, P]
@@ -385,8 +387,8 @@ def _bind_unet(L):
     L.fcm_coarse_levels.argtypes = [P, ip, ip, dp, dp]
     L.fcm_coarse_vcycle.argtypes = [P, ctypes.c_int, P, P]
     for f in ("fcm_unet_create", "fcm_unet_params", "fcm_unet_get", "fcm_unet_set", "fcm_unet_forward",
-              "fcm_unet_backward", "fcm_unet_zero_grad", "fcm_unet_adam", "fcm_coarse_restrict", "fcm_coarse_prolong",
-              "fcm_coarse_apply", "fcm_fpcg_solve", "fcm_fpcg_solve_host", "fcm_fpcg_set_stall_window",
+              "fcm_unet_backward", "fcm_unet_zero_grad", "fcm_unet_adam", "fcm_unet_status", "fcm_unet_set_wait_limit",
+              "fcm_coarse_restrict", "fcm_coarse_prolong", "fcm_coarse_apply", "fcm_fpcg_solve", "fcm_fpcg_solve_host", "fcm_fpcg_set_stall_window",
               "fcm_coarse_set_preconditioner", "fcm_coarse_set_storage", "fcm_coarse_levels", "fcm_coarse_vcycle"):
         getattr(L, f).restype = ctypes.c_int
     _unet_bound = True
@@ -454,6 +456,14 @@ class UNet:
 
     def adam(self, lr, step, beta1=0.9, beta2=0.999, eps=1e-8):
         _unet_check(load().fcm_unet_adam(self.h, lr, beta1, beta2, eps, step))
+
+    def check(self):
+        """Waits for the network's stream; FcmError (FCM_ETIMEOUT) if a convolution gave up its bounded wait."""
+        _unet_check(load().fcm_unet_status(self.h))
+
+    def set_wait_limit(self, tries):
+        """Polls of the convolutions' bounded wait for the tensor core (0: give up at once; < 0: default)."""
+        _unet_check(load().fcm_unet_set_wait_limit(self.h, int(tries)))
 
     def close(self):
         if getattr(self, "h", None) and self.h.value:

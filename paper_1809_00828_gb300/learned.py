@@ -133,13 +133,16 @@ def train(net, samples, gamma, steps=400, batch=4, lr=1e-3, seed=0, log=print, l
         history.append(loss)
         if log and (step % log_every == 0 or step == 1):
             log(f"  step {step:5d}  loss {np.mean(history[-log_every:]):.4f}")
+    net.check()
     return history
 
 
 def evaluate(net, samples, gamma):
     """Mean loss over all samples (no update)."""
     grid = samples[0].solver.workload.n
-    return float(np.mean([loss_and_grad(net, samples, [i], gamma, grid)[0] for i in range(len(samples))]))
+    loss = float(np.mean([loss_and_grad(net, samples, [i], gamma, grid)[0] for i in range(len(samples))]))
+    net.check()
+    return loss
 
 
 MAGIC = b"FCMUNET1"
