@@ -12,6 +12,7 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -575,6 +576,7 @@ struct fcm_unet {
     __nv_bfloat16 *tiles = nullptr;  // weight tiles of every layer (conv_tiles_kernel), made with w16
     float *part = nullptr;           // partial sums of a weight gradient
     float *host = nullptr;           // pinned copy of parameters and gradients for fcm_unet_get (made on first use)
+    std::mutex host_lock;            // held by the reader whose copies are in it
     int *err = nullptr;              // set by a convolution whose wait for the tensor core ran out, until reported
     int *seen = nullptr;             // the same in pinned host memory
     ConvWait wait = {};              // what the convolutions get: these flags, or those of the solve they run in
@@ -885,6 +887,7 @@ fcm_status fcm_unet_get(fcm_unet *N, float *w_host, float *g_host)
     if (!N || !w_host) return FCM_EINVAL;
     // through pinned memory: a copy to the caller's pageable buffers runs at 3.4 GB/s (2 MB each, 1.2 ms)
     const size_t bytes = sizeof(float) * N->nparam;
+    const std::lock_guard<std::mutex> lock(N->host_lock);
     if (!N->host) UN_CUDA(cudaMallocHost((void **)&N->host, 2 * bytes));
     UN_CUDA(cudaMemcpyAsync(N->host, N->w, bytes, cudaMemcpyDeviceToHost, N->stream));
     if (g_host) UN_CUDA(cudaMemcpyAsync(N->host + N->nparam, N->g, bytes, cudaMemcpyDeviceToHost, N->stream));
