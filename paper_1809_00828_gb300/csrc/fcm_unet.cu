@@ -270,28 +270,43 @@ __global__ void __launch_bounds__(kConvThreads, 2)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
 }
 
-// Weight tiles of one layer in the tensor core's layout, from the BF16 weights w[co][ci][27]: per block of 64
-// output channels, 16 input channels, (dy, dx) and slot 2 - dz, [channel / 8][K / 8][8 channels][8 K] (zeros beyond
-// the layer).
-// flip: the tiles of the data-gradient convolution, w'[ci][co][26 - tap] (cin, cout: those of that convolution).
-__global__ void conv_tiles_kernel(const __nv_bfloat16 *__restrict__ w, __nv_bfloat16 *__restrict__ t, int cin, int cout,
-                                  int flip)
+// Weight tiles of every layer in the tensor core's layout, from the FP32 weights w[co][ci][27] rounded to BF16: per
+// block of 64 output channels, 16 input channels, (dy, dx) and slot 2 - dz, [channel / 8][K / 8][8 channels][8 K] (zeros
+// beyond the layer).  Two sets per layer, one after the other: those of the layer, and those of the data-gradient
+// convolution, w'[ci][co][26 - tap].  One launch for all of them: an Adam step on four levels takes 23 us with its
+// update, 142 with a conversion and two launches per layer.
+constexpr int kMaxConv = 6 * 2 + 5 * 2 + 1;
+struct TileTable {
+    int64_t at[2 * kMaxConv];  // first entry of each set; a set is a multiple of 256 entries
+    int64_t woff[kMaxConv];
+    int cin[kMaxConv], cout[kMaxConv];
+    int sets;
+};
+static_assert(27 * 16 * 16 % 256 == 0, "a CTA's entries are of one set");
+
+__global__ void __launch_bounds__(256)
+    weight_tiles_kernel(const float *__restrict__ w, __nv_bfloat16 *__restrict__ t, const __grid_constant__ TileTable tab)
 {
+    const int64_t first = blockIdx.x * (int64_t)256;
+    int s = 0;
+#pragma unroll
+    for (int step = 32; step > 0; step >>= 1)
+        if (s + step < tab.sets && tab.at[s + step] <= first) s += step;
+    const bool flip = s & 1;
+    const int cin = flip ? tab.cout[s >> 1] : tab.cin[s >> 1], cout = flip ? tab.cin[s >> 1] : tab.cout[s >> 1];
     const int nb = conv_nb(cout), nch = up16(cin) / 16;
-    const int64_t n = conv_tile_entries(cin, cout);
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int k = (int)(e & 7), r = (int)(e >> 3 & 7), kc = (int)(e >> 6 & 1);
-        int64_t q = e >> 7;
-        const int n8 = (int)(q % (nb / 8));
-        q /= nb / 8;
-        const int tap = 9 * (2 - (int)(q % 3)) + (int)(q / 3 % 9);
-        q /= 27;
-        const int ci = 16 * (int)(q % nch) + 8 * kc + k, co = kCoMax * (int)(q / nch) + 8 * n8 + r;
-        __nv_bfloat16 v = __float2bfloat16(0.f);
-        if (ci < cin && co < cout)
-            v = flip ? w[((int64_t)ci * cout + co) * 27 + 26 - tap] : w[((int64_t)co * cin + ci) * 27 + tap];
-        t[e] = v;
-    }
+    const unsigned e = (unsigned)(first - tab.at[s]) + threadIdx.x;
+    const int k = (int)(e & 7), r = (int)(e >> 3 & 7), kc = (int)(e >> 6 & 1);
+    unsigned q = e >> 7;
+    const int n8 = (int)(q % (nb / 8));
+    q /= nb / 8;
+    const int tap = 9 * (2 - (int)(q % 3)) + (int)(q / 3 % 9);
+    q /= 27;
+    const int ci = 16 * (int)(q % nch) + 8 * kc + k, co = kCoMax * (int)(q / nch) + 8 * n8 + r;
+    const float *wl = w + tab.woff[s >> 1];
+    float v = 0.f;
+    if (ci < cin && co < cout) v = flip ? wl[((int64_t)ci * cout + co) * 27 + 26 - tap] : wl[((int64_t)co * cin + ci) * 27 + tap];
+    t[first + threadIdx.x] = __float2bfloat16_rn(v);
 }
 
 // ---- weight gradients: gw[co][ci][tap] += sum_{b,p} gout[b][co][p] in[b][ci][p + off(tap)], gb[co] += sum gout
@@ -529,12 +544,6 @@ __global__ void chan_copy_kernel(const float *src, int Csrc, int cs0, float *dst
     }
 }
 
-__global__ void to_bf16_kernel(const float *a, __nv_bfloat16 *b, int64_t n)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        b[i] = __float2bfloat16_rn(a[i]);
-}
-
 // Adam (Kingma & Ba, 2015) with bias correction; nothing if a convolution gave up its wait (*err): g is not valid.
 __global__ void adam_kernel(float *w, const float *g, float *m, float *v, int64_t n, float lr, float b1, float b2,
                             float eps, float c1, float c2, const int *err)
@@ -572,8 +581,8 @@ struct fcm_unet {
     std::vector<UConv> conv;  // enc (2 per level), dec (2 per level above the bottom, top-down), out
     int64_t nparam = 0;
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
-    __nv_bfloat16 *w16 = nullptr;
-    __nv_bfloat16 *tiles = nullptr;  // weight tiles of every layer (conv_tiles_kernel), made with w16
+    __nv_bfloat16 *tiles = nullptr;  // BF16 weight tiles of every layer (weight_tiles_kernel), made whenever w changes
+    int64_t ntiles = 0;              // their entries
     float *part = nullptr;           // partial sums of a weight gradient
     float *host = nullptr;           // pinned copy of parameters and gradients for fcm_unet_get (made on first use)
     std::mutex host_lock;            // held by the reader whose copies are in it
@@ -714,18 +723,20 @@ void conv_bwd(fcm_unet *N, int layer, const ConvSrc &in, const float *gout, cons
 
 ConvSrc plain(const float *a, int c) { return ConvSrc{nullptr, a, nullptr, 0, c}; }
 
-// BF16 copy of the parameters and every layer's weight tiles
+// every layer's weight tiles from the parameters
 void refresh_weights(fcm_unet *N)
 {
-    to_bf16_kernel<<<blocks_for(N->nparam), 256, 0, N->stream>>>(N->w, N->w16, N->nparam);
-    for (const UConv &c : N->conv) {
-        conv_tiles_kernel<<<blocks_for(conv_tile_entries(c.cin, c.cout)), 256, 0, N->stream>>>(N->w16 + c.woff,
-                                                                                             N->tiles + c.toff, c.cin,
-                                                                                             c.cout, 0);
-        conv_tiles_kernel<<<blocks_for(conv_tile_entries(c.cout, c.cin)), 256, 0, N->stream>>>(N->w16 + c.woff,
-                                                                                             N->tiles + c.doff, c.cout,
-                                                                                             c.cin, 1);
+    TileTable tab;
+    tab.sets = 2 * (int)N->conv.size();
+    for (size_t k = 0; k < N->conv.size(); ++k) {
+        const UConv &c = N->conv[k];
+        tab.at[2 * k] = c.toff;
+        tab.at[2 * k + 1] = c.doff;
+        tab.woff[k] = c.woff;
+        tab.cin[k] = c.cin;
+        tab.cout[k] = c.cout;
     }
+    weight_tiles_kernel<<<(unsigned)(N->ntiles / 256), 256, 0, N->stream>>>(N->w, N->tiles, tab);
 }
 
 uint64_t splitmix(uint64_t &s)
@@ -826,6 +837,7 @@ fcm_status fcm_unet_create(const fcm_unet_desc *d, void *cuda_stream, fcm_unet *
         npart = std::max(npart, pairs * kWTaps * wgrad_slabs(c.cin, c.cout, INT64_MAX));
     }
     N->nparam = off;
+    N->ntiles = toff;
     // Kaiming-uniform weights (bound sqrt(6 / fan_in)), zero biases; the output layer 10x smaller
     std::vector<float> h(off, 0.f);
     uint64_t s = d->seed;
@@ -849,7 +861,6 @@ fcm_status fcm_unet_create(const fcm_unet_desc *d, void *cuda_stream, fcm_unet *
         if ((e = cudaMalloc((void **)a, sizeof(float) * off)) != cudaSuccess) return fail(e);
         if ((e = cudaMemsetAsync(*a, 0, sizeof(float) * off, N->stream)) != cudaSuccess) return fail(e);
     }
-    if ((e = cudaMalloc((void **)&N->w16, sizeof(__nv_bfloat16) * off)) != cudaSuccess) return fail(e);
     if ((e = cudaMalloc((void **)&N->tiles, sizeof(__nv_bfloat16) * toff)) != cudaSuccess) return fail(e);
     if ((e = cudaMalloc((void **)&N->part, sizeof(float) * npart)) != cudaSuccess) return fail(e);
     if ((e = cudaMalloc((void **)&N->err, sizeof(int))) != cudaSuccess) return fail(e);
@@ -1016,7 +1027,7 @@ void fcm_unet_destroy(fcm_unet *N)
     if (!N) return;
     if (N->stream) cudaStreamSynchronize(N->stream);
     free_acts(N);
-    void *ptrs[] = {N->w, N->g, N->m, N->v, N->w16, N->tiles, N->part, N->err};
+    void *ptrs[] = {N->w, N->g, N->m, N->v, N->tiles, N->part, N->err};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (N->host) cudaFreeHost(N->host);
