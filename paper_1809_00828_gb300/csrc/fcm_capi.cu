@@ -515,6 +515,33 @@ fcm_status fcm_precond_build(fcm_ctx *C, const fcm_precond_opts *opts)
     return FCM_OK;
 }
 
+// The workspace of nr right-hand sides: the block products, and with `vectors` the solver's six vectors each (38 GB
+// for 8 right-hand sides of 80^3 cells at p = 4: only where something reads them).
+static fcm_status multi_workspace(fcm_ctx *C, int nr, bool vectors)
+{
+    if (C->m_nr != nr || (vectors && !C->h_ms)) {
+        if (C->d_m) cudaFree(C->d_m);
+        if (C->d_ms) cudaFree(C->d_ms);
+        C->d_m = nullptr;
+        C->d_ms = nullptr;
+        if (C->h_ms) cudaFreeHost(C->h_ms);
+        C->h_ms = nullptr;
+    }
+    if (C->m_nr != nr) {
+        if (C->d_mzb) cudaFree(C->d_mzb);
+        C->d_mzb = nullptr;
+        C->m_nr = 0;
+        API_CUDA(C, cudaMalloc(&C->d_mzb, sizeof(double) * (size_t)nr * C->plan.nslots * C->plan.zs));
+        C->m_nr = nr;
+    }
+    if (vectors && !C->h_ms) {
+        API_CUDA(C, cudaMalloc(&C->d_m, sizeof(double) * 6 * (size_t)nr * C->nlat));
+        API_CUDA(C, cudaMalloc(&C->d_ms, sizeof(CgScalars) * nr));
+        API_CUDA(C, cudaMallocHost((void **)&C->h_ms, sizeof(CgScalars) * nr));
+    }
+    return FCM_OK;
+}
+
 // nr independent PCG recurrences (one per right-hand side) that share every Schwarz launch: the block
 // factors are read once per iteration for all nr residuals.  K is applied per right-hand side; each
 // recurrence stops on its own ||S r|| / ||S b|| <= tol (its kernels then return at once).
@@ -523,22 +550,8 @@ static fcm_status solve_multi(fcm_ctx *C, const double *rhs, int nr, double tol,
 {
     const int64_t n = C->nlat;
     cudaStream_t st = C->stream;
-    if (C->m_nr != nr) {
-        if (C->d_m) cudaFree(C->d_m);
-        if (C->d_ms) cudaFree(C->d_ms);
-        if (C->h_ms) cudaFreeHost(C->h_ms);
-        if (C->d_mzb) cudaFree(C->d_mzb);
-        C->d_m = nullptr;
-        C->d_ms = nullptr;
-        C->h_ms = nullptr;
-        C->d_mzb = nullptr;
-        C->m_nr = 0;
-        API_CUDA(C, cudaMalloc(&C->d_m, sizeof(double) * 6 * (size_t)nr * n));
-        API_CUDA(C, cudaMalloc(&C->d_ms, sizeof(CgScalars) * nr));
-        API_CUDA(C, cudaMallocHost((void **)&C->h_ms, sizeof(CgScalars) * nr));
-        API_CUDA(C, cudaMalloc(&C->d_mzb, sizeof(double) * (size_t)nr * C->plan.nslots * C->plan.zs));
-        C->m_nr = nr;
-    }
+    const fcm_status ws = multi_workspace(C, nr, true);
+    if (ws != FCM_OK) return ws;
     double *X = C->d_m, *R = X + (size_t)nr * n, *Z = R + (size_t)nr * n, *Pd = Z + (size_t)nr * n,
            *Q = Pd + (size_t)nr * n, *B = Q + (size_t)nr * n;
     std::vector<CgWork> w(nr);
@@ -732,23 +745,8 @@ fcm_status fcm_apply_S_many(fcm_ctx *C, const double *r_dev, int nrhs, double *z
     if (nrhs == 1) return fcm_apply_S(C, r_dev, z_dev);
     StreamScope sc(C);
     const int64_t n = C->nlat;
-    if (C->m_nr != nrhs) {
-        // the multi-RHS workspace of the solver, shaped for nrhs vectors
-        if (C->d_m) cudaFree(C->d_m);
-        if (C->d_ms) cudaFree(C->d_ms);
-        if (C->h_ms) cudaFreeHost(C->h_ms);
-        if (C->d_mzb) cudaFree(C->d_mzb);
-        C->d_m = nullptr;
-        C->d_ms = nullptr;
-        C->h_ms = nullptr;
-        C->d_mzb = nullptr;
-        C->m_nr = 0;
-        API_CUDA(C, cudaMalloc(&C->d_m, sizeof(double) * 6 * (size_t)nrhs * n));
-        API_CUDA(C, cudaMalloc(&C->d_ms, sizeof(CgScalars) * nrhs));
-        API_CUDA(C, cudaMallocHost((void **)&C->h_ms, sizeof(CgScalars) * nrhs));
-        API_CUDA(C, cudaMalloc(&C->d_mzb, sizeof(double) * (size_t)nrhs * C->plan.nslots * C->plan.zs));
-        C->m_nr = nrhs;
-    }
+    const fcm_status ws = multi_workspace(C, nrhs, C->d_jac != nullptr);
+    if (ws != FCM_OK) return ws;
     const double *R = r_dev;
     const uint8_t *xmask = C->d_mask;
     if (C->d_jac) {  // as in fcm_apply_S
