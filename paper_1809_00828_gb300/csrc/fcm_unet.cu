@@ -391,8 +391,9 @@ __global__ void __launch_bounds__(256, 2)
             for (int c = 0; c < kWO; ++c) sg[c][tid] = v[c];
         }
         __syncthreads();
+        const int ye = z0 + zq < nz ? min(kWY, ny - y0) : 0;  // rows of the thread's plane inside the grid
 #pragma unroll 1
-        for (int y = 0; y < kWY; ++y) {
+        for (int y = 0; y < ye; ++y) {
             float g[2][8];
 #pragma unroll
             for (int o = 0; o < 2; ++o) {
