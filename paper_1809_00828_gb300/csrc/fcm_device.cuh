@@ -76,9 +76,15 @@ struct KCells {
     SfTablesFF sff;
 };
 // Whether n uncut cells go with the cut cells' dense product (a CTA per cell) instead of the modal form (32
-// cells per CTA): a grid of few cells leaves most SMs idle in the modal form, whose 32 cells take one SM's
-// FP64 pipe as long as about 5 (p = 2: 19 us, against 4.7 us for a cell's 81^2 dense product) or 2.5 (p = 3)
-// dense cells, so it pays from that many cells per SM on.  p = 1: 4.7 KB of K_ref against 250 operations.
+// cells per CTA): a grid of few cells leaves most SMs idle in the modal form, which takes about as long for 32
+// cells as for 152 times as many.  The line is set by FP64, where the dense product's pipe time grows with the
+// cells; in double-float it could lie at more than twice as many cells, but the choice is made before the
+// arithmetic is.  K x on uncut cubes, modal / dense form, us, FP64 and double-float:
+//   p = 1, 1,331 cells 17.1 / 12.8 and 17.0 / 12.4;  4,096 cells 17.0 / 16.9 and 17.0 / 14.7
+//   p = 2,   512 cells 27.1 / 20.6 and 21.0 / 14.4;  1,000 cells 27.1 / 26.7 and 21.3 / 16.5;  2,744 cells 28.0 /
+//            51.2 and 23.3 / 24.7
+//   p = 3,   216 cells 54.0 / 33.2 and 49.3 / 21.3;    512 cells 56.0 / 53.7 and 50.1 / 24.4;  1,000 cells 56.0 /
+//            80.9 and 51.9 / 34.7
 inline bool k_dense_uncut(int p, int64_t n) { return n <= 152 * (p == 1 ? 8 : p == 2 ? 4 : p == 3 ? 2 : 0); }
 // weight tables of fcm_modal.cuh: 3 components x kModalTabs x (p+1)^3
 void make_modal_tables(const double *h, double E, double nu, int p, std::vector<double> &tab);

@@ -21,17 +21,6 @@ namespace {
 __host__ __device__ constexpr int rnd32k(int v) { return (v + 31) / 32 * 32; }
 __host__ __device__ constexpr int ebe_threads(int rows) { return rnd32k(rows) < 512 ? rnd32k(rows) : 512; }
 
-// Barrier among the threads of one cell: a warp when the cell's points fit one warp (p <= 2), else
-// the CTA.  Only the table load at the start needs the whole CTA.
-template <int TPC>
-__device__ __forceinline__ void cell_sync()
-{
-    if constexpr (TPC == 32)
-        __syncwarp();
-    else
-        __syncthreads();
-}
-
 // S + C += sum over k < n of a_k b_k for double-float operands
 struct FFAcc {
     float S = 0.f, C = 0.f;
@@ -77,6 +66,7 @@ __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
     constexpr int Q = P + 1, NE = 3 * Q * Q * Q;
     if (done && *done) return;
     __shared__ __align__(16) float2 xe[(NE + 3) / 4 * 4], m[fold_entries(NE)];
+    static_assert(sizeof(xe) + sizeof(m) + 1024 <= 48 * 1024, "static shared memory");
     __shared__ uint64_t bar;
     const CutCell ce = cells[blockIdx.x];
     const int t = threadIdx.x, l = t / 3, ix = l % Q, iy = (l / Q) % Q, iz = l / (Q * Q);
@@ -141,14 +131,14 @@ __global__ void __launch_bounds__(256)
             for (int k = 0; k < Q; ++k) s.add(sB[tx][k], U[lc][c][k + Q * (ty + Q * tz)]);
             A[lc][t] = s.get();
         }
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {
             FFAcc s;
 #pragma unroll
             for (int k = 0; k < Q; ++k) s.add(sB[ty][k], A[lc][tx + Q * (k + Q * tz)]);
             Bq[lc][t] = s.get();
         }
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {
             FFAcc s;
 #pragma unroll
@@ -156,10 +146,10 @@ __global__ void __launch_bounds__(256)
             uq[c] = s.get();
         }
     }
-    cell_sync<TPC>();  // every point has read the nodal values of its cell
+    __syncthreads();  // every point has read the nodal values of its cell
     if (on)
         for (int c = 0; c < 3; ++c) U[lc][c][t] = uq[c];
-    cell_sync<TPC>();
+    __syncthreads();
     // gradients at the point by the collocation derivative along each axis
     float2 gr[3][3];
     if (on) {
@@ -190,10 +180,10 @@ __global__ void __launch_bounds__(256)
     }
     float2 out[3];
     for (int c = 0; c < 3; ++c) {
-        cell_sync<TPC>();  // the previous readers of U and A are done
+        __syncthreads();  // the previous readers of U and A are done
         if (on)
             for (int j = 0; j < 3; ++j) U[lc][j][t] = F[c][j];
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {  // transposed collocation derivative: point values of component c's force
             FFAcc v;
 #pragma unroll
@@ -204,21 +194,21 @@ __global__ void __launch_bounds__(256)
             }
             A[lc][t] = v.get();
         }
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {  // z^T: (qx, qy, iz)
             FFAcc s;
 #pragma unroll
             for (int k = 0; k < Q; ++k) s.add(sB[k][tz], A[lc][tx + Q * (ty + Q * k)]);
             Bq[lc][t] = s.get();
         }
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {  // y^T: (qx, iy, iz)
             FFAcc s;
 #pragma unroll
             for (int k = 0; k < Q; ++k) s.add(sB[k][ty], Bq[lc][tx + Q * (k + Q * tz)]);
             A[lc][t] = s.get();
         }
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {  // x^T: nodal force (ix, iy, iz)
             FFAcc s;
 #pragma unroll

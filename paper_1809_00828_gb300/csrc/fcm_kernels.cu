@@ -4,7 +4,7 @@
 // form, cut cells with their dense element matrix on a second stream beside them), then one kernel adds the
 // slots node by node (fcm_modal.cuh): three launches, no atomics, one fixed order of additions.  Eight
 // parity colours that added into y in place took 16 dependent launches, which a small grid pays in latency
-// (4^3 cells: K 8.5 us per launch) and a large one in tails.  (The Schwarz apply is in fcm_schwarz.cu.)
+// (4^3 cells, K and S together: 119.8 us, 35.9 with the slots) and a large one in tails.  (The Schwarz apply is in fcm_schwarz.cu.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -61,17 +61,6 @@ __global__ void __launch_bounds__(ebe_threads(P))
     if (t < NE) zk[t * nc + ce.cell] = s;
 }
 
-// Barrier among the threads of one cell: a warp when the cell's points fit one warp (p <= 2), else
-// the CTA.  Only the table load at the start needs the whole CTA.
-template <int TPC>
-__device__ __forceinline__ void cell_sync()
-{
-    if constexpr (TPC == 32)
-        __syncwarp();
-    else
-        __syncthreads();
-}
-
 // Zk slots K_ref x_e of uncut cells, without the matrix, by sum factorisation (p = 4).  Each displacement
 // component is interpolated to the (p+1)^3 Gauss points by one-dimensional contractions along
 // x, y, z (sum factorisation); its gradient there follows from the collocation derivative on
@@ -118,14 +107,14 @@ __global__ void __launch_bounds__(256)
             for (int k = 0; k < Q; ++k) s0 = fma(sB[tx][k], U[lc][c][k + Q * (ty + Q * tz)], s0);
             A[lc][t] = s0;
         }
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {
             double s1 = 0.0;
 #pragma unroll
             for (int k = 0; k < Q; ++k) s1 = fma(sB[ty][k], A[lc][tx + Q * (k + Q * tz)], s1);
             Bq[lc][t] = s1;
         }
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {
             double s2 = 0.0;
 #pragma unroll
@@ -133,10 +122,10 @@ __global__ void __launch_bounds__(256)
             uq[c] = s2;
         }
     }
-    cell_sync<TPC>();  // every point has read the nodal values of its cell
+    __syncthreads();  // every point has read the nodal values of its cell
     if (on)
         for (int c = 0; c < 3; ++c) U[lc][c][t] = uq[c];
-    cell_sync<TPC>();
+    __syncthreads();
     // gradients at the point by the collocation derivative along each axis
     double gr[3][3];
     if (on) {
@@ -163,10 +152,10 @@ __global__ void __launch_bounds__(256)
     }
     double out[3];
     for (int c = 0; c < 3; ++c) {
-        cell_sync<TPC>();  // the previous readers of U and A are done
+        __syncthreads();  // the previous readers of U and A are done
         if (on)
             for (int j = 0; j < 3; ++j) U[lc][j][t] = F[c][j];
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {  // transposed collocation derivative: point values of component c's force
             double v = 0.0;
 #pragma unroll
@@ -177,21 +166,21 @@ __global__ void __launch_bounds__(256)
             }
             A[lc][t] = v;
         }
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {  // z^T: (qx, qy, iz)
             double s2 = 0.0;
 #pragma unroll
             for (int k = 0; k < Q; ++k) s2 = fma(sB[k][tz], A[lc][tx + Q * (ty + Q * k)], s2);
             Bq[lc][t] = s2;
         }
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {  // y^T: (qx, iy, iz)
             double s1 = 0.0;
 #pragma unroll
             for (int k = 0; k < Q; ++k) s1 = fma(sB[k][ty], Bq[lc][tx + Q * (k + Q * tz)], s1);
             A[lc][t] = s1;
         }
-        cell_sync<TPC>();
+        __syncthreads();
         if (on) {  // x^T: nodal force (ix, iy, iz)
             double o = 0.0;
 #pragma unroll
@@ -292,11 +281,12 @@ cudaError_t k_prepare(int p)
 
 void make_modal_tables(const double *h, double E, double nu, int p, std::vector<double> &tab)
 {
+    tab.clear();
+    if (p > 3) return;  // dense tables (SfTables)
     const int q = p + 1, q3 = q * q * q;
     const double lam = E * nu / ((1.0 + nu) * (1.0 - 2.0 * nu)), mu = E / (2.0 * (1.0 + nu));
     const double detJ = h[0] * h[1] * h[2] / 8.0;
-    const double k4 = kModalK42 * kModalK2;
-    const double kap[5] = {1.0, 1.0, kModalK2, kModalK3, k4}, rho[5] = {1.0, kModalK2, kModalK3, k4, 0.0};
+    const double kap[4] = {1.0, 1.0, kModalK2, kModalK3}, rho[4] = {1.0, kModalK2, kModalK3, 0.0};
     tab.assign((size_t)3 * kModalTabs * q3, 0.0);
     for (int c = 0; c < 3; ++c) {
         const double H[3] = {2.0 / h[c], 2.0 / h[(c + 1) % 3], 2.0 / h[(c + 2) % 3]};

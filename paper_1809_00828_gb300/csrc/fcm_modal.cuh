@@ -1,12 +1,12 @@
-// K_ref x_e of uncut cells in Legendre modal form (internal to libfcm; FP64 and double-float).
+// K_ref x_e of uncut cells in Legendre modal form (internal to libfcm; FP64 and double-float; p <= 3).
 //
 // The integrated-Legendre basis is a sparse combination of Legendre polynomials: along one axis, with
 // v_j the coefficient of phi_j = (P_j - P_{j-2}) / sqrt(2(2j-1)) and u_0, u_1 the hats' values, twice the
 // Legendre coefficients are kappa_n r_n with
-//   r_0 = u_0 + u_1 - k2 v_2,  r_1 = u_1 - u_0 - k3 v_3,  r_2 = v_2 - (k4 / k2) v_4,  r_3 = v_3,  r_4 = v_4,
+//   r_0 = u_0 + u_1 - k2 v_2,  r_1 = u_1 - u_0 - k3 v_3,  r_2 = v_2,  r_3 = v_3,
 // kappa_n = k_n = sqrt(2 / (2n - 1)) for n >= 2, kappa_0 = kappa_1 = 1; and the derivative's coefficient n is
 // (2n + 1) sum_{m > n, m - n odd} of them, rho_n e_n with
-//   e_0 = r_1 + k3 r_3,  e_1 = r_2 + (k4 / k2) r_4,  e_2 = r_3,  e_3 = r_4   (rho = 1, k2, k3, k4).
+//   e_0 = r_1 + k3 r_3,  e_1 = r_2,  e_2 = r_3   (rho = 1, k2, k3).
 // Legendre polynomials are orthogonal, so the bilinear form of Eq. (1) couples only equal mode triples alpha:
 // every product of derivatives is one weight per alpha (modal_tables), and no Gauss point is needed.  p = 2
 // takes about 1,000 multiply-adds or additions per cell where the 1D contractions with dense tables at the
@@ -35,7 +35,6 @@ namespace fcm {
 
 constexpr double kModalK2 = 0.81649658092772603273;   // sqrt(2/3)
 constexpr double kModalK3 = 0.63245553203367586640;   // sqrt(2/5)
-constexpr double kModalK42 = 0.65465367070797714380;  // sqrt(2/7) / sqrt(2/3) = sqrt(3/7)
 constexpr int kModalTabs = 7;                         // weight tables per component (modal_tables)
 
 // Arithmetic of the transforms: V the stored value, Acc a running sum.
@@ -98,20 +97,13 @@ __device__ __forceinline__ void modal_forward(typename A::V *u)
     A::add(r1, A::neg(u0));
     if constexpr (P >= 2) A::mac(r0, A::constant(-kModalK2), u[ST]);
     if constexpr (P >= 3) A::mac(r1, A::constant(-kModalK3), u[2 * ST]);
-    V r2{}, r3{}, r4{};
+    V r2{}, r3{};
     if constexpr (P >= 2) r2 = u[ST];
     if constexpr (P >= 3) r3 = u[2 * ST];
-    if constexpr (P >= 4) {
-        r4 = u[3 * ST];
-        typename A::Acc t = A::start(r2);
-        A::mac(t, A::constant(-kModalK42), r4);
-        r2 = A::get(t);
-    }
     u[0] = A::get(r0);
     u[ST] = A::get(r1);
     if constexpr (P >= 2) u[2 * ST] = r2;
     if constexpr (P >= 3) u[3 * ST] = r3;
-    if constexpr (P >= 4) u[4 * ST] = r4;
 }
 
 // the transpose: o dual to r -> forces in lattice order, in place
@@ -123,7 +115,7 @@ __device__ __forceinline__ void modal_backward(typename A::V *o)
     typename A::Acc a = A::start(o0), b = A::start(o1);
     A::add(a, A::neg(o1));  // left hat
     A::add(b, o0);          // right hat
-    V w[5];
+    V w[4];
     if constexpr (P >= 2) {
         typename A::Acc t = A::start(o[2 * ST]);
         A::mac(t, A::constant(-kModalK2), o0);
@@ -133,11 +125,6 @@ __device__ __forceinline__ void modal_backward(typename A::V *o)
         typename A::Acc t = A::start(o[3 * ST]);
         A::mac(t, A::constant(-kModalK3), o1);
         w[2] = A::get(t);
-    }
-    if constexpr (P >= 4) {
-        typename A::Acc t = A::start(o[4 * ST]);
-        A::mac(t, A::constant(-kModalK42), o[2 * ST]);
-        w[3] = A::get(t);
     }
     o[0] = A::get(a);
     o[P * ST] = A::get(b);
@@ -155,12 +142,6 @@ __device__ __forceinline__ typename A::V modal_deriv(const typename A::V *f, int
             A::mac(t, A::constant(kModalK3), f[3 * ST]);
             return A::get(t);
         }
-    if constexpr (P >= 4)
-        if (n == 1) {
-            typename A::Acc t = A::start(f[ST]);
-            A::mac(t, A::constant(kModalK42), f[3 * ST]);
-            return A::get(t);
-        }
     return f[ST];
 }
 
@@ -171,14 +152,12 @@ __device__ __forceinline__ void modal_deriv_t(typename A::Acc *o, int n, typenam
     A::add(o[ST], t);
     if constexpr (P >= 3)
         if (n == 0) A::mac(o[3 * ST], A::constant(kModalK3), t);
-    if constexpr (P >= 4)
-        if (n == 1) A::mac(o[3 * ST], A::constant(kModalK42), t);
 }
 
 constexpr int kModalThreads = 96;  // one group of 32 cells per CTA
 // CTAs per SM the register budget is set for (the warps of a CTA spread over the SM's four partitions); shared
-// memory allows eight at p = 2, three at p = 3, one at p = 4
-__host__ __device__ constexpr int modal_ctas(int P) { return P <= 2 ? 5 : P == 3 ? 2 : 1; }
+// memory allows eight at p = 2 and three at p = 3
+__host__ __device__ constexpr int modal_ctas(int P) { return P <= 2 ? 5 : 2; }
 __host__ __device__ constexpr int modal_smem_bytes(int P)
 {
     return ((P + 1) * (P + 1) * (P + 1)) * 3 * 8 * (kModalTabs + 32);
@@ -241,7 +220,7 @@ __global__ void __launch_bounds__(kModalThreads, modal_ctas(P))
     for (int k = 0; k < (P >= 3 ? 3 : 1); ++k)
 #pragma unroll
         for (int i = 0; i < Q2; ++i) up[k][i] = A::zero();
-    V keep[P >= 4 ? 3 : P >= 3 ? 2 : 1][Q2];  // transformed planes 0 .. P - 2 for the backward step of axis 2
+    V keep[P >= 3 ? 2 : 1][Q2];  // transformed planes 0 .. P - 2 for the backward step of axis 2
 #pragma unroll (A::kPlanes == 0 ? Q : A::kPlanes)
     for (int a2 = 0; a2 < Q; ++a2) {
         const V *T = T0 + a2 * Q2, *ow = own + a2 * Q2 * 32;
@@ -281,8 +260,6 @@ __global__ void __launch_bounds__(kModalThreads, modal_ctas(P))
                 else up[0][i] = t;
                 if constexpr (P >= 3)
                     if (a2 == 0) A::mac(up[2][i], A::constant(kModalK3), v);
-                if constexpr (P >= 4)
-                    if (a2 == 1) A::mac(up[2][i], A::constant(kModalK42), v);
             }
         }
         V r[Q2];
@@ -307,17 +284,14 @@ __global__ void __launch_bounds__(kModalThreads, modal_ctas(P))
                 if constexpr (P >= 3) keep[1][i] = r[i];
             }
         } else {
-            const V k = a2 == 2 ? A::constant(-kModalK2) : a2 == 3 ? A::constant(-kModalK3) : A::constant(-kModalK42);
+            const V k = a2 == 2 ? A::constant(-kModalK2) : A::constant(-kModalK3);
 #pragma unroll
             for (int i = 0; i < Q2; ++i) {
                 Acc t = A::start(r[i]);
                 V b = keep[0][i];
                 if constexpr (P >= 3) b = a2 == 3 ? keep[1][i] : b;
-                if constexpr (P >= 4) b = a2 == 4 ? keep[2][i] : b;
                 A::mac(t, k, b);
                 store(a2 - 1, i, A::get(t));
-                if constexpr (P >= 4)
-                    if (a2 == 2) keep[2][i] = r[i];
             }
         }
     }

@@ -507,6 +507,7 @@ __global__ void __launch_bounds__(fold_threads(P))
 {
     if (done && *done) return;
     __shared__ __align__(16) T m[fold_smem(P, NR)];
+    static_assert(sizeof(m) + 1024 <= 48 * 1024, "static shared memory");
     __shared__ uint64_t bar;
     fold_block<P, NR, T>(r, nlat, nr, f32, items[blockIdx.x], g, zb, zs, zsize, pairs, xmask, err, wait_tries, m, &bar);
 }
@@ -524,6 +525,7 @@ __global__ void __launch_bounds__(fold_threads(P))
     if (done && *done) return;
     __shared__ __align__(16) float2 m[fold_smem(P, NR)];
     __shared__ uint64_t bar;
+    static_assert(sizeof(m) + 1024 <= 48 * 1024, "static shared memory");
     static_assert(sizeof(m) >= factor_ld<double>(sbox_max(P)) * NR * 8, "residuals of a streamed block");
     const int b = blockIdx.x;
     if (b < n32)

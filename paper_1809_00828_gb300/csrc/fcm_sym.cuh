@@ -1,7 +1,7 @@
 // Products with symmetric matrices stored once per pair of entries (internal to libfcm).
 //
 // A block factor F = A_B^+ and a cut cell's K_e are symmetric, so a product that streams them from HBM needs
-// half of the entries.  Matrices of at most kFoldMaxRows rows are stored folded: the upper triangle in a
+// half of the entries.  Matrices of p <= 2 (at most 81 rows) are stored folded: the upper triangle in a
 // rectangle of H = (n + 1) / 2 rows and W = n | 1 columns (n = 2 H or 2 H - 1 rows), row i < H of the triangle
 // at the right end of rectangle row i, row i >= H reversed at the left end of row 2 H - 1 - i.  A CTA copies
 // the rectangle to shared memory (one bulk copy; enough CTAs fit an SM to keep more than 100 KB in flight)
@@ -17,8 +17,6 @@
 #include "fcm_tma.cuh"
 
 namespace fcm {
-
-constexpr int kFoldMaxRows = 96;
 
 __host__ __device__ constexpr int fold_h(int n) { return (n + 1) / 2; }
 __host__ __device__ constexpr int fold_w(int n) { return n | 1; }

@@ -1,6 +1,6 @@
 // Bulk copies to shared memory, the mbarriers that complete them, and what the tensor-core kernels share
-// (internal to libfcm).  Every wait is
-// bounded: a kernel whose wait runs out marks the apply as failed and lets its copies in flight land.
+// (internal to libfcm).  Every wait is bounded: a kernel whose wait runs out marks its result as failed and lets
+// its copies and products in flight land.
 #pragma once
 
 #include <cuda_runtime.h>

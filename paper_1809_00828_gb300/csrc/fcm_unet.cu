@@ -514,9 +514,8 @@ __global__ void pool_bwd_kernel(const float *gcoarse, float *gfine, int64_t bc, 
     }
 }
 
-// gsrc[b][c][P] (=|+=) sum over the 8 children of gdst[b][c0 + c][.]
-__global__ void up_bwd_kernel(const float *gdst, float *gsrc, int B, int C, int Cdst, int c0, int nx, int ny, int nz,
-                              int accumulate)
+// gsrc[b][c][P] = sum over the 8 children of gdst[b][c0 + c][.]
+__global__ void up_bwd_kernel(const float *gdst, float *gsrc, int B, int C, int Cdst, int c0, int nx, int ny, int nz)
 {
     const int cx = nx / 2, cy = ny / 2, cz = nz / 2;
     const int64_t S = (int64_t)nx * ny * nz, Sc = (int64_t)cx * cy * cz, n = (int64_t)B * C * Sc;
@@ -527,21 +526,19 @@ __global__ void up_bwd_kernel(const float *gdst, float *gsrc, int B, int C, int 
         const float *g = gdst + ((int64_t)b * Cdst + c0 + c) * S;
         float s = 0.f;
         for (int k = 0; k < 8; ++k) s += g[((2 * Z + (k >> 2)) * ny + 2 * Y + ((k >> 1) & 1)) * nx + 2 * X + (k & 1)];
-        gsrc[e] = accumulate ? gsrc[e] + s : s;
+        gsrc[e] = s;
     }
 }
 
-// dst[b][c0 + c][p] (=|+=) src[b][cs0 + c][p] for c < C
+// dst[b][c0 + c][p] = src[b][cs0 + c][p] for c < C
 __global__ void chan_copy_kernel(const float *src, int Csrc, int cs0, float *dst, int Cdst, int c0, int B, int C,
-                                 int64_t S, int accumulate)
+                                 int64_t S)
 {
     const int64_t n = (int64_t)B * C * S;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t p = e % S, bc = e / S;
         const int c = (int)(bc % C), b = (int)(bc / C);
-        const float v = src[((int64_t)b * Csrc + cs0 + c) * S + p];
-        float &d = dst[((int64_t)b * Cdst + c0 + c) * S + p];
-        d = accumulate ? d + v : v;
+        dst[((int64_t)b * Cdst + c0 + c) * S + p] = src[((int64_t)b * Csrc + cs0 + c) * S + p];
     }
 }
 
@@ -984,11 +981,11 @@ fcm_status fcm_unet_backward(fcm_unet *N, const float *gout, float *gin)
         conv_bwd(N, N->dec_b(l), plain(N->dA[l], cs), N->gdB[l], N->dB[l], N->gdA[l], l);
         conv_bwd(N, N->dec_a(l), ConvSrc{prev, N->eB[l], nullptr, cu, cs}, N->gdA[l], N->dA[l], N->gcat[l], l);
         // skip part -> encoder output of level l (the pooling adds the other part below)
-        chan_copy_kernel<<<blocks_for(bs), 256, 0, N->stream>>>(N->gcat[l], cc, cu, N->geB[l], cs, 0, B, cs, S, 0);
+        chan_copy_kernel<<<blocks_for(bs), 256, 0, N->stream>>>(N->gcat[l], cc, cu, N->geB[l], cs, 0, B, cs, S);
         // upsampled part -> the level below
         float *gprev = (l + 1 == L - 1) ? N->geB[L - 1] : N->gdB[l + 1];
         up_bwd_kernel<<<blocks_for((int64_t)B * cu * N->S[l + 1]), 256, 0, N->stream>>>(
-            N->gcat[l], gprev, B, cu, cc, 0, N->lx[l], N->ly[l], N->lz[l], 0);
+            N->gcat[l], gprev, B, cu, cc, 0, N->lx[l], N->ly[l], N->lz[l]);
     }
     for (int l = L - 1; l >= 0; --l) {
         conv_bwd(N, N->enc_b(l), plain(N->eA[l], N->ch(l)), N->geB[l], N->eB[l], N->geA[l], l);
