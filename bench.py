@@ -71,14 +71,25 @@ COARSE_DEFAULTS = {"porous40_32_p3": ("jacobi", 20, "fp32"), "porous40_32_p2": (
                    "porous300_80_p2": ("vcycle", 2, "fp32")}
 
 
+# What the S apply's kernels are compiled from: the kernels, the folded layout and its loops, copies and waits, arithmetic.
+TRAFFIC_SOURCES = ("fcm_schwarz.cu", "fcm_sym.cuh", "fcm_tma.cuh", "fcm_ff.cuh")
+
+
+def _traffic_source_hash(folder=os.path.join(ROOT, "paper_1809_00828_gb300", "csrc")):
+    import hashlib
+    h = hashlib.sha256()
+    for name in TRAFFIC_SOURCES:
+        h.update(open(os.path.join(folder, name), "rb").read())
+    return h.hexdigest()
+
+
 def _schwarz_traffic(workload_name, precision):
     """DRAM bytes of one S apply from the committed ncu capture, or None.
 
     The capture (dram__bytes_read.sum + dram__bytes_write.sum over the launches of one S
     apply) holds for the kernel source it was taken with: the profile records the SHA-256 of
-    fcm_schwarz.cu, and any other source gives None.
+    TRAFFIC_SOURCES one after another, and any other source gives None.
     """
-    import hashlib
     import re
     if workload_name != DEFAULT_WORKLOAD or precision != "mixed" or not os.path.exists(TRAFFIC_PROFILE):
         return None
@@ -87,8 +98,7 @@ def _schwarz_traffic(workload_name, precision):
     m_h = re.search(r"kernel_source_sha256:\s*([0-9a-f]{64})", text)
     if not m_b or not m_h:
         return None
-    src = os.path.join(ROOT, "paper_1809_00828_gb300", "csrc", "fcm_schwarz.cu")
-    if hashlib.sha256(open(src, "rb").read()).hexdigest() != m_h.group(1):
+    if _traffic_source_hash() != m_h.group(1):
         return None
     return float(m_b.group(1))
 

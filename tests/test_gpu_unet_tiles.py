@@ -83,3 +83,38 @@ def test_infinities_and_nan_pass_through():
     assert torch.isinf(y[0, 0, 1, 1, 2]) or torch.isnan(y[0, 0, 1, 1, 2])
     assert float(y[0, 0, 3, 3, 7]) == float(np.float32(3.0e38)) and float(y[0, 0, 3, 0, 0]) == 1.0
     net.close()
+
+
+def test_where_infinities_go():
+    """Identity taps: an infinite voxel stays itself; 0 * inf makes its neighbours NaN, which a ReLU maps to 0 and the
+    output layer (no ReLU) passes on.  -inf and NaN are 0 after the first ReLU, and so are their neighbours."""
+    from paper_1809_00828_gb300 import fcm
+    net = fcm.UNet(in_ch=1, out_ch=1, base=1, levels=1, seed=1)
+    w = np.zeros(net.nparam, np.float32)
+    w[13] = w[28 + 13] = w[56 + 13] = 1.0
+    net.set(w)
+    x = np.ones((4, 4, 16), np.float32)
+    want = x.copy()
+    x[1, 1, 2], x[3, 1, 6], x[3, 1, 10], x[3, 3, 15] = np.inf, -np.inf, np.nan, 3.0e38
+    want[0:3, 0:3, 1:4] = np.nan
+    want[1, 1, 2] = np.inf
+    want[2:4, 0:3, 5:8] = want[2:4, 0:3, 9:12] = 0.0
+    want[3, 3, 15] = 3.0e38
+    y = net.forward(torch.from_numpy(x).cuda().view(1, 1, 4, 4, 16)).cpu().numpy().reshape(4, 4, 16)
+    assert np.array_equal(y, want, equal_nan=True)
+    net.close()
+
+
+def test_an_infinite_gradient_stays_infinite():
+    """The bias gradient (a plain sum) of a layer whose CTAs add several tiles to running sums."""
+    from paper_1809_00828_gb300 import fcm
+    net = fcm.UNet(in_ch=4, out_ch=3, base=100, levels=1, seed=1)
+    net.forward(torch.ones((1, 4, 20, 20, 20), device="cuda"))
+    g = torch.zeros((1, 3, 20, 20, 20), device="cuda")
+    g[0, 0, 9, 9, 9] = float("inf")
+    g[0, 1] = 1.0
+    net.zero_grad()
+    net.backward(g)
+    _, grad = net.get(with_grad=True)
+    assert np.array_equal(grad[-3:], [np.inf, 8000.0, 0.0])
+    net.close()
