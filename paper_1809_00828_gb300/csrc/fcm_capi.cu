@@ -411,8 +411,9 @@ fcm_status fcm_info(const fcm_ctx *C, fcm_info_t *out)
     out->n_blocks = C->n_blocks;
     out->n_blocks_fp32 = C->n_fp32_factors;
     {
-        // cut cells: dense ne x ne; uncut cells: 3 components x (8 forward + 8 transposed) contractions of
-        // Q^3 points x Q terms, plus ~21 multiply-adds of the stress per point
+        // a measure of work that no form of the kernels changes.  Cut cells: dense ne x ne; uncut cells: 3 components x
+        // (8 forward + 8 transposed) contractions of Q^3 points x Q terms, plus ~21 multiply-adds of the stress per
+        // point (the modal form of p <= 3 needs less than a third of them)
         const int64_t q = hp.p + 1;
         out->kapply_fmas = hp.ncut * (int64_t)hp.ne * hp.ne + (hp.nactive - hp.ncut) * (36 * q * q * q * q + 21 * q * q * q);
     }

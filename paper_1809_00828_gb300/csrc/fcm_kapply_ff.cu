@@ -54,9 +54,9 @@ __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
     }
 }
 
-// The same for p <= 2, K_e folded (fcm_sym.cuh): half of the matrix's bytes.  The FP32 pipe and the issue slots
-// bound it now (12 operations per entry and 8 around them): 370 us for 72,180 cells (1.92 GB, 285 us at the
-// copy rate) where streaming the full matrices took 697 us (3.8 GB).
+// The same for p <= 2, K_e folded (fcm_sym.cuh): half of the matrix's bytes.  The issue slots
+// bound it now (12 operations per entry and 8 around them; ncu, 64^3: 79 % of them busy, 63 % of the DRAM peak):
+// 370 us for 72,180 cells (1.92 GB, 285 us at the copy rate) where streaming the full matrices took 697 us (3.8 GB).
 template <int P>
 __global__ void __launch_bounds__(ebe_threads(3 * (P + 1) * (P + 1) * (P + 1)))
     ebe_fold_ff_kernel(const double *__restrict__ x, float2 *__restrict__ zk, const float2 *__restrict__ elem,

@@ -19,9 +19,10 @@
 // component c + 1 or c + 2 is then at a compile-time offset.  The result goes to the cells' slots of Zk, entry
 // (3 node + c) of cell i at Zk[(3 node + c) ncell + i], which k_sum_kernel adds up.
 //
-// FP64 is bound by its pipe (32^3 p = 3: 226 us for 30,543 uncut cells, about 180 us at 2 operations per clock
-// and SM; 745 us before).  Double-float is bound by the FP32 pipe and the issue slots: 214 us for 440k cells
-// at 80^3 p = 2, 1,091 us before.  There the loop over the mode planes of axis 2 stays rolled (90 KB of code
+// FP64 is bound by its pipe, 79 % of the active cycles (ncu, 32^3 p = 3: 201 us for 30,543 uncut cells, about 180 at
+// 2 operations per clock and SM; 745 us before).  Double-float takes 214 us for 440k cells at 80^3 p = 2 (1,091
+// before): 62 % of the issue slots and 43 % of the FP32 pipe (ncu, 64^3), the rest waits of 15 warps per SM, which
+// is what 128 registers allow, for their own results.  There the loop over the mode planes of axis 2 stays rolled (90 KB of code
 // otherwise, and warps that wait for instructions), a first product starts its sum instead of adding to 0, and
 // the sums stay unnormalised (370 -> 214 us together).
 #pragma once
@@ -305,7 +306,8 @@ __global__ void __launch_bounds__(kModalThreads, modal_ctas(P))
 // row's results go through shared memory so that the stores are consecutive too.  All loads of a row are
 // issued before the first addition (a row per warp and predicated loads instead of a loop over the rows of a
 // cell with a branch per neighbour: 171 -> 88 us at 80^3 p = 2, 111 -> 40 us at 32^3 p = 3, where
-// the slots (50 MB) stay in L2).
+// the slots (50 MB) stay in L2).  Loads bound it (long scoreboard; 48 % of the DRAM peak at 64^3 p = 2), in FP64 also
+// its pipe (57 % at 32^3 p = 3).
 constexpr int kSumWarps = 4;
 
 template <int P, class A>

@@ -420,7 +420,8 @@ __global__ void __launch_bounds__(cols_threads(P))
 //
 // Half of a symmetric factor's bytes, which bound the apply: a CTA per block, a thread per row, the columns in
 // ascending order as in schwarz_cols_kernel (an FP32 row's additions are the same, bit for bit).  At 80^3
-// p = 2 (107,741 FP32 and 37,771 double-float blocks, 1.43 + 1.00 GB): 246 + 211 us, the full factors 752 us.
+// p = 2 (107,741 FP32 and 37,771 double-float blocks, 1.43 + 1.00 GB; ncu, one kernel at a time): 237 + 199 us, the
+// full factors 731 us.
 
 __host__ __device__ constexpr int fold_threads(int P) { return rnd32(sbox_max(P)); }
 
@@ -1187,7 +1188,7 @@ void fold_launch(const double *r, int64_t nlat, int nr, const float *f32, const 
 
 // Whether one launch takes the own blocks of all kinds.  Kinds launched one after the other cost a small grid a
 // launch's latency each; many blocks fill the GPU with one kind, whose registers and shared memory fit it (80^3
-// p = 2: 246 + 211 us apart, 740 in one).  Measured apart / in one launch, us: element blocks, p = 2, 121 blocks
+// p = 2: 457 us apart, 740 in one).  Measured apart / in one launch, us: element blocks, p = 2, 121 blocks
 // 23.9 / 21.9, 822 blocks 28.5 / 24.0, 1,880 blocks 29.9 / 28.0; p = 1, 192 blocks 20.6 / 17.1, 3,344 blocks 22.6 /
 // 19.4.  Beside shared-factor products the line is lower: vertex patches, p = 2, six right-hand sides, 521 blocks
 // 236 / 236, 1,104 blocks 248 / 316.
