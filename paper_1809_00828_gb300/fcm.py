@@ -330,7 +330,7 @@ class Solver:
         self.info = self.get_info()
 
     def set_wait_limit(self, tries):
-        """Polls of the Schwarz kernels' bounded bulk-copy wait (0: give up at once; < 0: default)."""
+        """Polls of the S and K kernels' bounded bulk-copy waits (0: give up at once; < 0: default)."""
         self._check(load().fcm_set_wait_limit(self.ctx, int(tries)))
 
     def close(self):
